@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "pm.h"
+#include "pm_fx.cuh"
 #include "pm_launch.h"
 
 namespace {
@@ -293,28 +294,58 @@ int build_hhat(pm_ctx *c, GeoBuf &gb) {
     return PM_OK;
 }
 
+// Tables of one transform length: the twiddles w^m = exp(-2 pi i m / L) and
+// D(m) = exp(2 pi i m / L) - 1 = -2 sin^2(pi m / L) + i sin(2 pi m / L) (the
+// half-angle form keeps the real part accurate for small m).
+void make_tables(int L, std::vector<float2> &tw, std::vector<float2> &dt) {
+    for (int m = 0; m < L; ++m) {
+        const double a = 2.0 * M_PI * (double)m / (double)L, h = std::sin(M_PI * (double)m / (double)L);
+        tw.push_back(make_float2((float)std::cos(a), (float)(-std::sin(a))));
+        dt.push_back(make_float2((float)(-2.0 * h * h), (float)std::sin(a)));
+    }
+}
+// FP64 contexts: fixed-point twiddles (pm_fx.cuh); D's table in FP64 is
+// followed by D + i in units of 2^-59.  The long double functions behind them
+// are slow on some hosts: the largest length's are evaluated once per process
+// and the others take every 512/L-th.
+struct FxTables {
+    fxw tw[512];
+    double2 d[512];
+    longlong2 dz[512];
+    FxTables() {
+        const long double pi = 3.14159265358979323846264338327950288L;
+        for (int m = 0; m < 512; ++m) {
+            const long double a = 2.0L * pi * (long double)m / 512.0L;
+            const long double c = std::cos(a), s = std::sin(a), h = std::sin(0.5L * a), re = -2.0L * h * h;
+            pmfx::wsplit(std::llroundl(c * (1LL << pmfx::FX_Q)), tw[m].rh, tw[m].rl);
+            pmfx::wsplit(std::llroundl(-s * (1LL << pmfx::FX_Q)), tw[m].ih, tw[m].il);
+            d[m] = make_double2((double)re, (double)s);
+            dz[m].x = std::llroundl(re * (1LL << 59));
+            dz[m].y = std::llroundl((s + 1.0L) * (1LL << 59));
+        }
+    }
+};
+void make_tables(int L, std::vector<fxw> &tw, std::vector<double2> &dt) {
+    static const FxTables t;
+    for (int m = 0; m < L; ++m) {
+        tw.push_back(t.tw[m * (512 / L)]);
+        dt.push_back(t.d[m * (512 / L)]);
+    }
+    for (int m = 0; m < L; ++m) {
+        double2 z;
+        std::memcpy(&z, &t.dz[m * (512 / L)], sizeof(z));
+        dt.push_back(z);
+    }
+}
 template <typename T> int upload_twiddles(pm_ctx *c) {
-    typedef typename cplx_t<T>::type C;
     for (int i = 0; i < 6; ++i) {
-        const int L = 16 << i;
-        std::vector<C> tw(L);
-        for (int m = 0; m < L; ++m) {
-            const double a = 2.0 * M_PI * (double)m / (double)L;
-            tw[m].x = (T)std::cos(a);
-            tw[m].y = (T)(-std::sin(a));
-        }
-        PM_TRY(dev_alloc(c, &c->d_tw[i], L * sizeof(C)));
-        PM_CK(cudaMemcpyAsync(c->d_tw[i], tw.data(), L * sizeof(C), cudaMemcpyHostToDevice, c->user));
-        PM_CK(cudaStreamSynchronize(c->user));
-        // D(k) = exp(2 pi i k / L) - 1 = -2 sin^2(pi k / L) + i sin(2 pi k / L)
-        // (the half-angle form keeps the real part accurate for small k)
-        for (int m = 0; m < L; ++m) {
-            const double h = std::sin(M_PI * (double)m / (double)L);
-            tw[m].x = (T)(-2.0 * h * h);
-            tw[m].y = (T)std::sin(2.0 * M_PI * (double)m / (double)L);
-        }
-        PM_TRY(dev_alloc(c, &c->d_dt[i], L * sizeof(C)));
-        PM_CK(cudaMemcpyAsync(c->d_dt[i], tw.data(), L * sizeof(C), cudaMemcpyHostToDevice, c->user));
+        std::vector<typename comp_t<T>::W> tw;
+        std::vector<typename cplx_t<T>::type> dt;
+        make_tables(16 << i, tw, dt);
+        PM_TRY(dev_alloc(c, &c->d_tw[i], tw.size() * sizeof(tw[0])));
+        PM_CK(cudaMemcpyAsync(c->d_tw[i], tw.data(), tw.size() * sizeof(tw[0]), cudaMemcpyHostToDevice, c->user));
+        PM_TRY(dev_alloc(c, &c->d_dt[i], dt.size() * sizeof(dt[0])));
+        PM_CK(cudaMemcpyAsync(c->d_dt[i], dt.data(), dt.size() * sizeof(dt[0]), cudaMemcpyHostToDevice, c->user));
         PM_CK(cudaStreamSynchronize(c->user));
     }
     return PM_OK;

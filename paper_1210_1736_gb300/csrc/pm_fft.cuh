@@ -9,7 +9,9 @@
 // radix-2 stage of a transform held by one warp, by warp shuffles.
 #pragma once
 
-#include "pm_internal.cuh"
+#include <type_traits>
+
+#include "pm_fx.cuh"
 
 namespace pmfft {
 
@@ -64,8 +66,36 @@ template <int L, typename C> __device__ __forceinline__ void expand_twiddles(C *
     expand_stage_twiddles<L, 2, true>(tab, g);
 }
 
-// z * exp(SIGN * 2 pi i e / 16) for a compile-time-known e.
-template <int SIGN, typename C> __device__ __forceinline__ C rot16(int e, C z) {
+// Fixed point: z * exp(2 pi i e / 16); cos(pi/8), sin(pi/8), sqrt(1/2) in
+// units of 2^-60.  The odd multiples of pi/4 take two real products.
+__device__ __forceinline__ fx2 rot16_fx(int e, fx2 z) {
+    constexpr long long c1 = 1065160580698383124LL, s1 = 441203958630471860LL, r2 = 815238614083298888LL;
+    e &= 15;
+    fx2 r;
+    switch (e) {
+        case 0: return z;
+        case 4: r.x = -z.y; r.y = z.x; return r;
+        case 8: r.x = -z.x; r.y = -z.y; return r;
+        case 12: r.x = z.y; r.y = -z.x; return r;
+        case 1: return pmfx::cmulq(z, c1, s1);
+        case 3: return pmfx::cmulq(z, s1, c1);
+        case 5: return pmfx::cmulq(z, -s1, c1);
+        case 7: return pmfx::cmulq(z, -c1, s1);
+        case 9: return pmfx::cmulq(z, -c1, -s1);
+        case 11: return pmfx::cmulq(z, -s1, -c1);
+        case 13: return pmfx::cmulq(z, s1, -c1);
+        case 15: return pmfx::cmulq(z, c1, -s1);
+    }
+    int h, l;
+    pmfx::wsplit(r2, h, l);
+    const long long p = pmfx::mulr(z.x + z.y, h, l), m = pmfx::mulr(z.x - z.y, h, l);
+    if (e == 2) { r.x = m; r.y = p; }
+    else if (e == 6) { r.x = -p; r.y = m; }
+    else if (e == 10) { r.x = -m; r.y = -p; }
+    else { r.x = p; r.y = -m; }
+    return r;
+}
+template <int SIGN, typename C> __device__ __forceinline__ C rot16_fp(int e, C z) {
     typedef decltype(z.x) T;
     const T c1 = (T)0.92387953251128675613, s1 = (T)0.38268343236508977173,
             r2 = (T)0.70710678118654752440;
@@ -94,6 +124,11 @@ template <int SIGN, typename C> __device__ __forceinline__ C rot16(int e, C z) {
     r.x = z.x * c - z.y * s;
     r.y = z.x * s + z.y * c;
     return r;
+}
+// z * exp(SIGN * 2 pi i e / 16) for a compile-time-known e.
+template <int SIGN, typename C> __device__ __forceinline__ C rot16(int e, C z) {
+    if constexpr (std::is_same<C, fx2>::value) return rot16_fx(SIGN < 0 ? 16 - (e & 15) : e, z);
+    else return rot16_fp<SIGN>(e, z);
 }
 
 // In-register DFT of length R (natural order in and out):
@@ -188,10 +223,10 @@ __device__ __forceinline__ void dft16(C *v) {
 // tw: the stage tables of expand_twiddles (conjugated for SIGN > 0).
 // ZIN / HOUT select the pruned radix-16 (see dft16); they are only passed
 // for radix-16 stages.
-template <int L, int S, bool REV, int SIGN, bool ZIN = false, bool HOUT = false, typename C>
-__device__ __forceinline__ void stage_butterflies(C *v, int t, const C *tw) {
+template <int L, int S, bool REV, int SIGN, bool ZIN = false, bool HOUT = false, typename C, typename W>
+__device__ __forceinline__ void stage_butterflies(C *v, int t, const W *tw) {
     constexpr int R = radix(L, S, REV), Ns = stride_before(L, S, REV), TPC = L / E;
-    if constexpr (R == 2 && Ns == L / 2) {
+    if constexpr (R == 2 && Ns == L / 2 && !std::is_same<C, fx2>::value) {
         // a closing radix-2 stage: item j = t + kk TPC has the twiddle
         // w^j = w^t exp(-2 pi i kk / 16) (w^TPC = exp(-2 pi i / 16)): one
         // table entry per thread, the rest constant rotations.  HOUT keeps
@@ -209,10 +244,10 @@ __device__ __forceinline__ void stage_butterflies(C *v, int t, const C *tw) {
         for (int kk = 0; kk < E / R; ++kk) {
             const int j = t + kk * TPC;
             if (Ns > 1) {
-                const C *tws = tw + tw_offset(L, S, REV) + (j % Ns);
+                const W *tws = tw + tw_offset(L, S, REV) + (j % Ns);
 #pragma unroll
                 for (int r = 1; r < R; ++r) {
-                    C w = tws[r * Ns];
+                    const W w = tws[r * Ns];
                     v[kk * R + r] = (SIGN < 0) ? cmul(v[kk * R + r], w) : cconjmul(v[kk * R + r], w);
                 }
             }

@@ -5,6 +5,7 @@
 #include <utility>
 
 #include "pm_passes.cuh"
+#include "pm_passes_fx.cuh"
 #include "pm_particle.cuh"
 
 namespace pmk {
@@ -683,30 +684,6 @@ inline int particle_grid(long long n) {
     return (int)(b < cap ? (b > 0 ? b : 1) : cap);
 }
 
-template <typename T, int L, int MODE> int col_blocks_per_sm() {
-    static int cached = 0;
-    if (!cached) {
-        int nb = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, pmk::k_col<T, L, MODE>, pmk::CShape<T, L>::THREADS,
-                                                          pmk::col_smem<T, L, MODE>()) != cudaSuccess || nb < 1)
-            nb = 1;
-        cached = nb;
-    }
-    return cached;
-}
-
-template <typename T, int L, int DM> int colw_blocks_per_sm() {
-    static int cached = 0;
-    if (!cached) {
-        int nb = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, pmk::k_colw<T, L, DM>, pmk::WShape<T, L>::THREADS,
-                                                          pmk::colw_smem<T, L>()) != cudaSuccess || nb < 1)
-            nb = 1;
-        cached = nb;
-    }
-    return cached;
-}
-
 inline int num_sms() {
     static int n = 0;
     if (!n) {
@@ -717,38 +694,53 @@ inline int num_sms() {
     return n;
 }
 
-template <typename T, int L> cudaError_t attrs_L() {
-    cudaError_t e;
-    e = cudaFuncSetAttribute(pmk::k_col<T, L, COL_YFWD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)pmk::col_smem<T, L, COL_YFWD>());
-    if (e) return e;
-    e = cudaFuncSetAttribute(pmk::k_colw<T, L, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)pmk::colw_smem<T, L>());
-    if (e) return e;
-    e = cudaFuncSetAttribute(pmk::k_colw<T, L, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)pmk::colw_smem<T, L>());
-    if (e) return e;
-    if constexpr (L <= 256) {
-        e = cudaFuncSetAttribute(pmk::k_colw<T, L, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)pmk::colw_smem<T, L>());
-        if (e) return e;
-    }
-    e = cudaFuncSetAttribute(pmk::k_col<T, L, COL_YINV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)pmk::col_smem<T, L, COL_YINV>());
-    if (e) return e;
-    e = cudaFuncSetAttribute(pmk::k_xfwd<T, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pmk::xpass_smem<T, L>());
-    if (e) return e;
-    return cudaFuncSetAttribute(pmk::k_xinv<T, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)pmk::xpass_smem<T, L>());
-}
-
-// Persistent x passes: one wave of blocks (occupancy x SMs), each walking
-// groups of rows.
+// Persistent passes: one wave of blocks (occupancy x SMs), each walking
+// tiles or groups of rows.
 template <typename K> int resident_blocks(K kernel, int threads, size_t smem) {
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, threads, smem) != cudaSuccess || nb < 1) nb = 1;
     return nb;
 }
+
+// The pass kernels of a precision and length with their block sizes and
+// shared memory: FP32 in FP32, FP64 in fixed point.
+template <typename T, int L, int MODE> struct ColPass {
+    static auto kernel() { if constexpr (sizeof(T) == 4) return pmk::k_col<T, L, MODE>; else return pmk::k_yfx<L, MODE>; }
+    static constexpr int threads = pmk::CShape<T, L>::THREADS;
+    static size_t smem() { if constexpr (sizeof(T) == 4) return pmk::col_smem<T, L, MODE>(); else return pmk::fx_ysmem<L, MODE>(); }
+};
+template <typename T, int L, int DM> struct ZPass {
+    static auto kernel() { if constexpr (sizeof(T) == 4) return pmk::k_colw<T, L, DM>; else return pmk::k_zfx<L, DM>; }
+    static constexpr int threads = pmk::WShape<T, L>::THREADS;
+    static size_t smem() { if constexpr (sizeof(T) == 4) return pmk::colw_smem<T, L>(); else return pmk::fx_zsmem<L, DM>(); }
+};
+template <typename T, int L, bool INV> struct XPass {
+    static auto kernel() {
+        if constexpr (sizeof(T) == 8) return pmk::k_xfx<L, INV>;
+        else if constexpr (INV) return pmk::k_xinv<T, L>;
+        else return pmk::k_xfwd<T, L>;
+    }
+    static constexpr int threads = sizeof(T) == 4 ? pmk::NT : pmk::FXT;   // the most a block has
+    static size_t smem(int th) { if constexpr (sizeof(T) == 4) return pmk::xpass_smem<T, L>(); else return pmk::fx_xsmem<L>(th); }
+};
+template <class P> cudaError_t set_smem() {
+    return cudaFuncSetAttribute(P::kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::smem());
+}
+template <class P> cudaError_t set_xsmem() {
+    return cudaFuncSetAttribute(P::kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::smem(P::threads));
+}
+template <typename T, int L> cudaError_t attrs_L() {
+    cudaError_t e;
+    if ((e = set_smem<ColPass<T, L, COL_YFWD>>())) return e;
+    if ((e = set_smem<ColPass<T, L, COL_YINV>>())) return e;
+    if ((e = set_smem<ZPass<T, L, 0>>())) return e;
+    if ((e = set_smem<ZPass<T, L, 1>>())) return e;
+    if constexpr (L <= 256)
+        if ((e = set_smem<ZPass<T, L, 2>>())) return e;
+    if ((e = set_xsmem<XPass<T, L, false>>())) return e;
+    return set_xsmem<XPass<T, L, true>>();
+}
+
 // Launch with programmatic stream serialisation (the FFT passes of a chain:
 // each waits for its predecessor with griddepcontrol.wait after its
 // prologue).
@@ -773,49 +765,39 @@ inline int ilog2(long long v) {
     while ((1LL << l) < v) ++l;
     return l;
 }
-template <typename T, int L> cudaError_t xfwd_L(PassBatch b, cudaStream_t st) {
-    static int nb = resident_blocks(pmk::k_xfwd<T, L>, pmk::NT, pmk::xpass_smem<T, L>());
-    const long long gpi = std::max(1LL, (long long)b.a[0].ny * b.a[0].nz / pmk::XShape<L>::LINES);
-    b.lgi = ilog2(gpi);
-    const long long grid = std::min((long long)b.n << b.lgi, (long long)nb * num_sms());
-    return launch_pdl(pmk::k_xfwd<T, L>, (unsigned)grid, pmk::NT, pmk::xpass_smem<T, L>(), st, b);
+template <class P> cudaError_t launch_tiles(const PassBatch &b, cudaStream_t st) {
+    static const int nb = resident_blocks(P::kernel(), P::threads, P::smem());
+    const long long grid = std::max(1LL, std::min((long long)b.n << b.lgi, (long long)nb * num_sms()));
+    return launch_pdl(P::kernel(), (unsigned)grid, P::threads, P::smem(), st, b);
 }
-template <typename T, int L> cudaError_t xinv_L(PassBatch b, cudaStream_t st) {
-    static int nb = resident_blocks(pmk::k_xinv<T, L>, pmk::NT, pmk::xpass_smem<T, L>());
-    const long long gpi = std::max(1LL, (long long)b.a[0].ny * b.a[0].nz / pmk::XShape<L>::LINES);
-    b.lgi = ilog2(gpi);
+// Row groups of an x pass.  FP64: the largest block (at least a warp) that
+// still gives every SM one.
+template <typename T, int L, bool INV> cudaError_t xpass_L(PassBatch b, cudaStream_t st) {
+    typedef XPass<T, L, INV> P;
+    constexpr int TPC = pmk::XShape<L>::TPC;
+    const long long rows = (long long)b.a[0].ny * b.a[0].nz;
+    int threads = P::threads;
+    if (sizeof(T) == 8)
+        while (threads > 32 && b.n * rows * TPC < (long long)threads * num_sms()) threads /= 2;
+    b.lgi = ilog2(std::max(1LL, rows * TPC / threads));
+    static int cache[11];
+    int &nb = cache[ilog2(threads)];
+    if (!nb) nb = resident_blocks(P::kernel(), threads, P::smem(threads));
     const long long grid = std::min((long long)b.n << b.lgi, (long long)nb * num_sms());
-    return launch_pdl(pmk::k_xinv<T, L>, (unsigned)grid, pmk::NT, pmk::xpass_smem<T, L>(), st, b);
+    return launch_pdl(P::kernel(), (unsigned)grid, threads, P::smem(threads), st, b);
 }
 template <typename T, int L, int MODE> cudaError_t col_LM(PassBatch b, cudaStream_t st) {
     constexpr int COLS = pmk::CShape<T, L>::COLS;
     b.lgi = ilog2((long long)b.a[0].nz * ((2 * b.a[0].nx + COLS - 1) / COLS));
-    const long long ntiles = (long long)b.n << b.lgi;
-    long long grid = (long long)col_blocks_per_sm<T, L, MODE>() * num_sms();
-    if (grid > ntiles) grid = ntiles;
-    if (grid < 1) grid = 1;
-    return launch_pdl(pmk::k_col<T, L, MODE>, (unsigned)grid, pmk::CShape<T, L>::THREADS,
-                      pmk::col_smem<T, L, MODE>(), st, b);
+    return launch_tiles<ColPass<T, L, MODE>>(b, st);
 }
 template <typename T, int L> cudaError_t zconv_L(PassBatch b, cudaStream_t st) {
-    typedef pmk::WShape<T, L> S;
-    b.lgi = ilog2(((long long)4 * b.a[0].ny * b.a[0].nx) / S::COLS);   // COLS divides the 2ny x 2nx columns
-    const long long ntiles = (long long)b.n << b.lgi;
-    const bool dm = b.a[0].dmode != 0;
-    if constexpr (L <= 256) {
-        if (b.a[0].dmode == 3) {   // both difference fields in one pass (see PairArgs)
-            long long g2 = (long long)colw_blocks_per_sm<T, L, 2>() * num_sms();
-            if (g2 > ntiles) g2 = ntiles;
-            if (g2 < 1) g2 = 1;
-            return launch_pdl(pmk::k_colw<T, L, 2>, (unsigned)g2, S::THREADS, pmk::colw_smem<T, L>(), st, b);
-        }
-    }
+    b.lgi = ilog2(((long long)4 * b.a[0].ny * b.a[0].nx) / pmk::WShape<T, L>::COLS);   // COLS divides the columns
+    if constexpr (L <= 256)
+        if (b.a[0].dmode == 3) return launch_tiles<ZPass<T, L, 2>>(b, st);   // both difference fields (see PairArgs)
     if (b.a[0].dmode == 3) return cudaErrorInvalidValue;
-    long long grid = (long long)(dm ? colw_blocks_per_sm<T, L, 1>() : colw_blocks_per_sm<T, L, 0>()) * num_sms();
-    if (grid > ntiles) grid = ntiles;
-    if (grid < 1) grid = 1;
-    if (dm) return launch_pdl(pmk::k_colw<T, L, 1>, (unsigned)grid, S::THREADS, pmk::colw_smem<T, L>(), st, b);
-    return launch_pdl(pmk::k_colw<T, L, 0>, (unsigned)grid, S::THREADS, pmk::colw_smem<T, L>(), st, b);
+    if (b.a[0].dmode != 0) return launch_tiles<ZPass<T, L, 1>>(b, st);
+    return launch_tiles<ZPass<T, L, 0>>(b, st);
 }
 template <typename T, int L> cudaError_t col_L(const PassBatch &b, int mode, cudaStream_t st) {
     if (mode == COL_YFWD) return col_LM<T, L, COL_YFWD>(b, st);
@@ -848,13 +830,13 @@ template <typename T> cudaError_t pm_set_attrs() {
 
 template <typename T> cudaError_t pm_launch_xfwd(PassBatch b, cudaStream_t st) {
     if (b.n < 1 || b.n > PM_BATCH) return cudaErrorInvalidValue;
-#define PM_XF(LL) pmk_host::xfwd_L<T, LL>(b, st)
+#define PM_XF(LL) pmk_host::xpass_L<T, LL, false>(b, st)
     PM_SWITCH_L(2 * b.a[0].nx, PM_XF)
 #undef PM_XF
 }
 template <typename T> cudaError_t pm_launch_xinv(PassBatch b, cudaStream_t st) {
     if (b.n < 1 || b.n > PM_BATCH) return cudaErrorInvalidValue;
-#define PM_XI(LL) pmk_host::xinv_L<T, LL>(b, st)
+#define PM_XI(LL) pmk_host::xpass_L<T, LL, true>(b, st)
     PM_SWITCH_L(2 * b.a[0].nx, PM_XI)
 #undef PM_XI
 }

@@ -14,14 +14,14 @@ struct PairArgs {
     void *phi_b;                          // Phi_b (null without partner)
     void *phi_sum;                        // Phi_a + Phi_b (or Phi_a)
     const void *hhat;                     // H-hat octant [nz+1][ny+1][nx+1]
-    const void *tw;                       // exp(-2 pi i m / L), m < L, this pass's L
+    const void *tw;                       // exp(-2 pi i m / L), m < L, this pass's L (FP64: fixed point, fxw)
     int nx, ny, nz;
     double scale;                         // 2^-s
     int *err;                             // 1: a tensor copy never completed; 2: an unsupported launch
     // Difference fields of an unpaired grid (rho_b null).  D_L(k) =
     // exp(2 pi i k / L) - 1 multiplies the spectrum of a field f into that of
     // its forward difference f[n+1] - f[n]; dtx, dty, dtz are tables of D for
-    // the x, y and z lengths.  dmode (z pass): 0 multiplies by H-hat,
+    // the x, y and z lengths (FP64: followed by D + i in units of 2^-59).  dmode (z pass): 0 multiplies by H-hat,
     // 1 by H-hat (D_x + i D_y), 2 by H-hat (D_z + i); the inverse of a real
     // field's spectrum times such a factor is fx + i fy, or fz + i Phi.
     // 3: both from one forward transform (L <= 64, H-hat from the
@@ -53,10 +53,10 @@ struct PassBatch {
 };
 
 // Columns per tile of the column passes for transform length L and real
-// size esz: 16 threads per column, 256 threads per block, and a tensor-map
-// box row of at most 256 eight-byte elements.
+// size esz: L/16 threads per column, 256 threads per block (FP64: 128), and a
+// tensor-map box row of at most 256 eight-byte elements.
 __host__ __device__ constexpr int pm_col_cols(int L, int esz) {
-    return (4096 / L) < (esz == 4 ? 256 : 128) ? (4096 / L) : (esz == 4 ? 256 : 128);
+    return (esz == 4 ? 4096 : 2048) / L;
 }
 
 // Columns per swizzled sub-tile of the z pass: as many as fill a 128-byte

@@ -1,4 +1,5 @@
-// FFT passes of the doubled-grid convolution (Sec. 2.1) on pair-packed mass
+// FFT passes of the doubled-grid convolution (Sec. 2.1), FP32 contexts
+// (pm_passes_fx.cuh: FP64), on pair-packed mass
 // sets: two real densities of one geometry (grids 2 and 3, or 4 and 5) travel
 // as one complex field rho_a + i rho_b, so every transform is a plain complex
 // FFT of power-of-two length and, H being real, the result is
@@ -807,18 +808,10 @@ __global__ void __launch_bounds__(WShape<T, L>::THREADS, ((L >= 512 || DM == 2) 
                 if (!fused(hcol + t * E, false, true)) break;
             } else if constexpr (hhat_thread_major(L)) {
                 const T *hz = hcol + t * E;   // 16-byte aligned: L, E multiples of 16
-                if constexpr (sizeof(T) == 4) {
 #pragma unroll
-                    for (int e = 0; e < E; e += 4) {
-                        const float4 h = __ldg(reinterpret_cast<const float4 *>(hz + e));
-                        hmul(e, h.x); hmul(e + 1, h.y); hmul(e + 2, h.z); hmul(e + 3, h.w);
-                    }
-                } else {
-#pragma unroll
-                    for (int e = 0; e < E; e += 2) {
-                        const double2 h = __ldg(reinterpret_cast<const double2 *>(hz + e));
-                        hmul(e, h.x); hmul(e + 1, h.y);
-                    }
+                for (int e = 0; e < E; e += 4) {
+                    const float4 h = __ldg(reinterpret_cast<const float4 *>(hz + e));
+                    hmul(e, h.x); hmul(e + 1, h.y); hmul(e + 2, h.z); hmul(e + 3, h.w);
                 }
             } else if constexpr (FREE) {
                 cp_async_wait_all();

@@ -24,6 +24,7 @@
 #include <mutex>
 
 #include "pm.h"
+#include "pm_fx.cuh"
 #include "pm_launch.h"
 
 #define PM_STATIC_SCRATCH_BYTES (32u << 20)
@@ -67,12 +68,17 @@ __global__ void k_static_cosmat(double *c, int n) {
 }
 
 template <typename T>
-__global__ void k_static_twiddles(typename cplx_t<T>::type *tw, int L) {
+__global__ void k_static_twiddles(typename comp_t<T>::W *tw, int L) {
     for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < L; m += gridDim.x * blockDim.x) {
         double s, c;
         sincospi(2.0 * (double)m / (double)L, &s, &c);
-        tw[m].x = (T)c;
-        tw[m].y = (T)(-s);
+        if constexpr (sizeof(T) == 4) {
+            tw[m].x = (T)c;
+            tw[m].y = (T)(-s);
+        } else {
+            pmfx::wsplit(__double2ll_rn(ldexp(c, pmfx::FX_Q)), tw[m].rh, tw[m].rl);
+            pmfx::wsplit(__double2ll_rn(-ldexp(s, pmfx::FX_Q)), tw[m].ih, tw[m].il);
+        }
     }
 }
 
@@ -115,9 +121,10 @@ int run(const int64_t *rho, void *phi, int nx, int ny, int nz, double l_xy, doub
     double *t1 = (double *)take(oct * sizeof(double));
     double *cm = (double *)take((size_t)nmax * nmax * sizeof(double));
     int *err = (int *)take(sizeof(int));
-    C *twx = (C *)take((size_t)2 * nx * sizeof(C));
-    C *twy = (C *)take((size_t)2 * ny * sizeof(C));
-    C *twz = (C *)take((size_t)2 * nz * sizeof(C));
+    typedef typename comp_t<T>::W W;   // as large as C
+    W *twx = (W *)take((size_t)2 * nx * sizeof(W));
+    W *twy = (W *)take((size_t)2 * ny * sizeof(W));
+    W *twz = (W *)take((size_t)2 * nz * sizeof(W));
 
 #define SCK(call)                                                                               \
     do {                                                                                        \

@@ -1,0 +1,85 @@
+"""The FP64 transforms run in block floating point (pm_fx.cuh): exponents,
+zeros and values that overflow, where the arithmetic differs from FP64's."""
+import numpy as np
+import pytest
+
+from paper_1210_1736_gb300 import pm, workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _potential(w, G=1.0, mb=None, pos=None, m=None):
+    ww = dict(w, system=dict(w["system"], G=G))
+    m = w["m"] if m is None else m
+    ctx = pm.Context(ww, W.mass_bound(m) if mb is None else mb)
+    p = pm.Particles(w["pos"] if pos is None else pos, w["vel"], m, w["gal"], precision="fp64")
+    ctx.deposit(p)
+    ctx.solve()
+    out = {key: ctx.potential(*key) for key in ctx.shapes}
+    ctx.close()
+    return out
+
+
+def _box(nx, ny, nz, n=2000):
+    w = W.big_box(n, 64, precision="fp64")
+    g = w["galaxies"][0]
+    g["coarse"] = (nx, ny, nz, g["coarse"][3], 1.0)
+    w["system"]["r_sys"] = 0.8 * pm.cell_length(g["coarse"][3], nx) * (min(nx, ny, nz) / 2 - 3)
+    return w
+
+
+@pytest.mark.parametrize("shape", [(8, 16, 32), (64, 8, 128), (16, 256, 8), (256, 8, 64), (8, 64, 256)])
+@pytest.mark.parametrize("k", [-820, -400, 31, 600, 820])
+def test_scale_invariance(shape, k):
+    """G 2^k scales every intermediate by 2^k exactly, also where a group's
+    exponent leaves the fast path of the conversion."""
+    w = _box(*shape)
+    a, b = _potential(w)[(0, 5)], _potential(w, G=2.0 ** k)[(0, 5)]
+    assert np.abs(a).max() > 0
+    assert np.array_equal(np.ldexp(a, k), b)
+
+
+def test_nested_scale_invariance():
+    """Grid 1's difference-field pass too."""
+    w = W.galaxy_small(precision="fp64", n_total=4000)
+    a, b = _potential(w), _potential(w, G=2.0 ** -300)
+    for key in a:
+        assert np.array_equal(np.ldexp(a[key], -300), b[key]), key
+
+
+def test_empty_density_is_zero():
+    w = _box(32, 16, 8)
+    p = _potential(w, pos=w["pos"] + 1e6)[(0, 5)]   # every particle lost
+    assert np.array_equal(p, np.zeros_like(p))
+
+
+def test_overflow_is_not_finite():
+    """A Green's function beyond the FP64 range gives no finite potential."""
+    w = _box(16, 16, 16)
+    with np.errstate(over="ignore"):
+        p = _potential(w, G=1e308, m=w["m"] * 1e6)[(0, 5)]
+    assert not np.isfinite(p).any()
+
+
+@pytest.mark.parametrize("heavy", [True, False])
+@pytest.mark.parametrize("shape", [(32, 32, 32), (128, 16, 16), (16, 16, 256)])
+def test_mass_range(shape, heavy):
+    """Masses of 2^-40 of the mass bound, whose integer densities have few
+    bits, alone and beside one heavy cell."""
+    import oracle as O
+    w = _box(*shape)
+    m = w["m"] * 2.0 ** -40
+    mb = W.mass_bound(w["m"])
+    pos = w["pos"].copy()
+    pos[:, 0] = 0.0
+    if heavy:
+        m[0] = w["m"][0]
+    p = _potential(w, m=m, mb=mb, pos=pos)[(0, 5)]
+    ww = dict(w, m=m, pos=pos)
+    s = O.system_from_workload(ww, mb)
+    st = O.state_from_workload(ww)
+    rho, flags, sh = O.deposit(st, s)
+    ref = O.solve_all(rho, s, sh)[0][5]
+    # both sides round the stored passes and numpy's every operation: a few
+    # units of 2^-53 of the largest value
+    assert np.abs(p - ref).max() <= 16 * 2.0 ** -53 * np.abs(ref).max()
