@@ -253,47 +253,6 @@ int check_particles(const pm_particles *p) {
     return PM_OK;
 }
 
-// --- H-hat: FP64 octant of H, three cosine sums, scaled into storage ---
-int build_hhat(pm_ctx *c, GeoBuf &gb) {
-    const pm_geometry &g = gb.g;
-    const int P = g.nx + 1, Q = g.ny + 1, R = g.nz + 1;
-    const long long n = (long long)P * Q * R;
-    double *h = nullptr, *t1 = nullptr, *cm = nullptr;
-    PM_CK(cudaMalloc(&h, n * sizeof(double)));
-    PM_CK(cudaMalloc(&t1, n * sizeof(double)));
-    const int nmax = std::max(P, std::max(Q, R));
-    PM_CK(cudaMalloc(&cm, (size_t)nmax * nmax * sizeof(double)));
-    std::vector<double> hm((size_t)nmax * nmax);
-    auto cosmat = [&](int nn) {   // w_i cos(pi m i / nn), m, i in [0, nn]
-        const int n1 = nn + 1;
-        for (int m = 0; m < n1; ++m)
-            for (int i = 0; i < n1; ++i) {
-                const long long r = ((long long)m * i) % (2LL * nn);
-                const double w = (i == 0 || i == nn) ? 1.0 : 2.0;
-                hm[(size_t)m * n1 + i] = w * std::cos(M_PI * (double)r / (double)nn);
-            }
-        return cudaMemcpyAsync(cm, hm.data(), (size_t)n1 * n1 * sizeof(double), cudaMemcpyHostToDevice, c->user);
-    };
-    cudaStream_t st = c->user;
-    PM_CK(pm_green_octant(h, g.nx, g.ny, g.nz, g.l_z / g.l_xy, c->sys.h000, st));
-    PM_CK(cosmat(g.nx));
-    PM_CK(pm_axis_transform(h, t1, cm, P, (long long)R * Q, 1, st));
-    PM_CK(cudaStreamSynchronize(st));
-    PM_CK(cosmat(g.ny));
-    PM_CK(pm_axis_transform(t1, h, cm, Q, R, P, st));
-    PM_CK(cudaStreamSynchronize(st));
-    PM_CK(cosmat(g.nz));
-    PM_CK(pm_axis_transform(h, t1, cm, R, 1, (long long)Q * P, st));
-    const double scale = c->sys.G / (g.l_xy * 8.0 * g.nx * g.ny * g.nz);
-    if (c->prec == PM_FP32) PM_CK(pm_store_hhat<float>(t1, (float *)gb.hhat, g.nx, g.ny, g.nz, scale, st));
-    else PM_CK(pm_store_hhat<double>(t1, (double *)gb.hhat, g.nx, g.ny, g.nz, scale, st));
-    PM_CK(cudaStreamSynchronize(st));
-    cudaFree(h);
-    cudaFree(t1);
-    cudaFree(cm);
-    return PM_OK;
-}
-
 // Tables of one transform length: the twiddles w^m = exp(-2 pi i m / L) and
 // D(m) = exp(2 pi i m / L) - 1 = -2 sin^2(pi m / L) + i sin(2 pi m / L) (the
 // half-angle form keeps the real part accurate for small m).
@@ -325,8 +284,12 @@ struct FxTables {
         }
     }
 };
-void make_tables(int L, std::vector<fxw> &tw, std::vector<double2> &dt) {
+const FxTables &fx_tables() {
     static const FxTables t;
+    return t;
+}
+void make_tables(int L, std::vector<fxw> &tw, std::vector<double2> &dt) {
+    const FxTables &t = fx_tables();
     for (int m = 0; m < L; ++m) {
         tw.push_back(t.tw[m * (512 / L)]);
         dt.push_back(t.d[m * (512 / L)]);
@@ -337,6 +300,29 @@ void make_tables(int L, std::vector<fxw> &tw, std::vector<double2> &dt) {
         dt.push_back(z);
     }
 }
+// H-hat of every geometry.
+int build_hhat(pm_ctx *c) {
+    cudaStream_t st = c->user;
+    size_t n = 0;
+    for (const GeoBuf &gb : c->geos) n = std::max(n, (size_t)(gb.g.nx + 1) * (gb.g.ny + 1) * (gb.g.nz + 1));
+    const FxTables &t = fx_tables();
+    unsigned char *tmp = nullptr;   // the twiddles and one octant
+    PM_CK(cudaMalloc(&tmp, sizeof(t.tw) + n * sizeof(double)));
+    cudaError_t e = cudaMemcpyAsync(tmp, t.tw, sizeof(t.tw), cudaMemcpyHostToDevice, st);
+    for (const GeoBuf &gb : c->geos) {
+        const pm_geometry &g = gb.g;
+        const double q = g.l_z / g.l_xy, scale = c->sys.G / (g.l_xy * 8.0 * g.nx * g.ny * g.nz);
+        double *h = (double *)(tmp + sizeof(t.tw));
+        if (e != cudaSuccess) break;
+        e = c->prec == PM_FP32 ? pm_build_hhat<float>(h, (float *)gb.hhat, (fxw *)tmp, g.nx, g.ny, g.nz, q, c->sys.h000, scale, st)
+                               : pm_build_hhat<double>(h, (double *)gb.hhat, (fxw *)tmp, g.nx, g.ny, g.nz, q, c->sys.h000, scale, st);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    cudaFree(tmp);
+    if (e != cudaSuccess) return fail(PM_E_CUDA, "H-hat: %s", cudaGetErrorString(e));
+    return PM_OK;
+}
+
 template <typename T> int upload_twiddles(pm_ctx *c) {
     for (int i = 0; i < 6; ++i) {
         std::vector<typename comp_t<T>::W> tw;
@@ -1200,10 +1186,9 @@ int pm_create_grids(const pm_system *sys, const pm_galaxy *gals, void *stream, p
             return cleanup(fail(PM_E_CUDA, "cudaEventCreate failed"));
         c->ev_join.push_back(e);
     }
-    for (GeoBuf &gb : c->geos) {
+    for (GeoBuf &gb : c->geos)
         if ((rc = dev_alloc(c, &gb.hhat, gb.hatN * c->esz))) return cleanup(rc);
-        if ((rc = build_hhat(c, gb))) return cleanup(rc);
-    }
+    if ((rc = build_hhat(c))) return cleanup(rc);
     if ((rc = (c->prec == PM_FP32 ? upload_twiddles<float>(c) : upload_twiddles<double>(c)))) return cleanup(rc);
 
     // system description for the particle kernels

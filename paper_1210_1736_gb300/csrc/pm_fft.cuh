@@ -48,13 +48,13 @@ __host__ __device__ constexpr int tw_offset(int L, int S, bool rev) {
 }
 __host__ __device__ constexpr int tw_total(int L) { return tw_dir_size(L, false) + tw_dir_size(L, true); }
 
-template <int L, int S, bool REV, typename C>
+template <int L, int S, bool REV, int STEP = 1, typename C>   // g: every STEP-th entry is w^m
 __device__ __forceinline__ void expand_stage_twiddles(C *tab, const C *g) {
     if (S >= nstages(L)) return;
     constexpr int Ns = stride_before(L, S, REV), R = radix(L, S, REV), OFF = tw_offset(L, S, REV);
     for (int i = threadIdx.x; i < Ns * R; i += blockDim.x) {
         const int r = i / Ns, jm = i % Ns;
-        tab[OFF + i] = g[(jm * r * (L / (Ns * R))) & (L - 1)];
+        tab[OFF + i] = g[((jm * r * (L / (Ns * R))) & (L - 1)) * STEP];
     }
 }
 // Builds the stage tables in shared memory from the plain table

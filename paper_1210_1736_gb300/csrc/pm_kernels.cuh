@@ -649,26 +649,6 @@ __global__ void k_count_lost(PartK<T> p, unsigned long long *out) {
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
 }
 
-template <typename T, int L>
-__global__ void k_store_hhat(const double *oct, T *out, int nx, int ny, double scale) {
-    constexpr int NS = nstages(L), RL = radix(L, NS - 1, false), HS = pm_hhat_stride(L);
-    const long long ncol = (long long)(nx + 1) * (ny + 1);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < ncol * HS;
-         i += (long long)gridDim.x * blockDim.x) {
-        const long long col = i / HS;
-        const int w = (int)(i % HS);
-        int kzr;
-        if (hhat_thread_major(L)) {   // register w % 16 of thread w / 16
-            const int e = w % E, t = w / E;
-            const int kz = pmfft::in_row<L, NS - 1, false>(t, e / RL, e % RL);
-            kzr = kz <= L / 2 ? kz : L - kz;
-        } else {
-            kzr = w;                  // padding beyond nz = L/2
-        }
-        out[i] = kzr <= L / 2 ? (T)(oct[(long long)kzr * ncol + col] * scale) : (T)0;
-    }
-}
-
 }  // namespace pmk
 
 // ---------------------------------------------------------------------------
@@ -916,14 +896,6 @@ cudaError_t pm_launch_count_lost(const PartK<T> &p, unsigned long long *out, cud
     return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t pm_store_hhat(const double *oct, T *out, int nx, int ny, int nz, double scale, cudaStream_t st) {
-    const int g = pmk_host::particle_grid(pm_hhat_table_size(nx, ny, nz));
-#define PM_SH(LL) (pmk::k_store_hhat<T, LL><<<g, 256, 0, st>>>(oct, out, nx, ny, scale), cudaGetLastError())
-    PM_SWITCH_L(2 * nz, PM_SH)
-#undef PM_SH
-}
-
 #define PM_INSTANTIATE(T)                                                                                       \
     template cudaError_t pm_set_attrs<T>();                                                                    \
     template cudaError_t pm_launch_xfwd<T>(PassBatch, cudaStream_t);                                          \
@@ -937,5 +909,4 @@ cudaError_t pm_store_hhat(const double *oct, T *out, int nx, int ny, int nz, dou
     template cudaError_t pm_launch_count_lost<T>(const PartK<T> &, unsigned long long *, cudaStream_t);       \
     template cudaError_t pm_launch_sort<T>(const PartK<T> &, const PartK<T> &, const SysK &, const CenK *,     \
                                            const SortK &, unsigned *, unsigned *, unsigned *, unsigned *,       \
-                                           long long *, cudaStream_t);                                          \
-    template cudaError_t pm_store_hhat<T>(const double *, T *, int, int, int, double, cudaStream_t);
+                                           long long *, cudaStream_t);

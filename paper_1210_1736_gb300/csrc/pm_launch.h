@@ -156,15 +156,12 @@ template <typename T> cudaError_t pm_launch_diag_sums(const pmk::DiagP<T> &d, co
 template <typename T> cudaError_t pm_launch_diag_heat(const pmk::DiagP<T> &d, const double *xp, const double *fp,
                                                       int np, double *acc, cudaStream_t st);
 
-// FP64 H-hat construction (precision independent) and storage conversion.
-cudaError_t pm_green_octant(double *h, int nx, int ny, int nz, double q, double h000, cudaStream_t st);
-cudaError_t pm_axis_transform(const double *in, double *out, const double *cmat, int n1,
-                              long long outer, long long inner, cudaStream_t st);
-// H-hat table of the z pass from the FP64 octant oct[kzr][kyr][kxr]
-// (scaled by `scale`): for each octant column (kyr, kxr), for L = 2nz >= 128
-// the nz + 1 values H-hat(kzr) padded with zeros to pm_hhat_stride(L); for
-// L <= 64 the L values H-hat(kz) (kz > L/2 mirrored) in thread-major order,
-// register e of thread t at entry t * 16 + e (hhat_thread_major).
+// H-hat table of the z pass, scaled by `scale`: for each octant column
+// (kyr, kxr), for L = 2nz >= 128 the nz + 1 values H-hat(kzr) padded with
+// zeros to pm_hhat_stride(L); for L <= 64 the L values H-hat(kz) (kz > L/2
+// mirrored) in thread-major order, register e of thread t at entry t * 16 + e
+// (hhat_thread_major).  h: FP64 scratch of the octant's (nz+1)(ny+1)(nx+1)
+// values; tw: the fixed-point twiddles exp(-2 pi i m / 512), m < 512.
 // For L = 2nz >= 128 each octant column holds only H-hat(kzr), kzr = 0..nz,
 // padded to pm_hhat_stride(L) values: the smallest h >= nz + 1 with
 // h = TPC (mod 2 TPC), TPC = L/16 threads per column, so that the columns of
@@ -177,8 +174,10 @@ __host__ __device__ constexpr int pm_hhat_stride(int L) {
 inline long long pm_hhat_table_size(int nx, int ny, int nz) {
     return (long long)(nx + 1) * (ny + 1) * pm_hhat_stride(2 * nz);
 }
+struct fxw;
 template <typename T>
-cudaError_t pm_store_hhat(const double *oct, T *out, int nx, int ny, int nz, double scale, cudaStream_t st);
+cudaError_t pm_build_hhat(double *h, T *out, const fxw *tw, int nx, int ny, int nz, double q, double h000, double scale,
+                          cudaStream_t st);
 
 // Self-test of the bounded waits: one block waits on an mbarrier nothing
 // arrives at, gives up after the time limit and sets *err to 1.

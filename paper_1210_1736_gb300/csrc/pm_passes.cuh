@@ -797,7 +797,7 @@ __global__ void __launch_bounds__(WShape<T, L>::THREADS, ((L >= 512 || DM == 2) 
                 }
             }
         } else {
-            // H-hat of column (kyr, kxr), stored by pm_store_hhat in the
+            // H-hat of column (kyr, kxr), stored by pm_build_hhat in the
             // order hhat_thread_major gives for L
             const int q = lt * S::COLS + c;
             const int ky = q >> lnx2, kx = q & (nx2 - 1);   // nx2 is a power of two

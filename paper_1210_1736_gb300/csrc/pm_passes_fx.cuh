@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(FXT, DM == 2 ? 2 : 3) k_zfx(const __grid_const
         const int kyr = ky <= a.ny ? ky : ny2 - ky, kxr = kx <= a.nx ? kx : nx2 - kx;
         const double *hcol = ihhat[tile >> lgi] + ((size_t)kyr * (a.nx + 1) + kxr) * S::HS;
         auto slot_of = [&](int e) { return in + woff<double, L, S::RIN>(t + e * TPC, c); };
-        // H-hat of row kz (pm_store_hhat's order): register e of the last
+        // H-hat of row kz (pm_build_hhat's order): register e of the last
         // stage's order holds row kz, entry t * 16 + e of a thread-major table
         auto hval = [&](int e) {
             if constexpr (hhat_thread_major(L)) {

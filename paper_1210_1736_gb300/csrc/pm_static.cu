@@ -57,29 +57,25 @@ int sfail(int code, const char *fmt, ...) {
     return pm_internal_fail(code, buf);
 }
 
-__global__ void k_static_cosmat(double *c, int n) {
-    // c[m][i] = w_i cos(pi m i / n), w_0 = w_n = 1, else 2 (n a power of two)
-    const int n1 = n + 1;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n1 * n1; e += gridDim.x * blockDim.x) {
-        const int m = e / n1, i = e % n1;
-        const long long r = ((long long)m * i) % (2LL * n);
-        c[e] = ((i == 0 || i == n) ? 1.0 : 2.0) * cospi((double)r / (double)n);
-    }
+__device__ __forceinline__ void put_twiddle(float2 &w, double c, double s) { w = make_float2((float)c, (float)(-s)); }
+__device__ __forceinline__ void put_twiddle(fxw &w, double c, double s) {
+    pmfx::wsplit(__double2ll_rn(ldexp(c, pmfx::FX_Q)), w.rh, w.rl);
+    pmfx::wsplit(__double2ll_rn(-ldexp(s, pmfx::FX_Q)), w.ih, w.il);
 }
 
+// First kernel of a call: the passes' twiddles (three lengths), the H-hat
+// build's (length 512), and the error word's reset.
 template <typename T>
-__global__ void k_static_twiddles(typename comp_t<T>::W *tw, int L) {
-    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < L; m += gridDim.x * blockDim.x) {
-        double s, c;
-        sincospi(2.0 * (double)m / (double)L, &s, &c);
-        if constexpr (sizeof(T) == 4) {
-            tw[m].x = (T)c;
-            tw[m].y = (T)(-s);
-        } else {
-            pmfx::wsplit(__double2ll_rn(ldexp(c, pmfx::FX_Q)), tw[m].rh, tw[m].rl);
-            pmfx::wsplit(__double2ll_rn(-ldexp(s, pmfx::FX_Q)), tw[m].ih, tw[m].il);
-        }
-    }
+__global__ void k_static_tables(typename comp_t<T>::W *twx, int lx, typename comp_t<T>::W *twy, int ly,
+                                typename comp_t<T>::W *twz, int lz, fxw *tw512, int *err) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) *err = 0;
+    const int L = blockIdx.y == 0 ? lx : blockIdx.y == 1 ? ly : blockIdx.y == 2 ? lz : 512;
+    if (i >= L) return;
+    double s, c;
+    sincospi(2.0 * (double)i / (double)L, &s, &c);
+    if (blockIdx.y == 3) put_twiddle(tw512[i], c, s);
+    else put_twiddle((blockIdx.y == 0 ? twx : blockIdx.y == 1 ? twy : twz)[i], c, s);
 }
 
 // Last kernel of a call: if a pass's bounded wait expired (*err set), the
@@ -111,15 +107,13 @@ int run(const int64_t *rho, void *phi, int nx, int ny, int nz, double l_xy, doub
         int shift, unsigned char *base, cudaStream_t st) {
     typedef typename cplx_t<T>::type C;
     const size_t oct = (size_t)(nx + 1) * (ny + 1) * (nz + 1);
-    const int nmax = std::max(nx, std::max(ny, nz)) + 1;
     int *status = (int *)base;
     size_t off = PM_STATIC_STATUS_BYTES;
     auto take = [&](size_t bytes) { unsigned char *p = base + off; off += up256(bytes); return p; };
     C *work = (C *)take((size_t)nz * 2 * ny * 2 * nx * sizeof(C));
     T *hhat = (T *)take((size_t)pm_hhat_table_size(nx, ny, nz) * sizeof(T));
     double *h = (double *)take(oct * sizeof(double));
-    double *t1 = (double *)take(oct * sizeof(double));
-    double *cm = (double *)take((size_t)nmax * nmax * sizeof(double));
+    fxw *tw512 = (fxw *)take(512 * sizeof(fxw));
     int *err = (int *)take(sizeof(int));
     typedef typename comp_t<T>::W W;   // as large as C
     W *twx = (W *)take((size_t)2 * nx * sizeof(W));
@@ -132,26 +126,12 @@ int run(const int64_t *rho, void *phi, int nx, int ny, int nz, double l_xy, doub
         if (e_ != cudaSuccess) return sfail(PM_E_CUDA, "%s: %s", #call, cudaGetErrorString(e_)); \
     } while (0)
 
-    k_static_twiddles<T><<<1, 256, 0, st>>>(twx, 2 * nx);
-    k_static_twiddles<T><<<1, 256, 0, st>>>(twy, 2 * ny);
-    k_static_twiddles<T><<<1, 256, 0, st>>>(twz, 2 * nz);
+    k_static_tables<T><<<dim3(4, 4), 128, 0, st>>>(twx, 2 * nx, twy, 2 * ny, twz, 2 * nz, tw512, err);
     SCK(cudaGetLastError());
-    // H-hat: FP64 octant of H, three cosine sums (x, y, z), scaled into T
-    SCK(pm_green_octant(h, nx, ny, nz, l_z / l_xy, h000, st));
-    k_static_cosmat<<<64, 256, 0, st>>>(cm, nx);
-    SCK(cudaGetLastError());
-    SCK(pm_axis_transform(h, t1, cm, nx + 1, (long long)(nz + 1) * (ny + 1), 1, st));
-    k_static_cosmat<<<64, 256, 0, st>>>(cm, ny);
-    SCK(cudaGetLastError());
-    SCK(pm_axis_transform(t1, h, cm, ny + 1, nz + 1, nx + 1, st));
-    k_static_cosmat<<<64, 256, 0, st>>>(cm, nz);
-    SCK(cudaGetLastError());
-    SCK(pm_axis_transform(h, t1, cm, nz + 1, 1, (long long)(ny + 1) * (nx + 1), st));
-    SCK(pm_store_hhat<T>(t1, hhat, nx, ny, nz, G / (l_xy * 8.0 * nx * ny * nz), st));
+    SCK(pm_build_hhat<T>(h, hhat, tw512, nx, ny, nz, l_z / l_xy, h000, G / (l_xy * 8.0 * nx * ny * nz), st));
 
     CUtensorMap yfwd, yinv, zmap;
     if (pm_encode_col_maps(work, nx, ny, nz, (int)sizeof(T), &yfwd, &yinv, &zmap) != PM_OK) return PM_E_CUDA;
-    SCK(cudaMemsetAsync(err, 0, sizeof(int), st));
     PairArgs a;
     std::memset(&a, 0, sizeof(a));
     a.rho_a = (const long long *)rho;
@@ -178,6 +158,9 @@ int run(const int64_t *rho, void *phi, int nx, int ny, int nz, double l_xy, doub
     return PM_OK;
 }
 
+// The size that decides which grids are taken: at least what run() lays out,
+// but for the smallest grids (its one octant and table of 8 KB against two
+// octants here), which are far below the limit.
 size_t scratch_bytes(int nx, int ny, int nz, size_t esz) {
     const size_t oct = (size_t)(nx + 1) * (ny + 1) * (nz + 1);
     const size_t nmax = std::max(nx, std::max(ny, nz)) + 1;
