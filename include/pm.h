@@ -234,7 +234,7 @@ int pm_selftest_wait_expiry(pm_ctx *ctx);
  * 2^21 bins); lost particles go last.  Order within a cell is unspecified.
  * If perm is not NULL (device int64[n]) it receives perm[new] = old.
  * Results of the step do not depend on the order.  Allocates its scratch
- * (about 44 bytes per particle) on first use. */
+ * (about 48 bytes per particle) on first use. */
 int pm_sort(pm_ctx *ctx, const pm_particles *p, int64_t *perm);
 /* pm_step re-sorts the particles before every k-th step (k = 0: never, the
  * default); resets the step counter so the next step sorts. */
@@ -309,8 +309,8 @@ int pm_cic_vjp(pm_ctx *ctx, const pm_particles *p, const void *ux, const void *u
  * out (host, 6 + 4 nbins + 2 nring mmax doubles): [n, E_heat, sigma_R,
  * sigma_phi, sigma_z, annulus mass, then per bin (mean R, count,
  * sqrt<z^2>, mean v_phi), then per ring and mode (Re A~_m, Im A~_m)].
- * Synchronises (the bin edges take 8 radix passes with a host step each);
- * allocates 0.1 MB of scratch on the first call. */
+ * Synchronises; allocates its scratch (0.5 MB and 48 bytes per particle) on
+ * the first call and when n grows. */
 typedef struct {
     int32_t gal;
     int32_t nbins;

@@ -201,10 +201,10 @@ struct pm_ctx {
     size_t bytes = 0;
     std::vector<void *> allocs;
     bool any_recentre = false;
-    // disc diagnostics scratch (allocated on first use)
-    unsigned *dg_hist = nullptr;
-    unsigned long long *dg_pref = nullptr, *dg_edges = nullptr;
-    double *dg_acc = nullptr, *dg_tab = nullptr;
+    // disc diagnostics scratch (allocated on first use, the particles' part
+    // grown as needed)
+    pmk::DiagBuf dg = {};
+    long long dg_cap = 0;
 };
 
 namespace {
@@ -802,21 +802,22 @@ template <typename T> int cic_vjp_impl(pm_ctx *c, const pm_particles *p, const v
 }
 
 // ---- disc diagnostics (Sec. 6 quantities) ----------------------------------
-constexpr int DG_MAXBINS = 64, DG_MAXRM = 1024;
+constexpr int DG_MAXBINS = pmk::DIAG_MAXBINS, DG_MAXRM = 1024;
 
 template <typename T> int disc_impl(pm_ctx *c, const pm_particles *p, const uint8_t *sel, const pm_disc_query *q,
                                     double *out) {
     cudaStream_t st = c->user;
-    if (!c->dg_hist) {
-        PM_TRY(dev_alloc(c, (void **)&c->dg_hist, sizeof(unsigned) * 256 * DG_MAXBINS));
-        PM_TRY(dev_alloc(c, (void **)&c->dg_pref, sizeof(unsigned long long) * DG_MAXBINS));
-        PM_TRY(dev_alloc(c, (void **)&c->dg_edges, sizeof(unsigned long long) * DG_MAXBINS));
-        PM_TRY(dev_alloc(c, (void **)&c->dg_acc, sizeof(double) * (4 * DG_MAXBINS + 8 + 2 * DG_MAXRM)));
-        PM_TRY(dev_alloc(c, (void **)&c->dg_tab, sizeof(double) * 2 * DG_MAXBINS));
+    if (!c->dg.acc) {
+        PM_TRY(dev_alloc(c, (void **)&c->dg.state, sizeof(pmk::DiagState)));
+        PM_TRY(dev_alloc(c, (void **)&c->dg.hist, sizeof(unsigned) * 2048 * DG_MAXBINS));
+        PM_TRY(dev_alloc(c, (void **)&c->dg.acc, sizeof(double) * (4 * DG_MAXBINS + 8 + 2 * DG_MAXRM)));
     }
-    CenK ck;
-    PM_CK(cudaMemcpyAsync(&ck, c->d_cen, sizeof(CenK), cudaMemcpyDeviceToHost, st));
-    PM_CK(cudaStreamSynchronize(st));
+    if (p->n > c->dg_cap) {
+        PM_TRY(dev_alloc(c, (void **)&c->dg.key, sizeof(unsigned long long) * p->n));
+        PM_TRY(dev_alloc(c, (void **)&c->dg.idx, sizeof(long long) * p->n));
+        PM_TRY(dev_alloc(c, (void **)&c->dg.rest, sizeof(double4) * p->n));
+        c->dg_cap = p->n;
+    }
     pmk::DiagP<T> d;
     d.x = (const T *)p->x; d.y = (const T *)p->y; d.z = (const T *)p->z;
     d.vx = (const T *)p->vx; d.vy = (const T *)p->vy; d.vz = (const T *)p->vz;
@@ -826,62 +827,25 @@ template <typename T> int disc_impl(pm_ctx *c, const pm_particles *p, const uint
     d.gal_id = p->gal;
     d.gal = q->gal;
     d.n = p->n;
-    for (int k = 0; k < 3; ++k) d.c[k] = ck.c[q->gal][k];
     const int B = q->nbins, NR = q->nring, MM = q->mmax;
     const int nacc = 4 * B + 7 + 2 * NR * MM;
     const int nout = 6 + 4 * B + 2 * NR * MM;
     for (int k = 0; k < nout; ++k) out[k] = 0.0;
-
-    // exact bin edges: order statistics of R^2 at ranks floor(k n / B)
-    std::vector<unsigned long long> key(B > 1 ? B - 1 : 0, 0ull);
-    std::vector<long long> rank(key.size(), 0);
-    long long nsel = -1;
-    std::vector<unsigned> h(256 * DG_MAXBINS);
-    for (int pass = 0; pass < 8 && (!key.empty()); ++pass) {
-        std::vector<unsigned long long> uniq(key.begin(), key.end());
-        std::sort(uniq.begin(), uniq.end());
-        uniq.erase(std::unique(uniq.begin(), uniq.end()), uniq.end());
-        const int np = pass == 0 ? 1 : (int)uniq.size();
-        PM_CK(cudaMemcpyAsync(c->dg_pref, uniq.data(), sizeof(unsigned long long) * np, cudaMemcpyHostToDevice, st));
-        PM_CK(cudaMemsetAsync(c->dg_hist, 0, sizeof(unsigned) * 256 * np, st));
-        PM_CK(pm_launch_diag_hist<T>(d, pass, c->dg_pref, np, c->dg_hist, st));
-        PM_CK(cudaMemcpyAsync(h.data(), c->dg_hist, sizeof(unsigned) * 256 * np, cudaMemcpyDeviceToHost, st));
-        PM_CK(cudaStreamSynchronize(st));
-        if (pass == 0) {
-            nsel = 0;
-            for (int b = 0; b < 256; ++b) nsel += h[b];
-            if (nsel == 0) return check_device_error(c);
-            for (int k = 1; k < B; ++k) rank[k - 1] = ((long long)k * nsel) / B;
-        }
-        for (size_t k = 0; k < key.size(); ++k) {
-            const int j = pass == 0 ? 0 : (int)(std::lower_bound(uniq.begin(), uniq.end(), key[k]) - uniq.begin());
-            long long cum = 0;
-            int dgt = 0;
-            for (; dgt < 256; ++dgt) {
-                if (cum + h[j * 256 + dgt] > rank[k]) break;
-                cum += h[j * 256 + dgt];
-            }
-            if (dgt == 256) return fail(PM_E_STATE, "radix select lost a rank (particles changed during the call?)");
-            key[k] = (key[k] << 8) | (unsigned long long)dgt;
-            rank[k] -= cum;
-        }
-    }
-    if (!key.empty())
-        PM_CK(cudaMemcpyAsync(c->dg_edges, key.data(), sizeof(unsigned long long) * key.size(), cudaMemcpyHostToDevice,
-                              st));
     pmk::DiagQ dq;
     dq.nbins = B; dq.nring = NR; dq.mmax = MM;
     dq.r_ring = q->r_ring;
     dq.width = NR > 0 ? q->r_ring / NR : 1.0;
     dq.rlo = q->r0 - q->dr;
     dq.rhi = q->r0 + q->dr;
-    PM_CK(cudaMemsetAsync(c->dg_acc, 0, sizeof(double) * (nacc + 1), st));
-    PM_CK(pm_launch_diag_sums<T>(d, dq, c->dg_edges, c->dg_acc, st));
+    PM_CK(pm_launch_diag<T>(d, c->d_cen, dq, c->dg, st));
     std::vector<double> acc(nacc + 1);
-    PM_CK(cudaMemcpyAsync(acc.data(), c->dg_acc, sizeof(double) * nacc, cudaMemcpyDeviceToHost, st));
-    PM_CK(cudaStreamSynchronize(st));
+    pmk::DiagState ds;
+    PM_CK(cudaMemcpyAsync(acc.data(), c->dg.acc, sizeof(double) * (nacc + 1), cudaMemcpyDeviceToHost, st));
+    PM_CK(cudaMemcpyAsync(&ds, c->dg.state, sizeof(ds), cudaMemcpyDeviceToHost, st));
+    PM_TRY(check_device_error(c));   // synchronises
+    if (ds.err) return fail(PM_E_STATE, "radix select lost a rank (particles changed during the call?)");
+    if (ds.nsel == 0) return PM_OK;
 
-    std::vector<double> xp, fp;
     long long ntot = 0;
     for (int b = 0; b < B; ++b) {
         const double cnt = acc[4 * b + 1];
@@ -892,8 +856,6 @@ template <typename T> int disc_impl(pm_ctx *c, const pm_particles *p, const uint
             o[0] = acc[4 * b] / cnt;
             o[2] = std::sqrt(acc[4 * b + 2] / cnt);
             o[3] = acc[4 * b + 3] / cnt;
-            xp.push_back(o[0]);
-            fp.push_back(o[3]);
         }
     }
     out[0] = (double)ntot;
@@ -913,16 +875,8 @@ template <typename T> int disc_impl(pm_ctx *c, const pm_particles *p, const uint
         for (int mo = 0; mo < MM; ++mo)
             for (int k = 0; k < 2; ++k) out[6 + 4 * B + 2 * (r * MM + mo) + k] = a[7 + 2 * (r * MM + mo) + k] / S;
     }
-    if (!xp.empty()) {
-        std::vector<double> tab(xp);
-        tab.insert(tab.end(), fp.begin(), fp.end());
-        PM_CK(cudaMemcpyAsync(c->dg_tab, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice, st));
-        PM_CK(cudaMemsetAsync(c->dg_acc + nacc, 0, sizeof(double), st));
-        PM_CK(pm_launch_diag_heat<T>(d, c->dg_tab, c->dg_tab + xp.size(), (int)xp.size(), c->dg_acc + nacc, st));
-        PM_CK(cudaMemcpyAsync(&out[1], c->dg_acc + nacc, sizeof(double), cudaMemcpyDeviceToHost, st));
-        PM_CK(cudaStreamSynchronize(st));
-    }
-    return check_device_error(c);
+    out[1] = acc[nacc];
+    return PM_OK;
 }
 
 template <typename T> int force_impl(pm_ctx *c, int mode, const pm_particles *p, double dt, void *ax, void *ay,
@@ -1399,9 +1353,9 @@ int pm_diagnostics(pm_ctx *c, const pm_particles *p, double dt, double *out) {
     PM_TRY(PM_DISPATCH(c, force_impl, c, 3, p, dt, nullptr, nullptr, nullptr, c->d_diag));
     double h[8];
     PM_CK(cudaMemcpyAsync(h, c->d_diag, sizeof(h), cudaMemcpyDeviceToHost, c->user));
-    PM_CK(cudaStreamSynchronize(c->user));
+    const int rc = check_device_error(c);   // synchronises
     for (int k = 0; k < 7; ++k) out[k] = h[k];
-    return check_device_error(c);
+    return rc;
 }
 
 int pm_cic_deposit(pm_ctx *c, const pm_particles *p) {

@@ -3,11 +3,19 @@
 // annulus, Fourier modes A~_m in rings) as FP64 reductions over the selected
 // particles, positions and velocities taken relative to a galaxy centre.
 //
-// Radial bins of equal particle numbers are bounded by exact order
-// statistics of R^2: an MSD radix select over the IEEE bits of R^2 (a
-// non-negative double, so its bits order like its value), 8 bits per pass,
-// one histogram per distinct prefix of the boundaries still being resolved.
+// Bound by the FP64 pipe (2 lanes per clock and SM), so nothing is computed
+// twice and nothing returns to the host in between: one pass compacts the
+// selected particles' R^2 and index; the bins' bounds, exact order statistics
+// of R^2, come from a radix select over the IEEE bits of R^2 (a non-negative
+// double, so its bits order like its value) whose digits are resolved on the
+// device; one pass forms every sum and leaves what the heat needs.  1M
+// particles, 400k selected, launches under ncu: radix passes over all particles
+// 353 us (and a host step each), sums by FP64 shared atomics 318, heat 130;
+// now select and radix passes 155, sums 113 (FP64 operations and read-modify-
+// writes of 4 warps per SM, as many as the columns leave room for), heat 18.
 #pragma once
+
+#include <algorithm>
 
 #include "pm_launch.h"
 #include "pm_particle.cuh"
@@ -20,119 +28,329 @@ __device__ __forceinline__ bool diag_take(const DiagP<T> &d, long long i) {
     return d.sel ? d.sel[i] != 0 : d.gal_id[i] == d.gal;
 }
 
-// R^2 with the same operations as the FP64 reference (no contraction).
+// Compacts the selected particles: key = bits of R^2 (the same operations as
+// the FP64 reference, no contraction) and index, in blocks of 1024 particles.
 template <typename T>
-__device__ __forceinline__ double diag_r2(const DiagP<T> &d, long long i, double &dx, double &dy) {
-    dx = __dsub_rn((double)d.x[i], d.c[0]);
-    dy = __dsub_rn((double)d.y[i], d.c[1]);
-    return __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
-}
-
-// One pass of the radix select: particles whose key agrees with one of the
-// npref sorted prefixes (the key's top 8*pass bits) count their next digit.
-template <typename T>
-__global__ void __launch_bounds__(256) k_diag_hist(DiagP<T> d, int pass, const unsigned long long *pref, int npref,
-                                                   unsigned *hist) {
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < d.n; i += stride) {
-        if (!diag_take(d, i)) continue;
-        double dx, dy;
-        const unsigned long long key = (unsigned long long)__double_as_longlong(diag_r2(d, i, dx, dy));
-        int j = 0;
-        if (pass > 0) {
-            const unsigned long long pk = key >> (64 - 8 * pass);
-            int lo = 0, hi = npref - 1;
-            j = -1;
-            while (lo <= hi) {
-                const int mid = (lo + hi) >> 1;
-                if (pref[mid] == pk) { j = mid; break; }
-                if (pref[mid] < pk) lo = mid + 1; else hi = mid - 1;
-            }
-            if (j < 0) continue;
+__global__ void __launch_bounds__(256) k_diag_select(DiagP<T> d, const CenK *cen, DiagState *st,
+                                                     unsigned long long *key, long long *idx) {
+    __shared__ int wtot[8];
+    __shared__ unsigned long long base;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const double cx = cen->c[d.gal][0], cy = cen->c[d.gal][1];
+    for (long long b = (long long)blockIdx.x * 1024; b < d.n; b += (long long)gridDim.x * 1024) {
+        bool take[4];
+        unsigned before[4];
+        int tot = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const long long i = b + u * 256 + threadIdx.x;
+            take[u] = i < d.n && diag_take(d, i);
         }
-        atomicAdd(hist + j * 256 + (int)((key >> (56 - 8 * pass)) & 255u), 1u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const unsigned m = __ballot_sync(0xffffffffu, take[u]);
+            before[u] = tot + __popc(m & ((1u << lane) - 1u));
+            tot += __popc(m);
+        }
+        if (lane == 0) wtot[w] = tot;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int s = 0;
+            for (int k = 0; k < 8; ++k) {
+                const int v = wtot[k];
+                wtot[k] = s;
+                s += v;
+            }
+            base = s ? atomicAdd(&st->nsel, (unsigned long long)s) : 0;
+        }
+        __syncthreads();
+        const long long o = (long long)base + wtot[w];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (take[u]) {
+                const long long i = b + u * 256 + threadIdx.x;
+                const double dx = __dsub_rn((double)d.x[i], cx), dy = __dsub_rn((double)d.y[i], cy);
+                key[o + before[u]] = (unsigned long long)__double_as_longlong(
+                    __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
+                idx[o + before[u]] = i;
+            }
+        __syncthreads();   // wtot and base are rewritten
     }
 }
 
-__device__ __forceinline__ void diag_add(double *sh, int k, double v) { atomicAdd(sh + k, v); }
+// Digits of the radix select: DG_BITS bits per pass from the top, the last
+// pass the remaining ones.
+constexpr int DG_BITS = 11, DG_PASSES = 6, DG_ROW = 1 << DG_BITS;
+__device__ __forceinline__ int diag_low(int pass) { return pass + 1 < DG_PASSES ? 64 - DG_BITS * (pass + 1) : 0; }
+__device__ __forceinline__ int diag_high(int pass) { return 64 - DG_BITS * pass; }
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_diag_sums(DiagP<T> d, DiagQ q, const unsigned long long *edges,
-                                                   double *acc) {
-    extern __shared__ double sh[];
-    const int nacc = 4 * q.nbins + 7 + 2 * q.nring * q.mmax;
-    for (int k = threadIdx.x; k < nacc; k += blockDim.x) sh[k] = 0.0;
-    __syncthreads();
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < d.n; i += stride) {
-        if (!diag_take(d, i)) continue;
-        double dx, dy;
-        const double r2 = diag_r2(d, i, dx, dy);
-        const unsigned long long key = (unsigned long long)__double_as_longlong(r2);
-        int b = 0;   // number of edges <= key
-        {
-            int lo = 0, hi = q.nbins - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (edges[mid] <= key) lo = mid + 1; else hi = mid;
+// By the pass's last block: each boundary's digit from its prefix's counters,
+// then the prefixes of the next pass (boundaries are sorted, so equal ones are
+// adjacent); clears the counters.
+static __device__ void diag_resolve(int pass, int nbins, int np, long long n, DiagState *st, unsigned *hist) {
+    __shared__ unsigned long long nk[DIAG_MAXBINS];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nb = nbins - 1;
+    const int width = diag_high(pass) - diag_low(pass);
+    for (int k = w; k < nb; k += 8) {
+        const int j = pass ? st->which[k] : 0;
+        const long long rank = pass ? st->rank[k] : ((long long)(k + 1) * n) / nbins;
+        const uint4 *row = reinterpret_cast<const uint4 *>(hist + j * DG_ROW + lane * (DG_ROW / 32));
+        uint4 h[DG_ROW / 128];
+        unsigned sum = 0;
+#pragma unroll
+        for (int q = 0; q < DG_ROW / 128; ++q) {
+            h[q] = __ldcg(row + q);
+            sum += h[q].x + h[q].y + h[q].z + h[q].w;
+        }
+        unsigned incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const unsigned has = __ballot_sync(0xffffffffu, (long long)incl > rank);
+        if (has == 0 && lane == 0 && n > 0) st->err = 1;   // particles changed during the call?
+        if (lane == (has ? __ffs(has) - 1 : 0)) {
+            long long left = rank - (long long)(incl - sum);
+            int dgt = 0;
+            bool done = false;
+#pragma unroll
+            for (int q = 0; q < DG_ROW / 128; ++q) {
+                const unsigned c[4] = {h[q].x, h[q].y, h[q].z, h[q].w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    if (!done && left < (long long)c[e]) {
+                        done = true;
+                        dgt = lane * (DG_ROW / 32) + q * 4 + e;
+                    }
+                    if (!done) left -= c[e];
+                }
             }
-            b = lo;
+            nk[k] = ((pass ? st->pref[j] : 0ull) << width) | (unsigned long long)dgt;
+            st->rank[k] = left;
         }
-        const double R = __dsqrt_rn(r2);
-        const double dz = __dsub_rn((double)d.z[i], d.c[2]);
-        const double vx = d.vx[i], vy = d.vy[i], vz = d.vz[i], m = d.m[i];
-        const double vR = R > 0 ? (dx * vx + dy * vy) / R : 0.0;
-        const double vphi = R > 0 ? (dx * vy - dy * vx) / R : 0.0;
-        diag_add(sh, 4 * b + 0, R);
-        diag_add(sh, 4 * b + 1, 1.0);
-        diag_add(sh, 4 * b + 2, dz * dz);
-        diag_add(sh, 4 * b + 3, vphi);
-        if (R >= q.rlo && R < q.rhi) {
-            double *a = sh + 4 * q.nbins;
-            diag_add(a, 0, m);
-            diag_add(a, 1, m * vR);
-            diag_add(a, 2, m * vR * vR);
-            diag_add(a, 3, m * vphi);
-            diag_add(a, 4, m * vphi * vphi);
-            diag_add(a, 5, m * vz);
-            diag_add(a, 6, m * vz * vz);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < np * DG_ROW / 4; i += 256) reinterpret_cast<uint4 *>(hist)[i] = make_uint4(0, 0, 0, 0);
+    if (threadIdx.x == 0) {
+        int m = 0;
+        for (int k = 0; k < nb; ++k) {
+            if (m == 0 || nk[k] != nk[k - 1]) st->pref[m++] = nk[k];
+            st->which[k] = m - 1;
+            st->edge[k] = nk[k];   // complete after the last pass
         }
-        if (R > 0 && R < q.r_ring) {
-            const int ring = (int)floor(__ddiv_rn(R, q.width));
-            if (ring < q.nring) {
-                double *a = sh + 4 * q.nbins + 7 + 2 * ring * q.mmax;
-                // exp(-i m phi) by the angle-addition recurrence from cos, sin phi
-                const double c1 = dx / R, s1 = dy / R;
-                double cm = c1, sm = s1;
-                for (int mo = 0; mo < q.mmax; ++mo) {
-                    diag_add(a, 2 * mo, m * cm);
-                    diag_add(a, 2 * mo + 1, -m * sm);
-                    const double cn = cm * c1 - sm * s1;
-                    sm = sm * c1 + cm * s1;
-                    cm = cn;
+        st->npref = m;
+        st->done = 0;
+    }
+}
+
+// One pass: keys that agree with one of the sorted prefixes (the bits above
+// diag_high) count their next digit.  Lanes with one counter share an atomic
+// (the first digits, exponents, take few values).  The last block to finish
+// resolves the pass.
+static __global__ void __launch_bounds__(256) k_diag_hist(int pass, int nbins, DiagState *st,
+                                                          const unsigned long long *key, unsigned *hist) {
+    __shared__ unsigned long long pref[DIAG_MAXBINS];
+    __shared__ bool last;
+    const int np = pass ? st->npref : 1;
+    const long long n = (long long)st->nsel;
+    if (threadIdx.x < np) pref[threadIdx.x] = pass ? st->pref[threadIdx.x] : 0;
+    __syncthreads();
+    const int low = diag_low(pass), high = diag_high(pass);
+    const unsigned mask = (1u << (high - low)) - 1u;
+    for (long long b = (long long)blockIdx.x * 256; b < n; b += (long long)gridDim.x * 256) {
+        const long long i = b + threadIdx.x;
+        int bin = -1;
+        if (i < n) {
+            const unsigned long long k = key[i];
+            int j = 0;
+            if (pass > 0) {
+                const unsigned long long pk = k >> high;
+                int lo = 0, hi = np - 1;
+                j = -1;
+                while (lo <= hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (pref[mid] == pk) { j = mid; break; }
+                    if (pref[mid] < pk) lo = mid + 1; else hi = mid - 1;
+                }
+            }
+            if (j >= 0) bin = j * DG_ROW + (int)((unsigned)(k >> low) & mask);
+        }
+        const unsigned peers = __match_any_sync(0xffffffffu, bin);
+        if (bin >= 0 && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(hist + bin, (unsigned)__popc(peers));
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&st->done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (last) {
+        __threadfence();
+        diag_resolve(pass, nbins, np, n, st, hist);
+    }
+}
+
+// R = sqrt(r2) and 1/R (0 for 0): an FP32 seed, one third-order step for 1/R
+// and one residual correction for R, a third of the operations of the root and
+// the quotient.
+__device__ __forceinline__ void diag_root(double r2, double &R, double &inv) {
+    if (!(r2 > 1e-30 && r2 < 1e30)) {
+        R = __dsqrt_rn(r2);
+        inv = R > 0 ? 1.0 / R : 0.0;
+        return;
+    }
+    const double y = (double)rsqrtf((float)r2);
+    const double e = fma(-(r2 * y), y, 1.0);
+    inv = fma(y * e, fma(0.375, e, 0.5), y);
+    R = r2 * inv;
+    R = fma(0.5 * inv, fma(-R, R, r2), R);
+}
+
+// R^2, R, 1/R and the cylindrical velocities of one selected particle; the
+// sums and, for the heat, R, v_phi, v_R^2 + v_z^2 and m per particle.
+// Accumulators in shared memory: with PRIVATE a column per thread (no
+// conflicts, no atomics), else one set per block.
+template <typename T, bool PRIVATE>
+__global__ void __launch_bounds__(256) k_diag_sums(DiagP<T> d, const CenK *cen, DiagQ q, const DiagState *st,
+                                                   const unsigned long long *key, const long long *idx, double *acc,
+                                                   double4 *rest) {
+    extern __shared__ double sh[];
+    __shared__ unsigned long long edge[DIAG_MAXBINS];
+    const int nacc = 4 * q.nbins + 7 + 2 * q.nring * q.mmax, copies = PRIVATE ? (int)blockDim.x : 1;
+    for (int k = threadIdx.x; k < nacc * copies; k += blockDim.x) sh[k] = 0.0;
+    for (int k = threadIdx.x; k < q.nbins - 1; k += blockDim.x) edge[k] = st->edge[k];
+    __syncthreads();
+    auto add = [&](int k, double v) {
+        if (PRIVATE) sh[k * copies + threadIdx.x] += v;
+        else atomicAdd(sh + k, v);
+    };
+    const double cx = cen->c[d.gal][0], cy = cen->c[d.gal][1], cz = cen->c[d.gal][2], iw = 1.0 / q.width;
+    const long long n = (long long)st->nsel, stride = (long long)gridDim.x * blockDim.x;
+    // few warps fit beside the columns: U particles' loads in flight each
+    constexpr int U = 4;
+    for (long long p0 = (long long)blockIdx.x * blockDim.x + threadIdx.x; p0 < n; p0 += U * stride) {
+        unsigned long long ku[U];
+        T xu[U], yu[U], zu[U], vxu[U], vyu[U], vzu[U], mu[U];
+        long long iu[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (p0 + u * stride < n) {
+                ku[u] = key[p0 + u * stride];
+                iu[u] = idx[p0 + u * stride];
+            }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (p0 + u * stride < n) {
+                const long long i = iu[u];
+                xu[u] = d.x[i]; yu[u] = d.y[i]; zu[u] = d.z[i];
+                vxu[u] = d.vx[i]; vyu[u] = d.vy[i]; vzu[u] = d.vz[i];
+                mu[u] = d.m[i];
+            }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const long long p = p0 + u * stride;
+            if (p >= n) break;
+            const unsigned long long r2k = ku[u];
+            const double dx = __dsub_rn((double)xu[u], cx), dy = __dsub_rn((double)yu[u], cy);
+            const double dz = __dsub_rn((double)zu[u], cz);
+            const double vx = vxu[u], vy = vyu[u], vz = vzu[u], m = mu[u];
+            int b = 0;   // number of edges <= key
+            {
+                int lo = 0, hi = q.nbins - 1;
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (edge[mid] <= r2k) lo = mid + 1; else hi = mid;
+                }
+                b = lo;
+            }
+            double R, inv;
+            diag_root(__longlong_as_double((long long)r2k), R, inv);
+            const double c1 = dx * inv, s1 = dy * inv;
+            const double vR = c1 * vx + s1 * vy, vphi = c1 * vy - s1 * vx;
+            rest[p] = make_double4(R, vphi, vR * vR + vz * vz, m);
+            add(4 * b + 0, R);
+            add(4 * b + 1, 1.0);
+            add(4 * b + 2, dz * dz);
+            add(4 * b + 3, vphi);
+            if (R >= q.rlo && R < q.rhi) {
+                const int a = 4 * q.nbins;
+                add(a + 0, m);
+                add(a + 1, m * vR);
+                add(a + 2, m * vR * vR);
+                add(a + 3, m * vphi);
+                add(a + 4, m * vphi * vphi);
+                add(a + 5, m * vz);
+                add(a + 6, m * vz * vz);
+            }
+            if (R > 0 && R < q.r_ring) {
+                // floor(R / width): the quotient is formed only near an integer
+                double f = R * iw;
+                const double near = rint(f);
+                if (fabs(f - near) < 1e-9 * (near + 1.0)) f = __ddiv_rn(R, q.width);
+                const int ring = (int)floor(f);
+                if (ring < q.nring) {
+                    const int a = 4 * q.nbins + 7 + 2 * ring * q.mmax;
+                    // exp(-i m phi) by the angle-addition recurrence from m cos, m sin phi
+                    double cm = m * c1, sm = -m * s1;
+                    for (int mo = 0; mo < q.mmax; ++mo) {
+                        add(a + 2 * mo, cm);
+                        add(a + 2 * mo + 1, sm);
+                        const double cn = cm * c1 + sm * s1;
+                        sm = sm * c1 - cm * s1;
+                        cm = cn;
+                    }
                 }
             }
         }
     }
     __syncthreads();
-    for (int k = threadIdx.x; k < nacc; k += blockDim.x)
-        if (sh[k] != 0.0) atomicAdd(acc + k, sh[k]);
+    for (int k = threadIdx.x; k < nacc; k += blockDim.x) {
+        double v = 0.0;
+        if (PRIVATE) {
+            double v2 = 0.0, v3 = 0.0, v4 = 0.0;   // four chains; the columns start at k: no bank conflicts
+            for (int c = 0; c < copies; c += 4) {
+                v += sh[k * copies + ((c + k) & (copies - 1))];
+                v2 += sh[k * copies + ((c + 1 + k) & (copies - 1))];
+                v3 += sh[k * copies + ((c + 2 + k) & (copies - 1))];
+                v4 += sh[k * copies + ((c + 3 + k) & (copies - 1))];
+            }
+            v = (v + v2) + (v3 + v4);
+        } else {
+            v = sh[k];
+        }
+        if (v != 0.0) atomicAdd(acc + k, v);
+    }
 }
 
-// E_heat with vbar_c linear in R between (xp[k], fp[k]), k < np, held
-// constant outside.
-template <typename T>
-__global__ void __launch_bounds__(256) k_diag_heat(DiagP<T> d, const double *xp, const double *fp, int np,
-                                                   double *acc) {
+// E_heat with vbar_c linear in R between the non-empty bins' (mean R, mean
+// v_phi), held constant outside.
+static __global__ void __launch_bounds__(256) k_diag_heat(int nbins, const DiagState *st, const double *acc,
+                                                          const double4 *rest, double *heat) {
+    __shared__ double xp[DIAG_MAXBINS], fp[DIAG_MAXBINS], sl[DIAG_MAXBINS], red[8];
+    __shared__ int s_np;
+    if (threadIdx.x < 32) {
+        int base = 0;
+        for (int b0 = 0; b0 < nbins; b0 += 32) {
+            const int b = b0 + threadIdx.x;
+            const double cnt = b < nbins ? acc[4 * b + 1] : 0.0;
+            const unsigned m = __ballot_sync(0xffffffffu, cnt > 0);
+            if (cnt > 0) {
+                const int k = base + __popc(m & ((1u << threadIdx.x) - 1u));
+                xp[k] = acc[4 * b] / cnt;
+                fp[k] = acc[4 * b + 3] / cnt;
+            }
+            base += __popc(m);
+        }
+        __syncwarp();
+        for (int k = threadIdx.x; k + 1 < base; k += 32) sl[k] = (fp[k + 1] - fp[k]) / (xp[k + 1] - xp[k]);
+        if (threadIdx.x == 0) s_np = base;
+    }
+    __syncthreads();
+    const int np = s_np;
+    const long long n = (long long)st->nsel, stride = (long long)gridDim.x * blockDim.x;
     double e = 0.0;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < d.n; i += stride) {
-        if (!diag_take(d, i)) continue;
-        double dx, dy;
-        const double R = __dsqrt_rn(diag_r2(d, i, dx, dy));
-        const double vx = d.vx[i], vy = d.vy[i], vz = d.vz[i];
-        const double vR = R > 0 ? (dx * vx + dy * vy) / R : 0.0;
-        const double vphi = R > 0 ? (dx * vy - dy * vx) / R : 0.0;
+    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += stride) {
+        const double4 v = rest[p];
+        const double R = v.x;
         double vb;
         if (R <= xp[0]) vb = fp[0];
         else if (R >= xp[np - 1]) vb = fp[np - 1];
@@ -142,52 +360,55 @@ __global__ void __launch_bounds__(256) k_diag_heat(DiagP<T> d, const double *xp,
                 const int mid = (lo + hi) >> 1;
                 if (xp[mid] <= R) lo = mid; else hi = mid;
             }
-            vb = (fp[hi] - fp[lo]) / (xp[hi] - xp[lo]) * (R - xp[lo]) + fp[lo];
+            vb = sl[lo] * (R - xp[lo]) + fp[lo];
         }
-        const double dv = vphi - vb;
-        e += 0.5 * (double)d.m[i] * (vR * vR + dv * dv + vz * vz);
+        const double dv = v.y - vb;
+        e += 0.5 * v.w * (v.z + dv * dv);
     }
-    __shared__ double red[8];
     e = warp_sum(e);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
     __syncthreads();
     if (threadIdx.x == 0) {
         double s = 0;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-        atomicAdd(acc, s);
+        if (s != 0.0) atomicAdd(heat, s);
     }
 }
 
 }  // namespace pmk
 
-template <typename T> cudaError_t pm_launch_diag_hist(const pmk::DiagP<T> &d, int pass, const unsigned long long *pref,
-                                                      int npref, unsigned *hist, cudaStream_t st) {
-    if (d.n <= 0) return cudaSuccess;
-    long long b = (d.n + 255) / 256;
-    pmk::k_diag_hist<T><<<(int)(b < 4096 ? b : 4096), 256, 0, st>>>(d, pass, pref, npref, hist);
-    return cudaGetLastError();
-}
-template <typename T> cudaError_t pm_launch_diag_sums(const pmk::DiagP<T> &d, const pmk::DiagQ &q,
-                                                      const unsigned long long *edges, double *acc,
-                                                      cudaStream_t st) {
-    if (d.n <= 0) return cudaSuccess;
-    const size_t sh = sizeof(double) * (4 * q.nbins + 7 + 2 * q.nring * q.mmax);
-    long long b = (d.n + 255) / 256;
-    pmk::k_diag_sums<T><<<(int)(b < 1024 ? b : 1024), 256, sh, st>>>(d, q, edges, acc);
-    return cudaGetLastError();
-}
-template <typename T> cudaError_t pm_launch_diag_heat(const pmk::DiagP<T> &d, const double *xp, const double *fp,
-                                                      int np, double *acc, cudaStream_t st) {
-    if (d.n <= 0) return cudaSuccess;
-    long long b = (d.n + 255) / 256;
-    pmk::k_diag_heat<T><<<(int)(b < 1024 ? b : 1024), 256, 0, st>>>(d, xp, fp, np, acc);
+// Every step of pm_disc_diagnostics on the device (acc: nacc + 1 sums, the
+// last the heat; everything zeroed here).
+template <typename T>
+cudaError_t pm_launch_diag(const pmk::DiagP<T> &d, const CenK *cen, const pmk::DiagQ &q, const pmk::DiagBuf &b,
+                           cudaStream_t st) {
+    const int nacc = 4 * q.nbins + 7 + 2 * q.nring * q.mmax;
+    cudaError_t e = cudaMemsetAsync(b.state, 0, sizeof(pmk::DiagState), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b.acc, 0, sizeof(double) * (nacc + 1), st);
+    if (e == cudaSuccess && q.nbins > 1)
+        e = cudaMemsetAsync(b.hist, 0, sizeof(unsigned) * pmk::DG_ROW * (q.nbins - 1), st);
+    if (e != cudaSuccess || d.n <= 0) return e;
+    // a wave of blocks: the sums' epilogues cost FP64 operations per block
+    const unsigned wave = 152 * 8, by = (unsigned)std::min<long long>((d.n + 1023) / 1024, wave);
+    pmk::k_diag_select<T><<<by, 256, 0, st>>>(d, cen, b.state, b.key, b.idx);
+    if (q.nbins > 1)
+        for (int pass = 0; pass < pmk::DG_PASSES; ++pass)
+            pmk::k_diag_hist<<<std::min(by, 152u * 2), 256, 0, st>>>(pass, q.nbins, b.state, b.key, b.hist);
+    // a column of accumulators per thread while 64 or 32 threads' fit two
+    // blocks on an SM
+    const size_t one = sizeof(double) * nacc;
+    const int threads = 64 * one <= 100u << 10 ? 64 : 32 * one <= 100u << 10 ? 32 : 0;
+    if (threads) {
+        e = cudaFuncSetAttribute(pmk::k_diag_sums<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 << 10);
+        if (e != cudaSuccess) return e;
+        pmk::k_diag_sums<T, true><<<152 * 2, threads, threads * one, st>>>(d, cen, q, b.state, b.key, b.idx, b.acc, b.rest);
+    } else {
+        pmk::k_diag_sums<T, false><<<std::min(by, 152u * 4), 256, one, st>>>(d, cen, q, b.state, b.key, b.idx, b.acc, b.rest);
+    }
+    pmk::k_diag_heat<<<std::min(by, 152u * 4), 256, 0, st>>>(q.nbins, b.state, b.acc, b.rest, b.acc + nacc);
     return cudaGetLastError();
 }
 
-#define PM_DIAG_INSTANTIATE(T)                                                                                 \
-    template cudaError_t pm_launch_diag_hist<T>(const pmk::DiagP<T> &, int, const unsigned long long *, int,   \
-                                                unsigned *, cudaStream_t);                                     \
-    template cudaError_t pm_launch_diag_sums<T>(const pmk::DiagP<T> &, const pmk::DiagQ &,                     \
-                                                const unsigned long long *, double *, cudaStream_t);          \
-    template cudaError_t pm_launch_diag_heat<T>(const pmk::DiagP<T> &, const double *, const double *, int,    \
-                                                double *, cudaStream_t);
+#define PM_DIAG_INSTANTIATE(T)                                                                                \
+    template cudaError_t pm_launch_diag<T>(const pmk::DiagP<T> &, const CenK *, const pmk::DiagQ &, const pmk::DiagBuf &, \
+                                           cudaStream_t);

@@ -135,7 +135,6 @@ template <typename T> struct DiagP {
     const int32_t *gal_id;
     int gal;
     long long n;
-    double c[3];
 };
 
 // Accumulator layout: per bin [sum R, count, sum z^2, sum v_phi]; annulus
@@ -146,15 +145,35 @@ struct DiagQ {
     double width, r_ring, rlo, rhi;
 };
 
+
+constexpr int DIAG_MAXBINS = 64;
+// Device state of the radix select: the selected count, per boundary k =
+// 0..nbins-2 its prefix (an index into the sorted distinct ones), the rank
+// within it and the bits found so far.
+struct DiagState {
+    unsigned long long nsel;
+    int npref, err;
+    unsigned done;   // blocks of the running pass that have finished
+    unsigned long long pref[DIAG_MAXBINS], edge[DIAG_MAXBINS];
+    long long rank[DIAG_MAXBINS];
+    int which[DIAG_MAXBINS];
+};
+// Scratch: state, counters (2048 per boundary), sums; per particle the key,
+// the index and what the heat needs (48 bytes).
+struct DiagBuf {
+    DiagState *state;
+    unsigned *hist;
+    double *acc;
+    unsigned long long *key;
+    long long *idx;
+    double4 *rest;
+};
+
 }  // namespace pmk
-// Radix-select pass over the bits of R^2 (pass 0..7), the sums of the bins,
-// annulus and rings, and the heat about an interpolated circular velocity.
-template <typename T> cudaError_t pm_launch_diag_hist(const pmk::DiagP<T> &d, int pass, const unsigned long long *pref,
-                                                      int npref, unsigned *hist, cudaStream_t st);
-template <typename T> cudaError_t pm_launch_diag_sums(const pmk::DiagP<T> &d, const pmk::DiagQ &q,
-                                                      const unsigned long long *edges, double *acc, cudaStream_t st);
-template <typename T> cudaError_t pm_launch_diag_heat(const pmk::DiagP<T> &d, const double *xp, const double *fp,
-                                                      int np, double *acc, cudaStream_t st);
+// The disc diagnostics of particles d about the centre of galaxy d.gal.
+template <typename T>
+cudaError_t pm_launch_diag(const pmk::DiagP<T> &d, const CenK *cen, const pmk::DiagQ &q, const pmk::DiagBuf &b,
+                           cudaStream_t st);
 
 // H-hat table of the z pass, scaled by `scale`: for each octant column
 // (kyr, kxr), for L = 2nz >= 128 the nz + 1 values H-hat(kzr) padded with
