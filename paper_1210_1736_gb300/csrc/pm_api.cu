@@ -198,6 +198,9 @@ struct pm_ctx {
     long long sort_cap = 0;
     unsigned *s_count = nullptr, *s_key = nullptr, *s_rank = nullptr, *s_bsum = nullptr;
     void *s_arr[9] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    // processing order of the CIC kernels (a permutation of 0..ord_n - 1)
+    unsigned *o_key = nullptr, *o_rank = nullptr, *o_ord = nullptr;
+    long long ord_cap = 0, ord_n = 0;
     size_t bytes = 0;
     std::vector<void *> allocs;
     bool any_recentre = false;
@@ -748,16 +751,38 @@ template <typename T> int step_timed_impl(pm_ctx *c, const pm_particles *p, doub
 }
 
 // ---- CIC variant (differentiable runs) -------------------------------------
+// The particles' spatial order at their current positions, for the CIC kernels
+// (unsorted, their atomics and gathers touch a cache line each).  The calls after a deposit run in the deposit's order: results
+// depend on no order, so for other particles of the same number it is only a
+// worse one.
+constexpr long long CIC_ORDER_MIN = 1LL << 16, CIC_ORDER_MAX = 1LL << 32;
+template <typename T> int cic_order(pm_ctx *c, const pm_particles *p) {
+    c->ord_n = 0;
+    if (p->n < CIC_ORDER_MIN || p->n >= CIC_ORDER_MAX) return PM_OK;
+    if (p->n > c->ord_cap) {
+        PM_TRY(dev_alloc(c, (void **)&c->o_key, (size_t)p->n * 4));
+        PM_TRY(dev_alloc(c, (void **)&c->o_rank, (size_t)p->n * 4));
+        PM_TRY(dev_alloc(c, (void **)&c->o_ord, (size_t)p->n * 4));
+        c->ord_cap = p->n;
+    }
+    PM_CK(pm_launch_order<T>(part_k<T>(p), c->hs, c->d_cen, c->sortk, c->s_count, c->o_key, c->o_rank, c->s_bsum,
+                             c->o_ord, c->user));
+    c->ord_n = p->n;
+    return PM_OK;
+}
+const unsigned *cic_ord(const pm_ctx *c, const pm_particles *p) { return c->ord_n == p->n ? c->o_ord : nullptr; }
+
 template <typename T> int cic_deposit_impl(pm_ctx *c, const pm_particles *p) {
+    PM_TRY(cic_order<T>(c, p));
     PM_CK(cudaMemsetAsync(c->rho_all, 0, c->rho_bytes, c->user));
-    PM_CK(pm_launch_cic_deposit<T>(part_k<T>(p), c->hs, c->d_cen, c->user));
+    PM_CK(pm_launch_cic_deposit<T>(part_k<T>(p), c->hs, c->d_cen, cic_ord(c, p), c->user));
     return PM_OK;
 }
 
 template <typename T> int cic_field_impl(pm_ctx *c, int mode, const pm_particles *p, double dtk, double dtd,
                                          void *ox, void *oy, void *oz) {
     PM_CK(pm_launch_cic_field<T>(mode, part_k<T>(p), c->hs, c->d_cen, dtk, dtd, (T *)ox, (T *)oy, (T *)oz, nullptr,
-                                 nullptr, nullptr, 0.0, c->user));
+                                 nullptr, nullptr, 0.0, cic_ord(c, p), c->user));
     return PM_OK;
 }
 
@@ -777,9 +802,11 @@ template <typename T> int cic_vjp_impl(pm_ctx *c, const pm_particles *p, const v
                                        const void *uz, void *gx, void *gy, void *gz, void *gm) {
     const PartK<T> pk = part_k<T>(p);
     const T *u[3] = {(const T *)ux, (const T *)uy, (const T *)uz};
+    if (c->ord_n != p->n) PM_TRY(cic_order<T>(c, p));
+    const unsigned *ord = cic_ord(c, p);
     // direct term, with the forward potentials still in place
     PM_CK(pm_launch_cic_field<T>(2, pk, c->hs, c->d_cen, 0.0, 0.0, (T *)gx, (T *)gy, (T *)gz, u[0], u[1], u[2], 0.0,
-                                 c->user));
+                                 ord, c->user));
     // fixed-point scale of the adjoint densities: |cell sum| <= n max|u| bound
     PM_CK(cudaMemsetAsync(c->d_cnt, 0, sizeof(unsigned long long), c->user));
     PM_CK(pm_launch_cic_umax<T>(pk, u[0], u[1], u[2], (unsigned *)c->d_cnt, c->user));
@@ -795,7 +822,11 @@ template <typename T> int cic_vjp_impl(pm_ctx *c, const pm_particles *p, const v
     sa = std::min(120, std::max(-100, sa));
     PM_CK(cudaMemsetAsync(c->rho_all, 0, c->rho_bytes, c->user));
     PM_CK(pm_launch_cic_field<T>(3, pk, c->hs, c->d_cen, 0.0, 0.0, nullptr, nullptr, nullptr, u[0], u[1], u[2],
-                                 std::ldexp(1.0, sa), c->user));
+                                 std::ldexp(1.0, sa), ord, c->user));
+    for (int gi = 0; gi < c->sys.ngal; ++gi)   // sums and differences of the regions' spreads
+        for (int k = 1; k < PM_SETS; k += 2)
+            if (c->set_geo[gi][k] >= 0)
+                PM_CK(pm_launch_cic_slots(c->rho[gi][k], c->rho[gi][k + 1], c->geos[c->set_geo[gi][k]].A, c->user));
     PM_TRY(enqueue_solve<T>(c, c->user, nullptr, sa));
     PM_CK(pm_launch_cic_gather<T>(pk, c->hs, c->d_cen, (T *)gx, (T *)gy, (T *)gz, (T *)gm, c->user));
     return check_device_error(c);

@@ -25,11 +25,26 @@
 // Pair slots are loaded so that the solver's stored outputs are the lam_k
 // the mass sets need: medium a = psi_2 - psi_3, b = psi_3 (outputs
 // lam_2 = a + b, lam_3 = b); coarse a = psi_4 - psi_5, b = psi_5.
+//
+// Bound by the atomics (32 per point and level in the adjoint spread, 80 G/s
+// for unsorted points).  So the particles run in spatial order (an index
+// computed per deposit, pm_launch_order, 55 us for 1M), runs of particles in
+// one cell share their atomics, and each point spreads once per level.  1M
+// points of two galaxies: deposit 333 -> 129 us, spread 1600 -> 558, direct term
+// 160 -> 104.  From 2^16 particles; below, the launches of the order cost more
+// than it saves.
 #pragma once
+
+#include <algorithm>
 
 #include "pm_particle.cuh"
 
 namespace pmk {
+
+// Threads per block of the particle kernels of this file: small blocks, so that
+// a few ten thousand particles spread evenly over the SMs (FP64 runs are bound
+// by the SMs' FP64 pipes).
+constexpr int CIC_THREADS = 64;
 
 template <typename T> struct Cic {
     size_t base;          // offset of the lower cell (a0, b0, c0)
@@ -143,35 +158,75 @@ __device__ __forceinline__ void cic_gather(const GeomK &g, const void *Fv, const
             }
 }
 
-__device__ __forceinline__ long long cic_q(float v, float s) { return __float2ll_rn(v * s); }
-__device__ __forceinline__ long long cic_q(double v, double s) { return __double2ll_rn(v * s); }
+// Rounds a share, already scaled by the (power of two) fixed-point factor.
+// (Integer operations in place of the conversion, which runs on the FP64 pipe,
+// measured slower: adjoint spread of 1M points 558 -> 582 us.)
+__device__ __forceinline__ long long cic_q(float v) { return __float2ll_rn(v); }
+__device__ __forceinline__ long long cic_q(double v) { return __double2ll_rn(v); }
 
-// Forward deposit: m W into the 8 cells (fixed point, scale qs = 2^s).
+// Adjacent active lanes with one lower cell (the particles run in the order of
+// pm_launch_order) form a run; with runs of two or more on average every cell's
+// shares are summed over the run by a segmented scan (64-bit adds, exact) and
+// its last lane issues the atomic.  Every lane of the warp must call start
+// and add.
+struct CicRuns {
+    bool active, sum, tail;
+    int behind, longest;   // lanes since the run's first; the warp's largest
+    __device__ __forceinline__ void start(const unsigned long long *cell, bool act) {
+        const unsigned FULL = 0xffffffffu;
+        const int lane = (int)(threadIdx.x & 31);
+        active = act;
+        const unsigned long long key = act ? (unsigned long long)cell : 0ull;   // no cell lives at address 0
+        const unsigned long long prev = __shfl_up_sync(FULL, key, 1);
+        const unsigned heads = __ballot_sync(FULL, act && (lane == 0 || prev != key)), on = __ballot_sync(FULL, act);
+        const unsigned brk = heads | ~on;
+        const unsigned upto = lane == 31 ? FULL : ((2u << lane) - 1u);
+        behind = act ? lane - (31 - __clz(brk & upto)) : 0;
+        tail = act && (lane == 31 || ((brk >> (lane + 1)) & 1u));
+        sum = 2 * __popc(heads) <= __popc(on);
+        longest = sum ? (int)__reduce_max_sync(FULL, (unsigned)behind) : 0;
+    }
+    __device__ __forceinline__ void add(unsigned long long *addr, long long q) const {
+        unsigned long long v = (unsigned long long)q;
+        if (sum) {
+            for (int d = 1; d <= longest; d <<= 1) {
+                const unsigned long long u = __shfl_up_sync(0xffffffffu, v, d);
+                if (behind >= d) v += u;
+            }
+            if (tail) atomicAdd(addr, v);
+        } else if (active) {
+            atomicAdd(addr, v);
+        }
+    }
+};
+
+// Forward deposit: m W into the 8 cells (fixed point; m carries the scale).
 template <typename T>
-__device__ __forceinline__ void cic_spread_mass(const GeomK &g, unsigned long long *rho, const Cic<T> &c, T m, T qs) {
-    const long long sy = g.nx, sz = (long long)g.nx * g.ny;
+__device__ __forceinline__ void cic_spread_mass(const GeomK &g, unsigned long long *rho, const Cic<T> &c, T m,
+                                                bool active) {
+    const int sy = g.nx, sz = g.nx * g.ny;
     unsigned long long *b = rho + c.base;
+    CicRuns run;
+    run.start(b, active);
 #pragma unroll
     for (int dk = 0; dk < 2; ++dk)
 #pragma unroll
         for (int dj = 0; dj < 2; ++dj)
 #pragma unroll
-            for (int di = 0; di < 2; ++di) {
-                const T W = c.w[0][di] * c.w[1][dj] * c.w[2][dk];
-                atomicAdd(b + di + dj * sy + dk * sz, (unsigned long long)cic_q(m * W, qs));
-            }
+            for (int di = 0; di < 2; ++di)
+                run.add(b + di + dj * sy + dk * sz, active ? cic_q(m * (c.w[0][di] * c.w[1][dj] * c.w[2][dk])) : 0);
 }
 
-// Adjoint spread: sign * sum_d D_d^T (W u_d) into the 32 cells it touches
-// (fixed point, scale qs).  h[d] = u_d / (2 l_d).
+// Adjoint spread: sum_d D_d^T (W u_d) into the 32 cells it touches (fixed
+// point).  h[d] = u_d / (2 l_d) times the scale.
 template <typename T>
 __device__ __forceinline__ void cic_spread_adj(const GeomK &g, unsigned long long *rho, const Cic<T> &c, const T *h,
-                                               T qs) {
-    const long long sy = g.nx, sz = (long long)g.nx * g.ny;
+                                               bool active) {
+    const int sy = g.nx, sz = g.nx * g.ny;
     unsigned long long *b = rho + c.base;
-    auto add = [&](int di, int dj, int dk, T v) {
-        atomicAdd(b + di + dj * sy + dk * sz, (unsigned long long)cic_q(v, qs));
-    };
+    CicRuns run;
+    run.start(b, active);
+    auto add = [&](int di, int dj, int dk, T v) { run.add(b + di + dj * sy + dk * sz, active ? cic_q(v) : 0); };
     const T(&w)[3][2] = c.w;
 #pragma unroll
     for (int dk = 0; dk < 2; ++dk)
@@ -224,48 +279,63 @@ __device__ __forceinline__ Rel<T> rel_sys(const SysK &s, T x, T y, T z) {
     return r;
 }
 
+// Particle j of the processing order (ord null: as stored).
+__device__ __forceinline__ long long cic_at(const unsigned *ord, long long j) { return ord ? (long long)__ldg(ord + j) : j; }
+
 // Forward CIC deposit with the lost test and mass sets of the NGP deposit.
+// The loop is warp-uniform (the spreads are warp collectives).
 template <typename T>
-__global__ void __launch_bounds__(256) k_cic_deposit(PartK<T> p, const __grid_constant__ SysK s, const CenK *cen) {
+__global__ void __launch_bounds__(CIC_THREADS) k_cic_deposit(PartK<T> p, const __grid_constant__ SysK s,
+                                                             const CenK *cen, const unsigned *ord) {
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < p.n; i += stride) {
-        const uint32_t f = p.flags[i];
-        if (f & PM_FLAG_LOST) continue;
-        const T x = p.x[i], y = p.y[i], z = p.z[i];
-        const int g = p.gal[i];
-        const Rel<T> rs = rel_sys(s, x, y, z);
-        bool lost = !(pm_r2(rs.sx, rs.sy, rs.sz) < s.rsys2);
-        if (g < 0 || g >= s.ngal) lost = true;
-        Cell cc;
-        cc.i = cc.j = cc.k = 0; cc.ok = false;
-        for (int h = 0; h < s.ngal; ++h) {
-            const Cell ch = pm_cells(s.gal[h].coarse, rs.sx, rs.sy, rs.sz);
-            lost = lost || !ch.ok;
-            if (h == g) cc = ch;
+    for (long long b = (long long)blockIdx.x * blockDim.x; b < p.n; b += stride) {
+        const long long j = b + threadIdx.x;
+        const long long i = j < p.n ? cic_at(ord, j) : 0;
+        const uint32_t f = j < p.n ? p.flags[i] : PM_FLAG_LOST;
+        bool live = !(f & PM_FLAG_LOST);
+        Cic<T> kc = {}, km = {}, kf = {};
+        int reg = REG_OUTER, g = 0;
+        T m = 0;
+        if (live) {
+            const T x = p.x[i], y = p.y[i], z = p.z[i];
+            g = p.gal[i];
+            m = p.m[i] * pick<T>(s.mscale, s.mscale_f);   // a power of two: exact
+            const Rel<T> rs = rel_sys(s, x, y, z);
+            bool lost = !(pm_r2(rs.sx, rs.sy, rs.sz) < s.rsys2);
+            if (g < 0 || g >= s.ngal) lost = true;
+            Cell cc;
+            cc.i = cc.j = cc.k = 0; cc.ok = false;
+            for (int h = 0; h < s.ngal; ++h) {
+                const Cell ch = pm_cells(s.gal[h].coarse, rs.sx, rs.sy, rs.sz);
+                lost = lost || !ch.ok;
+                if (h == g) cc = ch;
+            }
+            if (lost) {
+                p.flags[i] = f | PM_FLAG_LOST;
+                live = false;
+                g = 0;
+            } else {
+                const GalK &G = s.gal[g];
+                const Cen1 ce = load_cen(cen, g);
+                Cell cf, cm;
+                reg = pm_region(G, pm_canon(x, ce.c[0], ce.hi[0], ce.lo[0]), pm_canon(y, ce.c[1], ce.hi[1], ce.lo[1]),
+                                pm_canon(z, ce.c[2], ce.hi[2], ce.lo[2]), cf, cm);
+                kc = cic_cell<T>(G.coarse, cc, rs.rsx, rs.rsy, rs.rsz);
+                if (reg != REG_OUTER) {
+                    const T rx = rel_off(x, ce.c[0], ce.hi[0], ce.lo[0]);
+                    const T ry = rel_off(y, ce.c[1], ce.hi[1], ce.lo[1]);
+                    const T rz = rel_off(z, ce.c[2], ce.hi[2], ce.lo[2]);
+                    km = cic_cell<T>(G.med, cm, rx, ry, rz);
+                    if (reg == REG_CORE) kf = cic_cell<T>(G.fine, cf, rx, ry, rz);
+                }
+            }
         }
-        if (lost) { p.flags[i] = f | PM_FLAG_LOST; continue; }
         const GalK &G = s.gal[g];
-        const Cen1 ce = load_cen(cen, g);
-        Cell cf, cm;
-        const int reg = pm_region(G, pm_canon(x, ce.c[0], ce.hi[0], ce.lo[0]), pm_canon(y, ce.c[1], ce.hi[1], ce.lo[1]),
-                                  pm_canon(z, ce.c[2], ce.hi[2], ce.lo[2]), cf, cm);
-        const T m = p.m[i], qs = pick<T>(s.mscale, s.mscale_f);
-        const Cic<T> kc = cic_cell<T>(G.coarse, cc, rs.rsx, rs.rsy, rs.rsz);
-        if (reg == REG_OUTER) {
-            cic_spread_mass<T>(G.coarse, G.rho[4], kc, m, qs);
-            continue;
-        }
-        const T rx = rel_off(x, ce.c[0], ce.hi[0], ce.lo[0]);
-        const T ry = rel_off(y, ce.c[1], ce.hi[1], ce.lo[1]);
-        const T rz = rel_off(z, ce.c[2], ce.hi[2], ce.lo[2]);
-        cic_spread_mass<T>(G.coarse, G.rho[3], kc, m, qs);
-        const Cic<T> km = cic_cell<T>(G.med, cm, rx, ry, rz);
-        if (reg == REG_CORE) {
-            cic_spread_mass<T>(G.med, G.rho[1], km, m, qs);
-            cic_spread_mass<T>(G.fine, G.rho[0], cic_cell<T>(G.fine, cf, rx, ry, rz), m, qs);
-        } else {
-            cic_spread_mass<T>(G.med, G.rho[2], km, m, qs);
-        }
+        cic_spread_mass<T>(G.coarse, G.rho[reg == REG_OUTER ? 4 : 3], kc, m, live);
+        if (!__any_sync(0xffffffffu, live && reg != REG_OUTER)) continue;
+        cic_spread_mass<T>(G.med, G.rho[reg == REG_CORE ? 1 : 2], km, m, live && reg != REG_OUTER);
+        if (__any_sync(0xffffffffu, live && reg == REG_CORE))
+            cic_spread_mass<T>(G.fine, G.rho[0], kf, m, live && reg == REG_CORE);
     }
 }
 
@@ -274,19 +344,26 @@ __global__ void __launch_bounds__(256) k_cic_deposit(PartK<T> p, const __grid_co
 //   MODE 2: g += u^T (d a / d x_i) direct term (positions' own weights)
 //   MODE 3: adjoint spread of u into the pair slots (scale qs)
 template <typename T, int MODE>
-__global__ void __launch_bounds__(256) k_cic_field(PartK<T> p, const __grid_constant__ SysK s, const CenK *cen,
-                                                   T dtk, T dtd, T *ox, T *oy, T *oz, const T *ux, const T *uy,
-                                                   const T *uz, T qs) {
+__global__ void __launch_bounds__(CIC_THREADS) k_cic_field(PartK<T> p, const __grid_constant__ SysK s, const CenK *cen,
+                                                           T dtk, T dtd, T *ox, T *oy, T *oz, const T *ux, const T *uy,
+                                                           const T *uz, T qs, const unsigned *ord) {
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < p.n; i += stride) {
-        if (p.flags[i] & PM_FLAG_LOST) {
+    for (long long b = (long long)blockIdx.x * blockDim.x; b < p.n; b += stride) {   // warp-uniform (MODE 3)
+        const long long j = b + threadIdx.x;
+        if (MODE != 3 && j >= p.n) continue;
+        const long long i = j < p.n ? cic_at(ord, j) : 0;
+        const bool live = j < p.n && !(p.flags[i] & PM_FLAG_LOST);
+        if (MODE != 3 && !live) {
             if (MODE == 1) { ox[i] = 0; oy[i] = 0; oz[i] = 0; }
             continue;
         }
-        const T xT = p.x[i], yT = p.y[i], zT = p.z[i];
-        const Rel<T> rs = rel_sys(s, xT, yT, zT);
+        T xT = 0, yT = 0, zT = 0;
         T u[3] = {0, 0, 0};
-        if (MODE >= 2) { u[0] = ux[i]; u[1] = uy[i]; u[2] = uz[i]; }
+        if (live) {
+            xT = p.x[i]; yT = p.y[i]; zT = p.z[i];
+            if (MODE >= 2) { u[0] = ux[i]; u[1] = uy[i]; u[2] = uz[i]; }
+        }
+        const Rel<T> rs = rel_sys(s, xT, yT, zT);
         T out[3] = {0, 0, 0};
         for (int h = 0; h < s.ngal; ++h) {
             const GalK &G = s.gal[h];
@@ -296,10 +373,11 @@ __global__ void __launch_bounds__(256) k_cic_field(PartK<T> p, const __grid_cons
                                       pm_canon(yT, ce.c[1], ce.hi[1], ce.lo[1]),
                                       pm_canon(zT, ce.c[2], ce.hi[2], ce.lo[2]), cf, cm);
             const Cell cc = pm_cells(G.coarse, rs.sx, rs.sy, rs.sz);
-            if (!cc.ok) continue;  // only after positions changed without a deposit
+            const bool on = live && cc.ok;   // not ok only after positions changed without a deposit
+            if (MODE != 3 && !on) continue;
             const Cic<T> kc = cic_cell<T>(G.coarse, cc, rs.rsx, rs.rsy, rs.rsz);
-            Cic<T> km, kf;
-            if (reg != REG_OUTER) {
+            Cic<T> km = {}, kf = {};
+            if (on && reg != REG_OUTER) {
                 const T rx = rel_off(xT, ce.c[0], ce.hi[0], ce.lo[0]);
                 const T ry = rel_off(yT, ce.c[1], ce.hi[1], ce.lo[1]);
                 const T rz = rel_off(zT, ce.c[2], ce.hi[2], ce.lo[2]);
@@ -307,19 +385,17 @@ __global__ void __launch_bounds__(256) k_cic_field(PartK<T> p, const __grid_cons
                 if (reg == REG_CORE) kf = cic_cell<T>(G.fine, cf, rx, ry, rz);
             }
             if (MODE == 3) {
-                T hp[3] = {u[0] * pick<T>(G.coarse.c_gx, G.coarse.fc_gx), u[1] * pick<T>(G.coarse.c_gx, G.coarse.fc_gx), u[2] * pick<T>(G.coarse.c_gz, G.coarse.fc_gz)};
-                T hm[3] = {-hp[0], -hp[1], -hp[2]};
-                cic_spread_adj<T>(G.coarse, G.rho[4], kc, hp, qs);         // psi_5 (all points)
-                if (reg == REG_OUTER) continue;
-                cic_spread_adj<T>(G.coarse, G.rho[3], kc, hm, qs);         // psi_4 - psi_5
-                T mp[3] = {u[0] * pick<T>(G.med.c_gx, G.med.fc_gx), u[1] * pick<T>(G.med.c_gx, G.med.fc_gx), u[2] * pick<T>(G.med.c_gz, G.med.fc_gz)};
-                cic_spread_adj<T>(G.med, G.rho[2], km, mp, qs);            // psi_3 (core, shell)
-                if (reg == REG_CORE) {
-                    T mm[3] = {-mp[0], -mp[1], -mp[2]};
-                    cic_spread_adj<T>(G.med, G.rho[1], km, mm, qs);        // psi_2 - psi_3
-                    T fp[3] = {u[0] * pick<T>(G.fine.c_gx, G.fine.fc_gx), u[1] * pick<T>(G.fine.c_gx, G.fine.fc_gx), u[2] * pick<T>(G.fine.c_gz, G.fine.fc_gz)};
-                    cic_spread_adj<T>(G.fine, G.rho[0], kf, fp, qs);       // psi_1
-                }
+                // each point once per level, into the slot of its region:
+                // k_cic_slots forms the sums and differences the solve takes
+                const T v[3] = {u[0] * qs, u[1] * qs, u[2] * qs};   // qs a power of two: exact
+                T c3[3] = {v[0] * pick<T>(G.coarse.c_gx, G.coarse.fc_gx), v[1] * pick<T>(G.coarse.c_gx, G.coarse.fc_gx), v[2] * pick<T>(G.coarse.c_gz, G.coarse.fc_gz)};
+                cic_spread_adj<T>(G.coarse, G.rho[reg == REG_OUTER ? 4 : 3], kc, c3, on);
+                if (!__any_sync(0xffffffffu, on && reg != REG_OUTER)) continue;
+                T m3[3] = {v[0] * pick<T>(G.med.c_gx, G.med.fc_gx), v[1] * pick<T>(G.med.c_gx, G.med.fc_gx), v[2] * pick<T>(G.med.c_gz, G.med.fc_gz)};
+                cic_spread_adj<T>(G.med, G.rho[reg == REG_CORE ? 1 : 2], km, m3, on && reg != REG_OUTER);
+                if (!__any_sync(0xffffffffu, on && reg == REG_CORE)) continue;
+                T f3[3] = {v[0] * pick<T>(G.fine.c_gx, G.fine.fc_gx), v[1] * pick<T>(G.fine.c_gx, G.fine.fc_gx), v[2] * pick<T>(G.fine.c_gz, G.fine.fc_gz)};
+                cic_spread_adj<T>(G.fine, G.rho[0], kf, f3, on && reg == REG_CORE);   // psi_1
                 continue;
             }
             constexpr bool VJP = (MODE == 2);
@@ -341,13 +417,30 @@ __global__ void __launch_bounds__(256) k_cic_field(PartK<T> p, const __grid_cons
     }
 }
 
+// The pair slots of the adjoint solve from the regions' spreads: medium
+// a = psi_2 - psi_3 (minus the core's), b = psi_3 (core and shell); coarse
+// a = psi_4 - psi_5 (minus the inner points'), b = psi_5 (all points).
+static __global__ void __launch_bounds__(256) k_cic_slots(long long *a, long long *b, long long n) {
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n / 2; i += stride) {   // n is even
+        longlong2 *pa = reinterpret_cast<longlong2 *>(a) + i, *pb = reinterpret_cast<longlong2 *>(b) + i;
+        longlong2 va = *pa, vb = *pb;
+        vb.x += va.x; vb.y += va.y;
+        va.x = -va.x; va.y = -va.y;
+        *pa = va;
+        *pb = vb;
+    }
+}
+
 // Field term of the adjoint for each particle's own mass sets: the adjoint
 // solve left lam_1 in the fine sum slot, lam_2 (medium sum), lam_3 (medium
 // b), lam_4 (coarse sum) and lam_5 (coarse b, or the sum without medium).
 template <typename T>
-__global__ void __launch_bounds__(256) k_cic_gather(PartK<T> p, const __grid_constant__ SysK s, const CenK *cen,
-                                                    T *gx, T *gy, T *gz, T *gm) {
+__global__ void __launch_bounds__(CIC_THREADS) k_cic_gather(PartK<T> p, const __grid_constant__ SysK s, const CenK *cen,
+                                                            T *gx, T *gy, T *gz, T *gm) {
     const long long stride = (long long)gridDim.x * blockDim.x;
+    // in stored order: the few gathers gain less than the indirect sums cost
+    // (1M points: 54 us, in spatial order 98)
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < p.n; i += stride) {
         if (p.flags[i] & PM_FLAG_LOST) continue;
         const int g = p.gal[i];
@@ -408,32 +501,40 @@ __global__ void __launch_bounds__(256) k_cic_umax(PartK<T> p, const T *ux, const
 // Host launchers (instantiated for float and double in pm_cic.cu)
 // ---------------------------------------------------------------------------
 namespace pmk_cic_host {
-inline int grid_for(long long n) {
-    long long b = (n + 255) / 256;
-    return (int)(b < (1LL << 16) ? (b > 0 ? b : 1) : (1LL << 16));
+inline int grid_for(long long n, int threads = pmk::CIC_THREADS) {
+    long long b = (n + threads - 1) / threads;
+    return (int)(b < (1LL << 18) ? (b > 0 ? b : 1) : (1LL << 18));
 }
 }  // namespace pmk_cic_host
 
 template <typename T>
-cudaError_t pm_launch_cic_deposit(const PartK<T> &p, const SysK &sk, const CenK *cen, cudaStream_t st) {
+cudaError_t pm_launch_cic_deposit(const PartK<T> &p, const SysK &sk, const CenK *cen, const unsigned *ord,
+                                  cudaStream_t st) {
     if (p.n <= 0) return cudaSuccess;
-    pmk::k_cic_deposit<T><<<pmk_cic_host::grid_for(p.n), 256, 0, st>>>(p, sk, cen);
+    pmk::k_cic_deposit<T><<<pmk_cic_host::grid_for(p.n), pmk::CIC_THREADS, 0, st>>>(p, sk, cen, ord);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t pm_launch_cic_field(int mode, const PartK<T> &p, const SysK &sk, const CenK *cen, double dtk, double dtd,
                                 T *ox, T *oy, T *oz, const T *ux, const T *uy, const T *uz, double qs,
-                                cudaStream_t st) {
+                                const unsigned *ord, cudaStream_t st) {
     if (p.n <= 0) return cudaSuccess;
     const int g = pmk_cic_host::grid_for(p.n);
+#define PM_CF(M) pmk::k_cic_field<T, M><<<g, pmk::CIC_THREADS, 0, st>>>(p, sk, cen, (T)dtk, (T)dtd, ox, oy, oz, ux, uy, uz, (T)qs, ord)
     switch (mode) {
-        case 0: pmk::k_cic_field<T, 0><<<g, 256, 0, st>>>(p, sk, cen, (T)dtk, (T)dtd, ox, oy, oz, ux, uy, uz, (T)qs); break;
-        case 1: pmk::k_cic_field<T, 1><<<g, 256, 0, st>>>(p, sk, cen, (T)dtk, (T)dtd, ox, oy, oz, ux, uy, uz, (T)qs); break;
-        case 2: pmk::k_cic_field<T, 2><<<g, 256, 0, st>>>(p, sk, cen, (T)dtk, (T)dtd, ox, oy, oz, ux, uy, uz, (T)qs); break;
-        case 3: pmk::k_cic_field<T, 3><<<g, 256, 0, st>>>(p, sk, cen, (T)dtk, (T)dtd, ox, oy, oz, ux, uy, uz, (T)qs); break;
+        case 0: PM_CF(0); break;
+        case 1: PM_CF(1); break;
+        case 2: PM_CF(2); break;
+        case 3: PM_CF(3); break;
         default: return cudaErrorInvalidValue;
     }
+#undef PM_CF
+    return cudaGetLastError();
+}
+
+static cudaError_t cic_slots(long long *a, long long *b, long long n, cudaStream_t st) {
+    pmk::k_cic_slots<<<(unsigned)std::min<long long>((n / 2 + 255) / 256, 152 * 16), 256, 0, st>>>(a, b, n);
     return cudaGetLastError();
 }
 
@@ -441,7 +542,7 @@ template <typename T>
 cudaError_t pm_launch_cic_gather(const PartK<T> &p, const SysK &sk, const CenK *cen, T *gx, T *gy, T *gz, T *gm,
                                  cudaStream_t st) {
     if (p.n <= 0) return cudaSuccess;
-    pmk::k_cic_gather<T><<<pmk_cic_host::grid_for(p.n), 256, 0, st>>>(p, sk, cen, gx, gy, gz, gm);
+    pmk::k_cic_gather<T><<<pmk_cic_host::grid_for(p.n), pmk::CIC_THREADS, 0, st>>>(p, sk, cen, gx, gy, gz, gm);
     return cudaGetLastError();
 }
 
@@ -449,15 +550,16 @@ template <typename T>
 cudaError_t pm_launch_cic_umax(const PartK<T> &p, const T *ux, const T *uy, const T *uz, unsigned *out,
                                cudaStream_t st) {
     if (p.n <= 0) return cudaSuccess;
-    pmk::k_cic_umax<T><<<pmk_cic_host::grid_for(p.n), 256, 0, st>>>(p, ux, uy, uz, out);
+    pmk::k_cic_umax<T><<<pmk_cic_host::grid_for(p.n, 256), 256, 0, st>>>(p, ux, uy, uz, out);
     return cudaGetLastError();
 }
 
 #define PM_CIC_INSTANTIATE(T)                                                                                  \
-    template cudaError_t pm_launch_cic_deposit<T>(const PartK<T> &, const SysK &, const CenK *, cudaStream_t); \
+    template cudaError_t pm_launch_cic_deposit<T>(const PartK<T> &, const SysK &, const CenK *, const unsigned *, \
+                                                  cudaStream_t);                                               \
     template cudaError_t pm_launch_cic_field<T>(int, const PartK<T> &, const SysK &, const CenK *, double,     \
                                                 double, T *, T *, T *, const T *, const T *, const T *, double, \
-                                                cudaStream_t);                                                 \
+                                                const unsigned *, cudaStream_t);                               \
     template cudaError_t pm_launch_cic_gather<T>(const PartK<T> &, const SysK &, const CenK *, T *, T *, T *,  \
                                                  T *, cudaStream_t);                                           \
     template cudaError_t pm_launch_cic_umax<T>(const PartK<T> &, const T *, const T *, const T *, unsigned *,  \

@@ -638,6 +638,13 @@ __global__ void __launch_bounds__(256) k_sort_scatter(PartK<T> p, PartK<T> d, co
     if (perm) perm[j] = i;
 }
 
+// The order alone: ord[new] = old.
+static __global__ void __launch_bounds__(256) k_sort_index(long long n, const unsigned *key, const unsigned *rank,
+                                                           const unsigned *off, unsigned *ord) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) ord[(long long)off[key[i]] + rank[i]] = (unsigned)i;
+}
+
 template <typename T>
 __global__ void k_count_lost(PartK<T> p, unsigned long long *out) {
     unsigned long long c = 0;
@@ -875,24 +882,43 @@ cudaError_t pm_launch_recentre(const PartK<T> &p, const SysK &sk, CenK *cen, lon
     return cudaGetLastError();
 }
 
+// Keys, ranks and the exclusive scan of the key counts (left in count).
+template <typename T>
+cudaError_t pm_sort_offsets(const PartK<T> &p, const SysK &sk, const CenK *cen, const SortK &so, unsigned *count,
+                            unsigned *key, unsigned *rank, unsigned *bsum, cudaStream_t st) {
+    cudaError_t e = cudaMemsetAsync(count, 0, (size_t)so.nkeys * sizeof(unsigned), st);
+    if (e) return e;
+    pmk::k_sort_key<T><<<(unsigned)((p.n + 255) / 256), 256, 0, st>>>(p, sk, cen, so, count, key, rank);
+    const int nb = (int)((so.nkeys + pmk::SCAN_TILE - 1) / pmk::SCAN_TILE);
+    pmk::k_scan_reduce<<<nb, 256, 0, st>>>(count, so.nkeys, bsum);
+    pmk::k_scan_top<<<1, 1024, 0, st>>>(bsum, nb);
+    pmk::k_scan_down<<<nb, 256, 0, st>>>(count, so.nkeys, bsum);
+    return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t pm_launch_sort(const PartK<T> &p, const PartK<T> &scratch, const SysK &sk, const CenK *cen,
                            const SortK &so, unsigned *count, unsigned *key, unsigned *rank, unsigned *bsum,
                            long long *perm, cudaStream_t st) {
     if (p.n <= 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(count, 0, (size_t)so.nkeys * sizeof(unsigned), st);
+    cudaError_t e = pm_sort_offsets(p, sk, cen, so, count, key, rank, bsum, st);
     if (e) return e;
     const unsigned g = (unsigned)((p.n + 255) / 256);
-    pmk::k_sort_key<T><<<g, 256, 0, st>>>(p, sk, cen, so, count, key, rank);
-    const int nb = (int)((so.nkeys + pmk::SCAN_TILE - 1) / pmk::SCAN_TILE);
-    pmk::k_scan_reduce<<<nb, 256, 0, st>>>(count, so.nkeys, bsum);
-    pmk::k_scan_top<<<1, 1024, 0, st>>>(bsum, nb);
-    pmk::k_scan_down<<<nb, 256, 0, st>>>(count, so.nkeys, bsum);
     pmk::k_sort_scatter<T><<<g, 256, 0, st>>>(p, scratch, key, rank, count, perm);
     if ((e = cudaGetLastError())) return e;
     PartK<T> sc = scratch;
     sc.n = p.n;
     pmk::k_copy_particles<T><<<g, 256, 0, st>>>(sc, p);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t pm_launch_order(const PartK<T> &p, const SysK &sk, const CenK *cen, const SortK &so, unsigned *count,
+                            unsigned *key, unsigned *rank, unsigned *bsum, unsigned *ord, cudaStream_t st) {
+    if (p.n <= 0) return cudaSuccess;
+    const cudaError_t e = pm_sort_offsets(p, sk, cen, so, count, key, rank, bsum, st);
+    if (e) return e;
+    pmk::k_sort_index<<<(unsigned)((p.n + 255) / 256), 256, 0, st>>>(p.n, key, rank, count, ord);
     return cudaGetLastError();
 }
 
@@ -916,4 +942,6 @@ cudaError_t pm_launch_count_lost(const PartK<T> &p, unsigned long long *out, cud
     template cudaError_t pm_launch_count_lost<T>(const PartK<T> &, unsigned long long *, cudaStream_t);       \
     template cudaError_t pm_launch_sort<T>(const PartK<T> &, const PartK<T> &, const SysK &, const CenK *,     \
                                            const SortK &, unsigned *, unsigned *, unsigned *, unsigned *,       \
-                                           long long *, cudaStream_t);
+                                           long long *, cudaStream_t);                                          \
+    template cudaError_t pm_launch_order<T>(const PartK<T> &, const SysK &, const CenK *, const SortK &, unsigned *, \
+                                            unsigned *, unsigned *, unsigned *, unsigned *, cudaStream_t);

@@ -110,17 +110,26 @@ cudaError_t pm_launch_sort(const PartK<T> &p, const PartK<T> &scratch, const Sys
 // CIC variant (differentiable runs).  field modes: 0 kick (dtk) and drift
 // (dtd), 1 write accelerations to o*, 2 add the direct term of the adjoint
 // for cotangent u to o*, 3 spread u into the density slots as int64 with
-// scale qs (adjoint densities).
+// scale qs (adjoint densities by region; pm_launch_cic_slots then forms the
+// pair slots a and b of one grid's n cells).  ord: the order in which the
+// particles are processed (a permutation of 0..n-1; null: as stored), which
+// no result depends on.
 template <typename T>
-cudaError_t pm_launch_cic_deposit(const PartK<T> &p, const SysK &sk, const CenK *cen, cudaStream_t st);
+cudaError_t pm_launch_cic_deposit(const PartK<T> &p, const SysK &sk, const CenK *cen, const unsigned *ord,
+                                  cudaStream_t st);
 template <typename T>
 cudaError_t pm_launch_cic_field(int mode, const PartK<T> &p, const SysK &sk, const CenK *cen, double dtk, double dtd,
                                 T *ox, T *oy, T *oz, const T *ux, const T *uy, const T *uz, double qs,
-                                cudaStream_t st);
+                                const unsigned *ord, cudaStream_t st);
+cudaError_t pm_launch_cic_slots(long long *a, long long *b, long long n, cudaStream_t st);
 // Adds the field term of the adjoint (from the adjoint solve's potentials).
 template <typename T>
 cudaError_t pm_launch_cic_gather(const PartK<T> &p, const SysK &sk, const CenK *cen, T *gx, T *gy, T *gz, T *gm,
                                  cudaStream_t st);
+// The order of pm_launch_sort as an index: ord[new] = old (n < 2^32).
+template <typename T>
+cudaError_t pm_launch_order(const PartK<T> &p, const SysK &sk, const CenK *cen, const SortK &so, unsigned *count,
+                            unsigned *key, unsigned *rank, unsigned *bsum, unsigned *ord, cudaStream_t st);
 // max |u| over live particles into *out (float bits, atomicMax; zero it first).
 template <typename T>
 cudaError_t pm_launch_cic_umax(const PartK<T> &p, const T *ux, const T *uy, const T *uz, unsigned *out,

@@ -1,0 +1,95 @@
+"""The CIC kernels' processing order: from 2^16 particles they run in spatial
+order, share atomics within runs of one cell and take each point once per
+level.  Densities, gradients and trajectories must not depend on it."""
+import numpy as np
+import pytest
+
+from paper_1210_1736_gb300 import pm, workloads as W
+from tests._harness import cast
+
+pytestmark = pytest.mark.gpu
+
+
+def _case(precision, n, crowd):
+    w = W.merger(n_gal=n - 3_000, n_sat=3_000, grids=((32,), (32,), (32, 32, 8), (16,)), seed_id=21,
+                 precision=precision, q_m=0.8, r_apo=3.0)
+    if crowd:   # runs longer than a warp: a tenth of the points in a few cells
+        k = n // 10
+        w["pos"][:, :k] = w["pos"][:, :1] + 1e-3 * np.sign(w["pos"][:, :k])
+    return w
+
+
+def _all(w, perm, order):
+    """Densities, accelerations and vector-Jacobian product with the particles
+    stored in the order perm, given back in w's; order: whether the library
+    may order them (with one particle fewer than it asks for, it may not)."""
+    import torch
+    m = cast(w, w["m"])
+    ctx = pm.Context(w, W.mass_bound(m))
+    rng = np.random.default_rng(5)
+    u = cast(w, rng.normal(size=w["pos"].shape))
+    p = pm.Particles(cast(w, w["pos"])[:, perm], cast(w, w["vel"])[:, perm], m[perm], w["gal"][perm],
+                     precision=w["precision"])
+    ctx.cic_deposit(p)
+    rho = {k: ctx.density(*k) for k in ctx.shapes}
+    ctx.solve()
+    acc = torch.stack(ctx.cic_force(p))
+    gx, gm = torch.zeros_like(acc), torch.zeros_like(p.m)
+    ctx.cic_vjp(p, torch.tensor(u[:, perm], device="cuda").contiguous(), gx, gm)
+    back = np.argsort(perm)
+    out = [t.cpu().numpy()[..., back] for t in (acc, gx, gm)]
+    ctx.close()
+    return rho, out
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("n,crowd", [(1 << 16, False), ((1 << 16) + 1, True), (70_003, False)])
+def test_order_changes_nothing(precision, n, crowd):
+    w = _case(precision, n, crowd)
+    a_rho, a = _all(w, np.arange(n), True)
+    b_rho, b = _all(w, np.random.default_rng(3).permutation(n), True)
+    for k in a_rho:
+        assert np.array_equal(a_rho[k], b_rho[k]), k
+    for s, t in zip(a, b):
+        assert np.array_equal(s, t)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_ordered_equals_unordered(precision):
+    """The same system just below the limit, and above it with massless
+    particles added: the sums are the same integers."""
+    n = (1 << 16) - 1
+    w = _case(precision, n, True)
+    big = dict(w)
+    for k in ("pos", "vel"):
+        big[k] = np.concatenate([w[k], w[k][:, :500]], axis=1)
+    big["m"] = np.concatenate([w["m"], np.zeros(500)])
+    big["gal"] = np.concatenate([w["gal"], w["gal"][:500]])
+    a_rho, a = _all(w, np.arange(n), False)
+    b_rho, b = _all(big, np.arange(n + 500), True)
+    for k in a_rho:
+        assert np.array_equal(a_rho[k], b_rho[k]), k
+    assert np.array_equal(a[0], b[0][:, :n])
+
+
+def test_other_particles_of_the_same_number():
+    """A call after another set's deposit runs in that set's order: results
+    are those of its own particles."""
+    import torch
+    n = 1 << 16
+    w, v = _case("fp32", n, False), _case("fp32", n, True)
+    m = cast(w, w["m"])
+    ctx = pm.Context(w, W.mass_bound(m))
+    ps = [pm.Particles(cast(q, q["pos"]), cast(q, q["vel"]), m, q["gal"]) for q in (w, v)]
+    ctx.cic_deposit(ps[0])
+    ctx.solve()
+    a = torch.stack(ctx.cic_force(ps[1]))    # p1 in p0's order
+    ctx2 = pm.Context(w, W.mass_bound(m))
+    half = pm.Particles.from_tensors(torch.stack([ps[0].x, ps[0].y, ps[0].z]), torch.stack([ps[0].vx, ps[0].vy, ps[0].vz]),
+                                     ps[0].m, ps[0].gal)
+    ctx2.cic_deposit(half)
+    ctx2.solve()
+    k = n - 7                                # another number: as stored
+    sub = pm.Particles(cast(v, v["pos"])[:, :k], cast(v, v["vel"])[:, :k], m[:k], v["gal"][:k])
+    b = torch.stack(ctx2.cic_force(sub))
+    assert torch.equal(a[:, :k], b)
