@@ -212,6 +212,14 @@ __global__ void __launch_bounds__(NT) k_xinv(const __grid_constant__ PassBatch B
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// The first A-aligned address of a shared array.  An offset, not a masked
+// address: through an integer the compiler loses the address space and reads
+// shared memory by generic loads (stalls of the global pipe, lg_throttle and
+// long_scoreboard, in the column passes).
+template <unsigned A> __device__ __forceinline__ unsigned char *aligned_smem(unsigned char *p) {
+    return p + (-smem_addr(p) & (A - 1));
+}
+
 __device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
 }
@@ -326,7 +334,7 @@ __global__ void __launch_bounds__(CShape<T, L>::THREADS, 3) k_col(const __grid_c
     constexpr int NBUF = col_nbuf<T, L, MODE>();
 
     extern __shared__ __align__(128) unsigned char smraw[];
-    unsigned char *base = reinterpret_cast<unsigned char *>(((uintptr_t)smraw + 127) & ~(uintptr_t)127);
+    unsigned char *base = aligned_smem<128>(smraw);
     uint64_t *bar = reinterpret_cast<uint64_t *>(base);                 // 2 mbarriers
     C *buf0 = reinterpret_cast<C *>(base + 128);
     C *buf1 = NBUF == 2 ? buf0 + ROWS * COLS : buf0;
@@ -546,7 +554,7 @@ __global__ void __launch_bounds__(WShape<T, L>::THREADS, ((L >= 512 || DM == 2) 
     // stage goes by shuffles)
     constexpr bool IREV = !pmfft::inv_fwd_plan(L);
     extern __shared__ __align__(128) unsigned char smraw[];
-    unsigned char *base = reinterpret_cast<unsigned char *>(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
+    unsigned char *base = aligned_smem<1024>(smraw);
     C *xch = reinterpret_cast<C *>(base + 2 * S::BUF);
     C *tw = xch + S::COLS * S::LDR;
     uint64_t *full = reinterpret_cast<uint64_t *>(tw + pmfft::tw_total(L));   // tile loaded (tx bytes)

@@ -256,7 +256,7 @@ template <int L, int MODE> __global__ void __launch_bounds__(FXT, 3) k_yfx(const
     constexpr int BOXR = ROWS < 256 ? ROWS : 256, NBOX = ROWS / BOXR;
     constexpr int OROWS = INV ? L / 2 : L, OBOX = OROWS < 256 ? OROWS : 256, NOUT = INV ? E / 2 : E;
     extern __shared__ __align__(128) unsigned char smraw[];
-    unsigned char *base = reinterpret_cast<unsigned char *>(((uintptr_t)smraw + 127) & ~(uintptr_t)127);
+    unsigned char *base = aligned_smem<128>(smraw);
     fx2 *in = reinterpret_cast<fx2 *>(base);
     fx2 *sm = in + ROWS * COLS;
     fxw *tw = reinterpret_cast<fxw *>(sm + L * COLS);
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(FXT, DM == 2 ? 2 : 3) k_zfx(const __grid_const
     static_assert(S::THREADS == FXT, "tile shape");
     constexpr int TPC = S::TPC;
     extern __shared__ __align__(128) unsigned char smraw[];
-    unsigned char *base = reinterpret_cast<unsigned char *>(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
+    unsigned char *base = aligned_smem<1024>(smraw);
     fx2 *xch = reinterpret_cast<fx2 *>(base + 2 * S::BUF);
     fx2 *keep = DM == 2 ? xch + S::COLS * S::LDR : xch;
     fxw *tw = reinterpret_cast<fxw *>(keep + S::COLS * S::LDR);
