@@ -43,10 +43,14 @@ __host__ __device__ constexpr int tw_stage_size(int L, int S, bool rev) {
 __host__ __device__ constexpr int tw_dir_size(int L, bool rev) {
     return tw_stage_size(L, 1, rev) * (nstages(L) > 1) + tw_stage_size(L, 2, rev) * (nstages(L) > 2);
 }
+__host__ __device__ constexpr bool one_plan(int L) { return L != 64 && L != 128; }
+__host__ __device__ constexpr int tw_rev_base(int L) { return L == 16 || L == 256 ? 0 : tw_dir_size(L, false); }
 __host__ __device__ constexpr int tw_offset(int L, int S, bool rev) {
-    return (rev ? tw_dir_size(L, false) : 0) + (S >= 2 ? tw_stage_size(L, 1, rev) : 0);
+    return (rev ? tw_rev_base(L) : 0) + (S >= 2 ? tw_stage_size(L, 1, rev) : 0);
 }
-__host__ __device__ constexpr int tw_total(int L) { return tw_dir_size(L, false) + tw_dir_size(L, true); }
+__host__ __device__ constexpr int tw_total(int L) {
+    return tw_dir_size(L, false) + (one_plan(L) ? 0 : tw_dir_size(L, true));
+}
 
 template <int L, int S, bool REV, int STEP = 1, typename C>   // g: every STEP-th entry is w^m
 __device__ __forceinline__ void expand_stage_twiddles(C *tab, const C *g) {
@@ -59,9 +63,12 @@ __device__ __forceinline__ void expand_stage_twiddles(C *tab, const C *g) {
 }
 // Builds the stage tables in shared memory from the plain table
 // g[m] = w^m, m < L (the caller synchronises before use).
+// A pass of both directions whose inverse runs the forward plan (inv_fwd_plan,
+// or a plan that equals its reverse) keeps the forward tables only.
 template <int L, typename C> __device__ __forceinline__ void expand_twiddles(C *tab, const C *g) {
     expand_stage_twiddles<L, 1, false>(tab, g);
     expand_stage_twiddles<L, 2, false>(tab, g);
+    if (one_plan(L)) return;
     expand_stage_twiddles<L, 1, true>(tab, g);
     expand_stage_twiddles<L, 2, true>(tab, g);
 }

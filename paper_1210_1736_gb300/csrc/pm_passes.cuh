@@ -19,11 +19,12 @@
 // passes run on both (fx + i fy, fz + i Phi_1).
 //
 // The column passes are persistent: each block walks tiles of COLS adjacent
-// columns; a TMA tensor copy brings the next-but-one tile's input rows into
-// shared memory (two buffers, mbarrier completion; the FP32 512-point y
-// inverse keeps one and loads the next tile) while the block transforms the
-// current one; every column pass stages its outputs in shared memory and
-// sends them by TMA store.
+// columns; a TMA tensor copy brings the next tile's input rows into shared
+// memory (y passes: one buffer, free once the inputs are in registers; z: two,
+// the next but one) while the block transforms the current one; every column
+// pass stages its outputs in shared memory and sends them by TMA store.  (A
+// second buffer cost the 512-point y forward 11 %: 463 us against 411 on the
+// 16.5M-particle step's grids; nothing at 256.)
 #pragma once
 
 #include <cuda.h>
@@ -63,12 +64,15 @@ template <typename T, int L> constexpr size_t xpass_smem() {
 // written straight between global memory and registers with warp-contiguous
 // addresses; shared memory only carries the exchanges between stages, in a
 // padded row private to the row's warp.
+// Blocks per SM: four for the forward pass (its loads want the warps: 527, 398,
+// 339 us with two, three, four on the 16.5M-particle step's grids), three for
+// the inverse (247 us, four 254, five 309: its stores want the registers).
 // ---------------------------------------------------------------------------
 // x forward: z[x] = rho_a + i rho_b (scaled to mass), forward FFT of length
 // L = 2nx, all L outputs written to the row of the work array.  Persistent:
 // each block walks groups of LINES rows (the twiddle tables are built once).
 template <typename T, int L>
-__global__ void __launch_bounds__(NT) k_xfwd(const __grid_constant__ PassBatch B) {
+__global__ void __launch_bounds__(NT, 4) k_xfwd(const __grid_constant__ PassBatch B) {
     typedef typename cplx_t<T>::type C;
     typedef XShape<L> S;
     constexpr int NX = L / 2, NS = nstages(L);
@@ -138,7 +142,7 @@ __global__ void __launch_bounds__(NT) k_xfwd(const __grid_constant__ PassBatch B
 // Phi_b = Im, Phi_sum = Re + Im (or Re without partner; with a.split,
 // Phi_sum = Re and Phi_b = Im).  Persistent as k_xfwd.
 template <typename T, int L>
-__global__ void __launch_bounds__(NT) k_xinv(const __grid_constant__ PassBatch B) {
+__global__ void __launch_bounds__(NT, 3) k_xinv(const __grid_constant__ PassBatch B) {
     typedef typename cplx_t<T>::type C;
     typedef XShape<L> S;
     constexpr int NX = L / 2, NS = nstages(L);
@@ -297,22 +301,14 @@ template <> struct ColRows<COL_YFWD> { __host__ __device__ static constexpr int 
 template <> struct ColRows<COL_ZCONV> { __host__ __device__ static constexpr int of(int L) { return L / 2; } };
 template <> struct ColRows<COL_YINV> { __host__ __device__ static constexpr int of(int L) { return L; } };
 
-// Input buffers of the y pass: two (a tile prefetched two ahead), or one
-// for the FP32 512-point inverse, whose 32 KB tiles would otherwise hold it
-// to two blocks per SM by shared memory (one buffer: three, as its registers
-// allow; the next tile's load still runs during this tile's transform, which
-// has read its inputs into registers first).
-template <typename T, int L, int MODE> __host__ __device__ constexpr int col_nbuf() {
-    return (MODE == COL_YINV && L == 512 && sizeof(T) == 4) ? 1 : 2;
-}
-// Shared memory of a y pass: the input buffers, the exchange buffer and the
+// Shared memory of a y pass: the input buffer, the exchange buffer and the
 // stage twiddles of the one plan the pass runs (forward, or reversed for the
 // inverse).
 template <typename T, int L, int MODE> constexpr size_t col_smem() {
     typedef typename cplx_t<T>::type C;
     constexpr int COLS = CShape<T, L>::COLS;
     return 128 + (size_t)pmfft::tw_dir_size(L, MODE == COL_YINV) * sizeof(C) + (size_t)L * COLS * sizeof(C) +
-           col_nbuf<T, L, MODE>() * (size_t)ColRows<MODE>::of(L) * COLS * sizeof(C) + 3 * 128;
+           (size_t)ColRows<MODE>::of(L) * COLS * sizeof(C) + 2 * 128;
 }
 
 // Persistent y pass (forward or inverse) over a batch: the items' maps
@@ -331,18 +327,16 @@ __global__ void __launch_bounds__(CShape<T, L>::THREADS, 3) k_col(const __grid_c
     constexpr unsigned TILE_BYTES = (unsigned)(ROWS * COLS * sizeof(C));
     constexpr bool REV_IN = (MODE == COL_YINV);
     constexpr int SIGN_IN = (MODE == COL_YINV) ? 1 : -1;
-    constexpr int NBUF = col_nbuf<T, L, MODE>();
 
     extern __shared__ __align__(128) unsigned char smraw[];
     unsigned char *base = aligned_smem<128>(smraw);
-    uint64_t *bar = reinterpret_cast<uint64_t *>(base);                 // 2 mbarriers
-    C *buf0 = reinterpret_cast<C *>(base + 128);
-    C *buf1 = NBUF == 2 ? buf0 + ROWS * COLS : buf0;
-    C *sm = buf0 + NBUF * ROWS * COLS;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(base);
+    C *in = reinterpret_cast<C *>(base + 128);
+    C *sm = in + ROWS * COLS;
     // only this pass's plan's tables follow the exchange buffer: for the
     // reversed plan, the forward tables' offsets fall on the exchange
     // buffer's tail and are never read
-    C *tw = sm + L * COLS - (REV_IN ? pmfft::tw_dir_size(L, false) : 0);
+    C *tw = sm + L * COLS - (REV_IN ? pmfft::tw_rev_base(L) : 0);
     const int tid = threadIdx.x;
     const int c = tid % COLS, t = tid / COLS;
     const int nx2 = 2 * B.a[0].nx, ny2 = 2 * B.a[0].ny;   // the items' common shape, read once
@@ -357,53 +351,36 @@ __global__ void __launch_bounds__(CShape<T, L>::THREADS, 3) k_col(const __grid_c
         x = (int)((lt & (tiles_per_z - 1)) * COLS * S::EPC);
         y = (int)((lt >> ltpz) * ny2);
     };
-    auto issue = [&](long long tile, int b) {
+    auto issue = [&](long long tile) {
         int x, y;
         coords(tile & lmask, x, y);
         const CUtensorMap *map = &B.lmap[tile >> B.lgi];
-        C *dst = b ? buf1 : buf0;
-        mbar_expect_tx(&bar[b], TILE_BYTES);
+        mbar_expect_tx(bar, TILE_BYTES);
 #pragma unroll
-        for (int k = 0; k < NBOX; ++k) tma_load_2d(dst + k * BOXR * COLS, map, x, y + k * BOXR, &bar[b]);
+        for (int k = 0; k < NBOX; ++k) tma_load_2d(in + k * BOXR * COLS, map, x, y + k * BOXR, bar);
     };
 
-    __shared__ C *iwork[PM_BATCH];   // the items' work arrays (read once; see k_xfwd)
-    if (tid < B.n) iwork[tid] = static_cast<C *>(B.a[tid].work);
     if (tid == 0) {
         for (int i = 0; i < B.n; ++i)
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&B.lmap[i])) : "memory");
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
+        mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     pmfft::expand_stage_twiddles<L, 1, REV_IN>(tw, static_cast<const C *>(B.a[0].tw));
     pmfft::expand_stage_twiddles<L, 2, REV_IN>(tw, static_cast<const C *>(B.a[0].tw));
     __syncthreads();
     pdl_wait();
-    int issued[2] = {0, 0};   // loads issued per buffer (thread 0's count)
-    if (tid == 0) {
-        if (blockIdx.x < ntiles) { issue(blockIdx.x, 0); ++issued[0]; }
-        if (NBUF == 2 && blockIdx.x + gridDim.x < ntiles) { issue(blockIdx.x + gridDim.x, 1); ++issued[1]; }
-    }
+    if (tid == 0 && blockIdx.x < ntiles) issue(blockIdx.x);
 
     int it = 0;
     for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
         if (tile + gridDim.x >= ntiles) pdl_release();
-        const int b = NBUF == 2 ? (it & 1) : 0;
-        const unsigned phase = NBUF == 2 ? (unsigned)((it >> 1) & 1) : (unsigned)(it & 1);
-        // a tensor copy that never lands: report, wait (bounded) for the other
-        // copy in flight, stop; the decision is the same for the whole block
-        if (!__syncthreads_and(mbar_wait(&bar[b], phase) ? 1 : 0)) {
-            if (tid == 0) {
-                atomicExch(err, 1);
-                if (NBUF == 2) {
-                    const int o = b ^ 1, used_o = it >> 1;   // uses of buffer o completed so far
-                    if (issued[o] > used_o) mbar_wait(&bar[o], (unsigned)(used_o & 1));
-                }
-            }
+        // a tensor copy that never lands: report and stop (it is the only one
+        // in flight); the decision is the same for the whole block
+        if (!__syncthreads_and(mbar_wait(bar, (unsigned)(it & 1)) ? 1 : 0)) {
+            if (tid == 0) atomicExch(err, 1);
             break;
         }
-        const C *in = b ? buf1 : buf0;
         C v[E];
         constexpr int R0 = radix(L, 0, REV_IN);
         constexpr int OROWS = (MODE == COL_YFWD) ? L : L / 2, OBOX = OROWS < 256 ? OROWS : 256;
@@ -417,11 +394,10 @@ __global__ void __launch_bounds__(CShape<T, L>::THREADS, 3) k_col(const __grid_c
         // the previous tile's outputs have been read out of the exchange
         // buffer before this tile's stages write to it
         if (tid == 0) bulk_wait_read();
-        __syncthreads();   // buffer b consumed, previous tile's exchange done
-        if (tid == 0 && tile + NBUF * (long long)gridDim.x < ntiles) {
+        __syncthreads();   // the input buffer is consumed, the previous tile's exchange done
+        if (tid == 0 && tile + gridDim.x < ntiles) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            issue(tile + NBUF * (long long)gridDim.x, b);
-            ++issued[b];
+            issue(tile + gridDim.x);
         }
 
         static_assert(MODE == COL_YFWD || MODE == COL_YINV, "the z pass is k_colw");
