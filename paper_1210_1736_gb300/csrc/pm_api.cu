@@ -377,11 +377,12 @@ struct BatchItems {
 };
 
 // Launches `pass` of every item in chunks of `chunk` (<= PM_BATCH) items.
-template <typename T> cudaError_t launch_items(int pass, const BatchItems &it, size_t chunk, cudaStream_t st) {
+template <typename T> cudaError_t launch_items(int pass, const BatchItems &it, size_t chunk, cudaStream_t st, bool half = false) {
     for (size_t i0 = 0; i0 < it.a.size(); i0 += chunk) {
         PassBatch b;
         std::memset(&b, 0, sizeof(b));
         b.n = (int)std::min<size_t>(chunk, it.a.size() - i0);
+        if (half) b.kend = pm_half_cols(it.a[i0].nx, it.a[i0].ny, it.a[i0].nz, (int)sizeof(T));
         for (int k = 0; k < b.n; ++k) {
             b.a[k] = it.a[i0 + k];
             if (it.l[i0 + k]) b.lmap[k] = *it.l[i0 + k];
@@ -413,25 +414,26 @@ template <typename T> int launch_pass(pm_ctx *c, int pass, cudaStream_t st, int 
     const size_t chunk = c->batched ? PM_BATCH : 1;
     for (int ui = 0; ui < (int)c->units.size(); ++ui) {
         if (only >= 0 && ui != only) continue;
-        BatchItems main, d1, d2;
+        BatchItems main, d1, d2, half;   // half: sets by half their spectrum
         for (int gi : c->units[ui]) {
             const GeoBuf &gb = c->geos[gi];
             const pm_geometry &sg = gb.g;
             for (const Pair &pr : gb.pairs) {
                 PairArgs a = pair_args(c, gb, pr, shift);
+                BatchItems &plain = pr.b < 0 && !pr.diff && pm_half_cols(sg.nx, sg.ny, sg.nz, (int)sizeof(T)) ? half : main;
                 switch (pass) {
                     case PASS_XFWD:
                         a.tw = c->d_tw[tw_index(2 * sg.nx)];
-                        main.add(a);
+                        plain.add(a);
                         break;
                     case PASS_YFWD:
                         a.tw = c->d_tw[tw_index(2 * sg.ny)];
-                        main.add(a, &pr.yfwd, &pr.yinv);   // stores: boxes of 2ny rows
+                        plain.add(a, &pr.yfwd, &pr.yinv);   // stores: boxes of 2ny rows
                         break;
                     case PASS_ZCONV:
                         a.tw = c->d_tw[tw_index(2 * sg.nz)];
                         if (!pr.diff) {
-                            main.add(a, &pr.zmap);
+                            plain.add(a, &pr.zmap);
                         } else if (sg.nz <= 32 ||
                                    ((sg.nz == 64 || sg.nz == 128) && pm_col_cols(2 * sg.nz, (int)c->esz) <= sg.nx)) {
                             // both difference fields from one forward transform (H-hat read from the
@@ -447,7 +449,7 @@ template <typename T> int launch_pass(pm_ctx *c, int pass, cudaStream_t st, int 
                         break;
                     case PASS_YINV:
                         a.tw = c->d_tw[tw_index(2 * sg.ny)];
-                        main.add(a, &pr.yinv, &pr.yfwd);   // stores: boxes of ny rows
+                        plain.add(a, &pr.yinv, &pr.yfwd);   // stores: boxes of ny rows
                         if (pr.diff) {
                             a.work = pr.work2;
                             main.add(a, &pr.yinv2, &pr.yfwd2);
@@ -464,7 +466,7 @@ template <typename T> int launch_pass(pm_ctx *c, int pass, cudaStream_t st, int 
                             a.phi_sum = c->fd[pr.gi][0];
                             a.phi_b = c->fd[pr.gi][1];
                         }
-                        main.add(a);
+                        plain.add(a);
                         break;
                 }
             }
@@ -472,6 +474,7 @@ template <typename T> int launch_pass(pm_ctx *c, int pass, cudaStream_t st, int 
         cudaError_t e = launch_items<T>(pass, main, chunk, st);
         if (e == cudaSuccess) e = launch_items<T>(pass, d1, chunk, st);
         if (e == cudaSuccess) e = launch_items<T>(pass, d2, chunk, st);
+        if (e == cudaSuccess) e = launch_items<T>(pass, half, chunk, st, true);
         if (e != cudaSuccess) return fail(PM_E_CUDA, "FFT pass %d launch failed: %s", pass, cudaGetErrorString(e));
     }
     return PM_OK;

@@ -743,22 +743,23 @@ template <typename K> int resident_blocks(K kernel, int threads, size_t smem) {
 }
 
 // The pass kernels of a precision and length with their block sizes and
-// shared memory: FP32 in FP32, FP64 in fixed point.
-template <typename T, int L, int MODE> struct ColPass {
-    static auto kernel() { if constexpr (sizeof(T) == 4) return pmk::k_col<T, L, MODE>; else return pmk::k_yfx<L, MODE>; }
+// shared memory: FP32 in FP32, FP64 in fixed point.  HALF: half spectra
+// (kernels of their own: a branch on PassBatch::kend cost the whole ones 1-2 %).
+template <typename T, int L, int MODE, bool HALF> struct ColPass {
+    static auto kernel() { if constexpr (sizeof(T) == 4) return pmk::k_col<T, L, MODE, HALF>; else return pmk::k_yfx<L, MODE, HALF>; }
     static constexpr int threads = pmk::CShape<T, L>::THREADS;
     static size_t smem() { if constexpr (sizeof(T) == 4) return pmk::col_smem<T, L, MODE>(); else return pmk::fx_ysmem<L, MODE>(); }
 };
-template <typename T, int L, int DM> struct ZPass {
-    static auto kernel() { if constexpr (sizeof(T) == 4) return pmk::k_colw<T, L, DM>; else return pmk::k_zfx<L, DM>; }
+template <typename T, int L, int DM, bool HALF> struct ZPass {
+    static auto kernel() { if constexpr (sizeof(T) == 4) return pmk::k_colw<T, L, DM, HALF>; else return pmk::k_zfx<L, DM, HALF>; }
     static constexpr int threads = pmk::WShape<T, L>::THREADS;
     static size_t smem() { if constexpr (sizeof(T) == 4) return pmk::colw_smem<T, L>(); else return pmk::fx_zsmem<L, DM>(); }
 };
-template <typename T, int L, bool INV> struct XPass {
+template <typename T, int L, bool INV, bool HALF> struct XPass {
     static auto kernel() {
-        if constexpr (sizeof(T) == 8) return pmk::k_xfx<L, INV>;
-        else if constexpr (INV) return pmk::k_xinv<T, L>;
-        else return pmk::k_xfwd<T, L>;
+        if constexpr (sizeof(T) == 8) return pmk::k_xfx<L, INV, HALF>;
+        else if constexpr (INV) return pmk::k_xinv<T, L, HALF>;
+        else return pmk::k_xfwd<T, L, HALF>;
     }
     static constexpr int threads = sizeof(T) == 4 ? pmk::NT : pmk::FXT;   // the most a block has
     static size_t smem(int th) { if constexpr (sizeof(T) == 4) return pmk::xpass_smem<T, L>(); else return pmk::fx_xsmem<L>(th); }
@@ -771,14 +772,19 @@ template <class P> cudaError_t set_xsmem() {
 }
 template <typename T, int L> cudaError_t attrs_L() {
     cudaError_t e;
-    if ((e = set_smem<ColPass<T, L, COL_YFWD>>())) return e;
-    if ((e = set_smem<ColPass<T, L, COL_YINV>>())) return e;
-    if ((e = set_smem<ZPass<T, L, 0>>())) return e;
-    if ((e = set_smem<ZPass<T, L, 1>>())) return e;
+    if ((e = set_smem<ColPass<T, L, COL_YFWD, false>>())) return e;
+    if ((e = set_smem<ColPass<T, L, COL_YINV, false>>())) return e;
+    if ((e = set_smem<ZPass<T, L, 0, false>>())) return e;
+    if ((e = set_smem<ZPass<T, L, 1, false>>())) return e;
     if constexpr (L <= 256)
-        if ((e = set_smem<ZPass<T, L, 2>>())) return e;
-    if ((e = set_xsmem<XPass<T, L, false>>())) return e;
-    return set_xsmem<XPass<T, L, true>>();
+        if ((e = set_smem<ZPass<T, L, 2, false>>())) return e;
+    if ((e = set_smem<ColPass<T, L, COL_YFWD, true>>())) return e;
+    if ((e = set_smem<ColPass<T, L, COL_YINV, true>>())) return e;
+    if ((e = set_smem<ZPass<T, L, 0, true>>())) return e;
+    if ((e = set_xsmem<XPass<T, L, false, false>>())) return e;
+    if ((e = set_xsmem<XPass<T, L, false, true>>())) return e;
+    if ((e = set_xsmem<XPass<T, L, true, false>>())) return e;
+    return set_xsmem<XPass<T, L, true, true>>();
 }
 
 // Launch with programmatic stream serialisation (the FFT passes of a chain:
@@ -807,15 +813,21 @@ inline int ilog2(long long v) {
 }
 template <class P> cudaError_t launch_tiles(const PassBatch &b, cudaStream_t st) {
     static const int nb = resident_blocks(P::kernel(), P::threads, P::smem());
-    const long long grid = std::max(1LL, std::min((long long)b.n << b.lgi, (long long)nb * num_sms()));
+    const long long tiles = b.kend ? (long long)b.n * b.tpi : (long long)b.n << b.lgi;
+    const long long grid = std::max(1LL, std::min(tiles, (long long)nb * num_sms()));
     return launch_pdl(P::kernel(), (unsigned)grid, P::threads, P::smem(), st, b);
+}
+// Tiles of half spectra: `rows` rows of kend columns per item.
+inline void half_tiles(PassBatch &b, int cols, int rows) {
+    b.tpr = b.kend / cols;
+    b.tpi = rows * b.tpr;
 }
 // Row groups of an x pass.  FP64: the largest block (at least a warp) that
 // still gives every SM one.
-template <typename T, int L, bool INV> cudaError_t xpass_L(PassBatch b, cudaStream_t st) {
-    typedef XPass<T, L, INV> P;
+template <typename T, int L, bool INV, bool HALF> cudaError_t xpass_LH(PassBatch b, cudaStream_t st) {
+    typedef XPass<T, L, INV, HALF> P;
     constexpr int TPC = pmk::XShape<L>::TPC;
-    const long long rows = (long long)b.a[0].ny * b.a[0].nz;
+    const long long rows = (long long)b.a[0].ny * b.a[0].nz / (HALF ? 2 : 1);   // transforms
     int threads = P::threads;
     if (sizeof(T) == 8)
         while (threads > 32 && b.n * rows * TPC < (long long)threads * num_sms()) threads /= 2;
@@ -826,18 +838,25 @@ template <typename T, int L, bool INV> cudaError_t xpass_L(PassBatch b, cudaStre
     const long long grid = std::min((long long)b.n << b.lgi, (long long)nb * num_sms());
     return launch_pdl(P::kernel(), (unsigned)grid, threads, P::smem(threads), st, b);
 }
+template <typename T, int L, bool INV> cudaError_t xpass_L(const PassBatch &b, cudaStream_t st) {
+    return b.kend ? xpass_LH<T, L, INV, true>(b, st) : xpass_LH<T, L, INV, false>(b, st);
+}
 template <typename T, int L, int MODE> cudaError_t col_LM(PassBatch b, cudaStream_t st) {
     constexpr int COLS = pmk::CShape<T, L>::COLS;
+    half_tiles(b, COLS, b.a[0].nz);
     b.lgi = ilog2((long long)b.a[0].nz * ((2 * b.a[0].nx + COLS - 1) / COLS));
-    return launch_tiles<ColPass<T, L, MODE>>(b, st);
+    if (b.kend) return launch_tiles<ColPass<T, L, MODE, true>>(b, st);
+    return launch_tiles<ColPass<T, L, MODE, false>>(b, st);
 }
 template <typename T, int L> cudaError_t zconv_L(PassBatch b, cudaStream_t st) {
     b.lgi = ilog2(((long long)4 * b.a[0].ny * b.a[0].nx) / pmk::WShape<T, L>::COLS);   // COLS divides the columns
+    half_tiles(b, pmk::WShape<T, L>::COLS, 2 * b.a[0].ny);
     if constexpr (L <= 256)
-        if (b.a[0].dmode == 3) return launch_tiles<ZPass<T, L, 2>>(b, st);   // both difference fields (see PairArgs)
+        if (b.a[0].dmode == 3) return launch_tiles<ZPass<T, L, 2, false>>(b, st);   // both difference fields (see PairArgs)
     if (b.a[0].dmode == 3) return cudaErrorInvalidValue;
-    if (b.a[0].dmode != 0) return launch_tiles<ZPass<T, L, 1>>(b, st);
-    return launch_tiles<ZPass<T, L, 0>>(b, st);
+    if (b.a[0].dmode != 0) return launch_tiles<ZPass<T, L, 1, false>>(b, st);
+    if (b.kend) return launch_tiles<ZPass<T, L, 0, true>>(b, st);
+    return launch_tiles<ZPass<T, L, 0, false>>(b, st);
 }
 template <typename T, int L> cudaError_t col_L(const PassBatch &b, int mode, cudaStream_t st) {
     if (mode == COL_YFWD) return col_LM<T, L, COL_YFWD>(b, st);

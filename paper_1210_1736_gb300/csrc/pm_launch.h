@@ -50,6 +50,12 @@ struct PassBatch {
     PairArgs a[PM_BATCH];
     int n;
     int lgi;
+    // kend > 0: single real sets (rho_b null, no difference fields) by half
+    // their spectrum (pm_half_cols): two rows of a set travel as one complex
+    // row of the x passes, the column passes cover the columns kx < kend, tpr
+    // tiles per row of columns and tpi per item (set by the launcher; the
+    // column passes then have no use for lgi).
+    int kend, tpr, tpi;
 };
 
 // Columns per tile of the column passes for transform length L and real
@@ -57,6 +63,18 @@ struct PassBatch {
 // tensor-map box row of at most 256 eight-byte elements.
 __host__ __device__ constexpr int pm_col_cols(int L, int esz) {
     return (esz == 4 ? 4096 : 2048) / L;
+}
+
+// Columns of a single real set's half spectrum: nx + 1 rounded up to whole
+// tiles of the y and z passes (the x pass fills the rest with zeros); 0 where
+// that is no fewer than all 2nx, and the set is transformed whole.  A 256^3
+// grid, FP32, whole -> half: x 97 + 64 -> 50 + 45 us, y 136 + 138 -> 78 + 78,
+// z 398 -> 232.  Rows of 32 cells in FP64, whose half fills all their tiles, took
+// 10.7 -> 12.4 us in the x inverse and gained nothing elsewhere.
+inline int pm_half_cols(int nx, int ny, int nz, int esz) {
+    const int cy = pm_col_cols(2 * ny, esz), cz = pm_col_cols(2 * nz, esz), g = cy > cz ? cy : cz;
+    const int k = (nx + g) / g * g;
+    return k < 2 * nx ? k : 0;
 }
 
 // Columns per swizzled sub-tile of the z pass: as many as fill a 128-byte

@@ -69,9 +69,11 @@ template <typename T, int L> constexpr size_t xpass_smem() {
 // the inverse (247 us, four 254, five 309: its stores want the registers).
 // ---------------------------------------------------------------------------
 // x forward: z[x] = rho_a + i rho_b (scaled to mass), forward FFT of length
-// L = 2nx, all L outputs written to the row of the work array.  Persistent:
+// L = 2nx, all L outputs written to the row of the work array.  HALF (sets by
+// half their spectrum): z = row y + i row y + 1, separated after the FFT and
+// written to kx < kend of both rows.  Persistent:
 // each block walks groups of LINES rows (the twiddle tables are built once).
-template <typename T, int L>
+template <typename T, int L, bool HALF>
 __global__ void __launch_bounds__(NT, 4) k_xfwd(const __grid_constant__ PassBatch B) {
     typedef typename cplx_t<T>::type C;
     typedef XShape<L> S;
@@ -95,10 +97,12 @@ __global__ void __launch_bounds__(NT, 4) k_xfwd(const __grid_constant__ PassBatc
     pmfft::expand_twiddles<L>(tw, static_cast<const C *>(B.a[0].tw));
     __syncthreads();
     pdl_wait();
-    const long long nrows = (long long)ny * B.a[0].nz;
+    // HALF: r counts the row pairs (y, y + 1), y even
+    const long long nrows = (long long)ny * B.a[0].nz >> (HALF ? 1 : 0);
     const long long ngroups = (long long)B.n << lgi;   // row groups of every item
     const int lny = __ffs(ny) - 1;   // row r = z*ny + y; ny is a power of two
-    const T scale = (T)B.a[0].scale;
+    const T scale = (T)B.a[0].scale * (HALF ? (T)0.5 : (T)1);   // the halves of the separation
+    const int kend = B.kend;
     for (long long grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
         if (grp + gridDim.x >= ngroups) pdl_release();
         const int item = (int)(grp >> lgi);
@@ -107,8 +111,8 @@ __global__ void __launch_bounds__(NT, 4) k_xfwd(const __grid_constant__ PassBatc
         C *work = static_cast<C *>(const_cast<void *>(ip[item][2]));
         const long long r = (grp & ((1LL << lgi) - 1)) * S::LINES + line;
         const bool valid = r < nrows;
-        const long long *ra = rho_a + (valid ? r * NX : 0);
-        const long long *rb = rho_b ? rho_b + (valid ? r * NX : 0) : nullptr;
+        const long long *ra = rho_a + (valid ? (HALF ? 2 : 1) * r * NX : 0);
+        const long long *rb = HALF ? ra + NX : rho_b ? rho_b + (valid ? r * NX : 0) : nullptr;
         C v[E];
         constexpr int R0 = radix(L, 0, false);
 #pragma unroll
@@ -126,7 +130,38 @@ __global__ void __launch_bounds__(NT, 4) k_xfwd(const __grid_constant__ PassBatc
         // a row's TPC threads are consecutive lanes of one warp and its
         // exchange row is private: the exchanges synchronise the warp only
         pmfft::fft_core<L, false, -1, true, false, true>(v, sm, pmfft::RowLayout{line * S::LDR}, t, tw);
-        if (valid) {
+        if constexpr (HALF) {
+            // rows F0, F1 from their sum F0 + i F1 at k and L - k, k = 0..nx
+            C *const sp = sm + line * S::LDR;
+            const pmfft::RowLayout lay{0};
+            constexpr int RL = radix(L, NS - 1, false);
+#pragma unroll
+            for (int kk = 0; kk < E / RL; ++kk)
+#pragma unroll
+                for (int q = 0; q < RL; ++q) sp[lay(pmfft::in_row<L, NS - 1, false>(t, kk, q))] = v[kk * RL + q];
+            __syncwarp();
+            if (valid) {
+                const long long z = 2 * r >> lny, y = 2 * r & (ny - 1);
+                C *out = work + ((size_t)z * 2 * ny + y) * L;
+#pragma unroll
+                for (int j = 0; j <= E / 2; ++j) {
+                    const int k = t + j * S::TPC;
+                    if (k <= NX) {
+                        const C p = sp[lay(k)], m = sp[lay((L - k) & (L - 1))];
+                        C f0, f1;
+                        f0.x = p.x + m.x; f0.y = p.y - m.y;
+                        f1.x = p.y + m.y; f1.y = m.x - p.x;
+                        __stcg(out + k, f0);
+                        __stcg(out + L + k, f1);
+                    }
+                }
+                for (int k = NX + 1 + t; k < kend; k += S::TPC) {
+                    __stcg(out + k, czero<C>());
+                    __stcg(out + L + k, czero<C>());
+                }
+            }
+            __syncwarp();   // read before the next rows' exchange
+        } else if (valid) {
             const long long z = r >> lny, y = r & (ny - 1);
             C *out = work + ((size_t)z * 2 * ny + y) * L;
             constexpr int RL = radix(L, NS - 1, false);
@@ -140,8 +175,8 @@ __global__ void __launch_bounds__(NT, 4) k_xfwd(const __grid_constant__ PassBatc
 
 // x inverse: inverse FFT of length L = 2nx of each row y < ny; x < nx kept:
 // Phi_b = Im, Phi_sum = Re + Im (or Re without partner; with a.split,
-// Phi_sum = Re and Phi_b = Im).  Persistent as k_xfwd.
-template <typename T, int L>
+// Phi_sum = Re and Phi_b = Im).  HALF: rows y and y + 1 together, Re and Im.  Persistent as k_xfwd.
+template <typename T, int L, bool HALF>
 __global__ void __launch_bounds__(NT, 3) k_xinv(const __grid_constant__ PassBatch B) {
     typedef typename cplx_t<T>::type C;
     typedef XShape<L> S;
@@ -162,7 +197,7 @@ __global__ void __launch_bounds__(NT, 3) k_xinv(const __grid_constant__ PassBatc
     pmfft::expand_twiddles<L>(tw, static_cast<const C *>(B.a[0].tw));
     __syncthreads();
     pdl_wait();
-    const long long nrows = (long long)ny * B.a[0].nz;
+    const long long nrows = (long long)ny * B.a[0].nz >> (HALF ? 1 : 0);   // HALF: row pairs, as in k_xfwd
     const long long ngroups = (long long)B.n << lgi;
     const int lny = __ffs(ny) - 1;   // row r = z*ny + y; ny is a power of two
     for (long long grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
@@ -174,21 +209,56 @@ __global__ void __launch_bounds__(NT, 3) k_xinv(const __grid_constant__ PassBatc
         const C *work = static_cast<const C *>(ip[item][2]);
         const long long r = (grp & ((1LL << lgi) - 1)) * S::LINES + line;
         const bool valid = r < nrows;
-        const long long z = valid ? r >> lny : 0, y = valid ? r & (ny - 1) : 0;
+        const long long row = (HALF ? 2 : 1) * r;
+        const long long z = valid ? row >> lny : 0, y = valid ? row & (ny - 1) : 0;
         const C *in = work + ((size_t)z * 2 * ny + y) * L;
         C v[E];
         // the reversed plan, or the forward one where it closes with radix 2
         // (its exchange into that stage goes by shuffles)
         constexpr bool IREV = !pmfft::inv_fwd_plan(L);
         constexpr int R0 = radix(L, 0, IREV);
+        // HALF: k = 0, a potential's largest coefficient, is added after the
+        // transform: rounded once, not in every stage (the mean over k and -k
+        // that a whole spectrum forms in the real part has to be made up for:
+        // error of the potential 0.98e-7 whole, 1.01e-7 half, 0.93e-7
+        // half so; 128^3, FP32, relative 2-norm)
+        C dc = czero<C>();
+        if constexpr (HALF) {
+            // F0 + i F1 at k and, from the rows' symmetry, at L - k; at k = 0 and
+            // nx both are real (what their imaginary parts hold is rounding)
+            C *const sp = sm + line * S::LDR;
+            const pmfft::RowLayout lay{0};
 #pragma unroll
-        for (int kk = 0; kk < E / R0; ++kk)
+            for (int j = 0; j <= E / 2; ++j) {
+                const int k = t + j * S::TPC;
+                if (k <= NX) {
+                    C f0 = czero<C>(), f1 = f0, p, m;
+                    if (valid) { f0 = __ldg(in + k); f1 = __ldg(in + L + k); }
+                    if (k == 0 || k == NX) f0.y = f1.y = 0;
+                    p.x = f0.x - f1.y; p.y = f0.y + f1.x;
+                    m.x = f0.x + f1.y; m.y = f1.x - f0.y;
+                    sp[lay(k)] = p;
+                    if (k > 0 && k < NX) sp[lay(L - k)] = m;
+                }
+            }
+            __syncwarp();
+            dc = sp[lay(0)];
 #pragma unroll
-            for (int q = 0; q < R0; ++q)
-                v[kk * R0 + q] = valid ? __ldg(in + pmfft::in_row<L, 0, IREV>(t, kk, q)) : czero<C>();
+            for (int kk = 0; kk < E / R0; ++kk)
+#pragma unroll
+                for (int q = 0; q < R0; ++q) v[kk * R0 + q] = sp[lay(pmfft::in_row<L, 0, IREV>(t, kk, q))];
+            if (t == 0) v[0] = czero<C>();
+            __syncwarp();   // read before the exchange
+        } else {
+#pragma unroll
+            for (int kk = 0; kk < E / R0; ++kk)
+#pragma unroll
+                for (int q = 0; q < R0; ++q)
+                    v[kk * R0 + q] = valid ? __ldg(in + pmfft::in_row<L, 0, IREV>(t, kk, q)) : czero<C>();
+        }
         pmfft::fft_core<L, IREV, 1, false, true, true>(v, sm, pmfft::RowLayout{line * S::LDR}, t, tw);
         if (valid) {
-            T *phi_s = phi_sum + r * NX;
+            T *phi_s = phi_sum + row * NX;
             constexpr int RL = radix(L, NS - 1, IREV);
 #pragma unroll
             for (int kk = 0; kk < E / RL; ++kk)
@@ -197,7 +267,10 @@ __global__ void __launch_bounds__(NT, 3) k_xinv(const __grid_constant__ PassBatc
                     const int x = pmfft::in_row<L, NS - 1, IREV>(t, kk, q);
                     const C val = v[kk * RL + q];
                     // the arrays are global memory (pointers read from shared memory: say so)
-                    if (split) {
+                    if (HALF) {
+                        __stcg(phi_s + x, val.x + dc.x);
+                        __stcg(phi_s + NX + x, val.y + dc.y);
+                    } else if (split) {
                         __stcg(phi_s + x, val.x);
                         __stcg(phi_b + r * NX + x, val.y);
                     } else if (phi_b) {
@@ -318,7 +391,7 @@ template <typename T, int L, int MODE> constexpr size_t col_smem() {
 // as a tile, and leave by tensor stores through B.smap (boxes of the output
 // rows: 2ny for the forward, ny for the inverse; columns beyond nx2 are
 // clipped by the copy).
-template <typename T, int L, int MODE>
+template <typename T, int L, int MODE, bool HALF>
 __global__ void __launch_bounds__(CShape<T, L>::THREADS, 3) k_col(const __grid_constant__ PassBatch B) {
     typedef typename cplx_t<T>::type C;
     typedef CShape<T, L> S;
@@ -343,18 +416,25 @@ __global__ void __launch_bounds__(CShape<T, L>::THREADS, 3) k_col(const __grid_c
     int *const err = B.a[0].err;
     const long long tiles_per_z = (nx2 + COLS - 1) / COLS;   // a power of two, as nx2 and COLS
     const int ltpz = __ffs((int)tiles_per_z) - 1;
-    const long long ntiles = (long long)B.n << B.lgi;
+    const long long ntiles = HALF ? (long long)B.n * B.tpi : (long long)B.n << B.lgi;
     const long long lmask = (1LL << B.lgi) - 1;
 
-    // an item's tile -> TMA coordinates and the first column it covers
-    auto coords = [&](long long lt, int &x, int &y) {
+    // tile -> item and TMA coordinates
+    auto coords = [&](long long tile, int &x, int &y) {
+        if (HALF) {
+            const int item = (int)tile / B.tpi, lt = (int)tile - item * B.tpi, z = lt / B.tpr;
+            x = (lt - z * B.tpr) * COLS * S::EPC;
+            y = z * ny2;
+            return item;
+        }
+        const long long lt = tile & lmask;
         x = (int)((lt & (tiles_per_z - 1)) * COLS * S::EPC);
         y = (int)((lt >> ltpz) * ny2);
+        return (int)(tile >> B.lgi);
     };
     auto issue = [&](long long tile) {
         int x, y;
-        coords(tile & lmask, x, y);
-        const CUtensorMap *map = &B.lmap[tile >> B.lgi];
+        const CUtensorMap *map = &B.lmap[coords(tile, x, y)];
         mbar_expect_tx(bar, TILE_BYTES);
 #pragma unroll
         for (int k = 0; k < NBOX; ++k) tma_load_2d(in + k * BOXR * COLS, map, x, y + k * BOXR, bar);
@@ -421,8 +501,7 @@ __global__ void __launch_bounds__(CShape<T, L>::THREADS, 3) k_col(const __grid_c
         __syncthreads();
         if (tid == 0) {
             int x, y;
-            coords(tile & lmask, x, y);
-            const CUtensorMap *smap = &B.smap[tile >> B.lgi];
+            const CUtensorMap *smap = &B.smap[coords(tile, x, y)];
 #pragma unroll
             for (int k = 0; k < OROWS / OBOX; ++k) tma_store_2d(smap, x, y + k * OBOX, sm + k * OBOX * COLS);
             bulk_commit();
@@ -517,7 +596,7 @@ __device__ __forceinline__ uint32_t woff(int row, int c) {
 // products' outputs stored through smap, the second's in place through
 // lmap.  The modes are separate instantiations so that the plain pass
 // carries no mode branch.
-template <typename T, int L, int DM>
+template <typename T, int L, int DM, bool HALF>
 __global__ void __launch_bounds__(WShape<T, L>::THREADS, ((L >= 512 || DM == 2) ? 2 : 3))
     k_colw(const __grid_constant__ PassBatch B) {
     typedef WShape<T, L> S;
@@ -544,27 +623,38 @@ __global__ void __launch_bounds__(WShape<T, L>::THREADS, ((L >= 512 || DM == 2) 
     const int nx2 = 2 * a.nx, ny2 = 2 * a.ny, lnx2 = __ffs(nx2) - 1;
     // tile indices fit in 32 bits: at most 8 items of (2 * 256)^2 / COLS tiles
     const int lgi = B.lgi, lmask = (1 << lgi) - 1;
+    // tile -> item and first column
+    auto locate = [&](int tile, int &q0) {
+        if (HALF) {
+            const int item = tile / B.tpi, lt = tile - item * B.tpi, ky = lt / B.tpr;
+            q0 = (ky << lnx2) + (lt - ky * B.tpr) * S::COLS;
+            return item;
+        }
+        q0 = (tile & lmask) * S::COLS;
+        return tile >> lgi;
+    };
 
     // an item's tile <-> sub-tiles of the buffer, each NBOXI boxes of BOXI rows
     auto issue_load = [&](int tile, int b) {
-        const CUtensorMap *map = &B.lmap[tile >> lgi];
-        const int lt = tile & lmask;
+        int q0;
+        const CUtensorMap *map = &B.lmap[locate(tile, q0)];
         mbar_expect_tx(&full[b], S::BUF);
 #pragma unroll
         for (int s = 0; s < S::NSUB; ++s)
 #pragma unroll
             for (int k = 0; k < S::NBOXI; ++k)
                 tma_load_2d(base + b * S::BUF + s * S::RIN * S::P + k * S::BOXI * S::P, map,
-                            (int)((lt * S::COLS + s * S::SW) * S::EPC), k * S::BOXI, &full[b]);
+                            (q0 + s * S::SW) * S::EPC, k * S::BOXI, &full[b]);
     };
     auto issue_store = [&](int tile, const unsigned char *src, bool to_lmap = false) {
-        const CUtensorMap *smap = to_lmap ? &B.lmap[tile >> lgi] : &B.smap[tile >> lgi];
-        const int lt = tile & lmask;
+        int q0;
+        const int item = locate(tile, q0);
+        const CUtensorMap *smap = to_lmap ? &B.lmap[item] : &B.smap[item];
 #pragma unroll
         for (int s = 0; s < S::NSUB; ++s)
 #pragma unroll
             for (int k = 0; k < S::NBOXI; ++k)
-                tma_store_2d(smap, (int)((lt * S::COLS + s * S::SW) * S::EPC), k * S::BOXI,
+                tma_store_2d(smap, (q0 + s * S::SW) * S::EPC, k * S::BOXI,
                              src + s * S::RIN * S::P + k * S::BOXI * S::P);
     };
 
@@ -600,7 +690,7 @@ __global__ void __launch_bounds__(WShape<T, L>::THREADS, ((L >= 512 || DM == 2) 
     // thread 0 issues every copy; counts per buffer of loads issued and of
     // tiles sent (to drain after an expired wait)
     int issued0 = 0, issued1 = 0, done0 = 0, done1 = 0;
-    const int nt0 = B.n << lgi;
+    const int nt0 = HALF ? B.n * B.tpi : B.n << lgi;
     int deferred = -1;   // thread 0: tile whose buffer awaits its refill
     if (tid == 0) {
         if ((int)blockIdx.x < nt0) { issue_load(blockIdx.x, 0); ++issued0; }
@@ -622,12 +712,12 @@ __global__ void __launch_bounds__(WShape<T, L>::THREADS, ((L >= 512 || DM == 2) 
             break;
         }
         unsigned char *in = base + b * S::BUF;
-        const int lt = tile & lmask;                       // the tile within its item
-        const T *hhat = ihhat[tile >> lgi];
+        int q0;                                            // the tile's first column
+        const T *hhat = ihhat[locate(tile, q0)];
         if constexpr (FREE) {
             // this warp's column (one per warp): its H-hat column lands in
             // shared memory while the forward FFT runs
-            const int qc = lt * S::COLS + c;
+            const int qc = q0 + c;
             const int ky = qc >> lnx2, kx = qc & (nx2 - 1);
             const int kyr = ky <= a.ny ? ky : ny2 - ky, kxr = kx <= a.nx ? kx : nx2 - kx;
             const unsigned char *src =
@@ -663,7 +753,6 @@ __global__ void __launch_bounds__(WShape<T, L>::THREADS, ((L >= 512 || DM == 2) 
             }
             deferred = -1;
         }
-        const int q0 = lt * S::COLS;
         const int k0 = (int)(q0 & (nx2 - 1));
         if (hstage && tid == 0) {
             const int ky0 = (int)(q0 >> lnx2);
@@ -681,7 +770,7 @@ __global__ void __launch_bounds__(WShape<T, L>::THREADS, ((L >= 512 || DM == 2) 
         // the last forward stage's output row)
         C dxy = czero<C>();
         if ((DM == 1 && a.dmode == 1) || DM == 2) {
-            const int qc = lt * S::COLS + c;
+            const int qc = q0 + c;
             const C ex = static_cast<const C *>(a.dtx)[qc & (nx2 - 1)];
             const C ey = static_cast<const C *>(a.dty)[qc >> lnx2];
             dxy.x = ex.x - ey.y;
@@ -783,7 +872,7 @@ __global__ void __launch_bounds__(WShape<T, L>::THREADS, ((L >= 512 || DM == 2) 
         } else {
             // H-hat of column (kyr, kxr), stored by pm_build_hhat in the
             // order hhat_thread_major gives for L
-            const int q = lt * S::COLS + c;
+            const int q = q0 + c;
             const int ky = q >> lnx2, kx = q & (nx2 - 1);   // nx2 is a power of two
             const int kyr = ky <= a.ny ? ky : ny2 - ky;
             const int kxr = kx <= a.nx ? kx : nx2 - kx;

@@ -139,7 +139,7 @@ template <int L> constexpr size_t fx_xsmem(int threads) {
 
 // INV = false: integer densities in, spectrum rows out; INV: spectrum rows
 // in, potentials out (as k_xfwd and k_xinv).
-template <int L, bool INV> __global__ void __launch_bounds__(FXT, 3) k_xfx(const __grid_constant__ PassBatch B) {
+template <int L, bool INV, bool HALF> __global__ void __launch_bounds__(FXT, 3) k_xfx(const __grid_constant__ PassBatch B) {
     typedef XShape<L> S;
     constexpr int NX = L / 2, TPC = S::TPC;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -159,7 +159,8 @@ template <int L, bool INV> __global__ void __launch_bounds__(FXT, 3) k_xfx(const
     pmfft::expand_stage_twiddles<L, 2, false>(tw, static_cast<const fxw *>(B.a[0].tw));
     __syncthreads();
     pdl_wait();
-    const long long nrows = (long long)ny * B.a[0].nz;
+    const long long nrows = (long long)ny * B.a[0].nz >> (HALF ? 1 : 0);   // HALF: row pairs, as in k_xfwd
+    const int kend = B.kend;
     const long long ngroups = (long long)B.n << lgi;
     const int lny = __ffs(ny) - 1;   // row r = z*ny + y; ny is a power of two
     const int ex0 = exponent_of(B.a[0].scale);
@@ -170,11 +171,61 @@ template <int L, bool INV> __global__ void __launch_bounds__(FXT, 3) k_xfx(const
         const int item = (int)(grp >> lgi);
         const long long r = (grp & ((1LL << lgi) - 1)) * lines + line;
         const bool valid = r < nrows;
-        const long long z = valid ? r >> lny : 0, y = valid ? r & (ny - 1) : 0;
+        const long long r1 = (HALF ? 2 : 1) * r;   // the (first) row
+        const long long z = valid ? r1 >> lny : 0, y = valid ? r1 & (ny - 1) : 0;
         double2 *row = static_cast<double2 *>(ip[item][2]) + ((size_t)z * 2 * ny + y) * L;
         fx2 v[E];
         FxScale<false> sc{ex0, nullptr, 0};
-        if constexpr (INV) {
+        if constexpr (INV && HALF) {
+            // slots k <= nx: F0(k); above: F1(L - k), and F1(0), F1(nx) beside
+            unsigned m = 0;
+            double2 ends = make_double2(0.0, 0.0);   // F1(0) (t = 0) and F1(nx)
+#pragma unroll
+            for (int e = 0; e <= E / 2; ++e) {
+                const int k = t + e * TPC;
+                if (k > NX) continue;
+                double2 d = make_double2(0.0, 0.0), f = d;
+                if (valid) {
+                    d = __ldg(row + k);
+                    f = __ldg(row + L + k);
+                }
+                m = max(m, max(max(pmfx::dmag(d.x), pmfx::dmag(d.y)), max(pmfx::dmag(f.x), pmfx::dmag(f.y))));
+                *reinterpret_cast<double2 *>(sm + lay(k)) = d;
+                if (k > 0 && k < NX) *reinterpret_cast<double2 *>(sm + lay(L - k)) = f;
+                else if (k == 0) ends.x = f.x;   // real, up to rounding
+                else ends.y = f.x;
+            }
+            // a bit less than FX_TOP: F0 + i F1 adds two components
+            const int em = pmfx::group_em(pmfx::warp_max(m));
+            sc.ex = pmfx::group_ex(em, pmfx::FX_TOP) + 1;
+            __syncwarp();
+            fx_from(E, em + 1, mine);
+            __syncwarp();
+            // F0 + i F1 at k, and at L - k from the rows' symmetry
+#pragma unroll 1
+            for (int e = 0; e <= E / 2; ++e) {
+                const int k = t + e * TPC;
+                if (k > NX) break;
+                const fx2 f0 = sm[lay(k)];
+                if (k == 0 || k == NX) {
+                    fx2 p;
+                    p.x = f0.x;
+                    p.y = pmfx::from_double<pmfx::FX_TOP>(k == 0 ? ends.x : ends.y, em + 1);
+                    sm[lay(k)] = p;
+                    continue;
+                }
+                const fx2 f1 = sm[lay(L - k)];
+                fx2 p, q;
+                p.x = f0.x - f1.y; p.y = f0.y + f1.x;
+                q.x = f0.x + f1.y; q.y = f1.x - f0.y;
+                sm[lay(k)] = p;
+                sm[lay(L - k)] = q;
+            }
+            __syncwarp();
+#pragma unroll
+            for (int e = 0; e < E; ++e) v[e] = swapped(*mine(e));
+            __syncwarp();   // read before the exchange writes
+        } else if constexpr (INV) {
             unsigned m = 0;
 #pragma unroll
             for (int e = 0; e < E; ++e) {
@@ -190,9 +241,9 @@ template <int L, bool INV> __global__ void __launch_bounds__(FXT, 3) k_xfx(const
             for (int e = 0; e < E; ++e) v[e] = swapped(*mine(e));
             __syncwarp();   // read before the exchange writes
         } else {
-            const long long *ra = static_cast<const long long *>(ip[item][0]) + (valid ? r * NX : 0);
-            const long long *rb = static_cast<const long long *>(ip[item][1]);
-            if (rb) rb += valid ? r * NX : 0;
+            const long long *ra = static_cast<const long long *>(ip[item][0]) + (valid ? r1 * NX : 0);
+            const long long *rb = HALF ? ra + NX : static_cast<const long long *>(ip[item][1]);
+            if (!HALF && rb) rb += valid ? r * NX : 0;
 #pragma unroll
             for (int e = 0; e < E; ++e) {
                 v[e] = czero<fx2>();
@@ -209,8 +260,33 @@ template <int L, bool INV> __global__ void __launch_bounds__(FXT, 3) k_xfx(const
         sc.template measure<16>(v, 0);
         sc.apply(v, 0, fx_top<L>(0));
         fx_fft<L, false>(v, sm, lay, t, tw, sc);
+        if constexpr (HALF && !INV) {
+            // rows F0, F1 from their sum F0 + i F1 at k and L - k, k = 0..nx
+#pragma unroll
+            for (int e = 0; e < E; ++e) *mine(e) = v[e];
+            __syncwarp();
+            const int ex = sc.ex - 1;   // the halves of the separation
+#pragma unroll 1
+            for (int e = 0; e <= E / 2; ++e) {
+                const int k = t + e * TPC;
+                if (k > NX || !valid) break;
+                const fx2 p = sm[lay(k)], q = sm[lay((L - k) & (L - 1))];
+                fx2 f0, f1;
+                f0.x = p.x + q.x; f0.y = p.y - q.y;
+                f1.x = p.y + q.y; f1.y = q.x - p.x;
+                __stcg(row + k, fx_out<true>(f0, ex));
+                __stcg(row + L + k, fx_out<true>(f1, ex));
+            }
+            if (valid)
+                for (int k = NX + 1 + t; k < kend; k += TPC) {
+                    __stcg(row + k, make_double2(0.0, 0.0));
+                    __stcg(row + L + k, make_double2(0.0, 0.0));
+                }
+            __syncwarp();   // the slots are read before the next rows' exchange
+            continue;
+        }
         bool sum = false;
-        if constexpr (INV) sum = ip[item][0] && !isplit[item];   // Phi_a + Phi_b beside Phi_b
+        if constexpr (INV && !HALF) sum = ip[item][0] && !isplit[item];   // Phi_a + Phi_b beside Phi_b
 #pragma unroll
         for (int e = 0; e < (INV ? E / 2 : E); ++e) {
             if (INV) v[e] = swapped(v[e]);
@@ -220,8 +296,9 @@ template <int L, bool INV> __global__ void __launch_bounds__(FXT, 3) k_xfx(const
         fx_to(INV ? E / 2 : E, sc.ex, mine);
         if (valid) {
             if constexpr (INV) {
-                double *phi_b = static_cast<double *>(ip[item][0]), *phi_s = static_cast<double *>(ip[item][1]) + r * NX;
-                if (phi_b) phi_b += r * NX;
+                double *phi_b = static_cast<double *>(ip[item][0]), *phi_s = static_cast<double *>(ip[item][1]) + r1 * NX;
+                if (HALF) phi_b = phi_s + NX;   // the second row
+                else if (phi_b) phi_b += r * NX;
 #pragma unroll
                 for (int e = 0; e < E / 2; ++e) {   // outputs x < nx
                     const double2 d = *reinterpret_cast<const double2 *>(mine(e));
@@ -248,7 +325,7 @@ template <int L, int MODE> constexpr size_t fx_ysmem() {
                      sizeof(fx2);
 }
 
-template <int L, int MODE> __global__ void __launch_bounds__(FXT, 3) k_yfx(const __grid_constant__ PassBatch B) {
+template <int L, int MODE, bool HALF> __global__ void __launch_bounds__(FXT, 3) k_yfx(const __grid_constant__ PassBatch B) {
     typedef CShape<double, L> S;
     static_assert(S::THREADS == FXT, "tile shape");
     constexpr bool INV = MODE == COL_YINV;
@@ -266,11 +343,22 @@ template <int L, int MODE> __global__ void __launch_bounds__(FXT, 3) k_yfx(const
     const int nx2 = 2 * B.a[0].nx, ny2 = 2 * B.a[0].ny;   // the items' common shape, read once
     const long long tiles_per_z = (nx2 + COLS - 1) / COLS;
     const int ltpz = __ffs((int)tiles_per_z) - 1;
-    const long long ntiles = (long long)B.n << B.lgi, lmask = (1LL << B.lgi) - 1;
-    auto issue = [&](long long tile) {
+    const long long ntiles = HALF ? (long long)B.n * B.tpi : (long long)B.n << B.lgi, lmask = (1LL << B.lgi) - 1;
+    auto coords = [&](long long tile, int &x, int &y) {   // and the item
+        if (HALF) {
+            const int item = (int)tile / B.tpi, lt = (int)tile - item * B.tpi, z = lt / B.tpr;
+            x = (lt - z * B.tpr) * COLS * S::EPC;
+            y = z * ny2;
+            return item;
+        }
         const long long lt = tile & lmask;
-        const int x = (int)((lt & (tiles_per_z - 1)) * COLS * S::EPC), y = (int)((lt >> ltpz) * ny2);
-        const CUtensorMap *map = &B.lmap[tile >> B.lgi];
+        x = (int)((lt & (tiles_per_z - 1)) * COLS * S::EPC);
+        y = (int)((lt >> ltpz) * ny2);
+        return (int)(tile >> B.lgi);
+    };
+    auto issue = [&](long long tile) {
+        int x, y;
+        const CUtensorMap *map = &B.lmap[coords(tile, x, y)];
         mbar_expect_tx(&bar, (unsigned)(ROWS * COLS * sizeof(fx2)));
 #pragma unroll
         for (int k = 0; k < NBOX; ++k) tma_load_2d(in + k * BOXR * COLS, map, x, y + k * BOXR, &bar);
@@ -335,9 +423,8 @@ template <int L, int MODE> __global__ void __launch_bounds__(FXT, 3) k_yfx(const
         fence_async_smem();   // the staged outputs are visible to the tensor copies
         __syncthreads();
         if (tid == 0) {
-            const long long lt = tile & lmask;
-            const int x = (int)((lt & (tiles_per_z - 1)) * COLS * S::EPC), y = (int)((lt >> ltpz) * ny2);
-            const CUtensorMap *smap = &B.smap[tile >> B.lgi];
+            int x, y;
+            const CUtensorMap *smap = &B.smap[coords(tile, x, y)];
 #pragma unroll
             for (int k = 0; k < OROWS / OBOX; ++k) tma_store_2d(smap, x, y + k * OBOX, sm + k * OBOX * COLS);
             bulk_commit();
@@ -357,7 +444,7 @@ template <int L, int DM> constexpr size_t fx_zsmem() {
            (size_t)pmfft::tw_dir_size(L, false) * sizeof(fxw);
 }
 
-template <int L, int DM>
+template <int L, int DM, bool HALF>
 __global__ void __launch_bounds__(FXT, DM == 2 ? 2 : 3) k_zfx(const __grid_constant__ PassBatch B) {
     typedef WShape<double, L> S;
     static_assert(S::THREADS == FXT, "tile shape");
@@ -372,23 +459,33 @@ __global__ void __launch_bounds__(FXT, DM == 2 ? 2 : 3) k_zfx(const __grid_const
     const int t = lane % TPC, c = warp * (32 / TPC) + lane / TPC;   // column within the tile
     const PairArgs &a = B.a[0];   // the shape, tables and mode are the items' common ones
     const int nx2 = 2 * a.nx, ny2 = 2 * a.ny, lnx2 = __ffs(nx2) - 1;
-    const int lgi = B.lgi, lmask = (1 << lgi) - 1, nt = B.n << lgi;
+    const int lgi = B.lgi, lmask = (1 << lgi) - 1, nt = HALF ? B.n * B.tpi : B.n << lgi;
+    auto locate = [&](int tile, int &q0) {   // first column, and the item
+        if (HALF) {
+            const int item = tile / B.tpi, lt = tile - item * B.tpi, ky = lt / B.tpr;
+            q0 = (ky << lnx2) + (lt - ky * B.tpr) * S::COLS;
+            return item;
+        }
+        q0 = (tile & lmask) * S::COLS;
+        return tile >> lgi;
+    };
     auto issue_load = [&](int tile, int b) {
-        const CUtensorMap *map = &B.lmap[tile >> lgi];
+        int q0;
+        const CUtensorMap *map = &B.lmap[locate(tile, q0)];
         mbar_expect_tx(&full[b], S::BUF);
 #pragma unroll
         for (int s = 0; s < S::NSUB; ++s)
 #pragma unroll
             for (int k = 0; k < S::NBOXI; ++k)
                 tma_load_2d(base + b * S::BUF + s * S::RIN * S::P + k * S::BOXI * S::P, map,
-                            (int)(((tile & lmask) * S::COLS + s * S::SW) * S::EPC), k * S::BOXI, &full[b]);
+                            (q0 + s * S::SW) * S::EPC, k * S::BOXI, &full[b]);
     };
-    auto issue_store = [&](int tile, const unsigned char *src, const CUtensorMap *map) {
+    auto issue_store = [&](int q0, const unsigned char *src, const CUtensorMap *map) {
 #pragma unroll
         for (int s = 0; s < S::NSUB; ++s)
 #pragma unroll
             for (int k = 0; k < S::NBOXI; ++k)
-                tma_store_2d(map, (int)(((tile & lmask) * S::COLS + s * S::SW) * S::EPC), k * S::BOXI,
+                tma_store_2d(map, (q0 + s * S::SW) * S::EPC, k * S::BOXI,
                              src + s * S::RIN * S::P + k * S::BOXI * S::P);
     };
     __shared__ const double *ihhat[PM_BATCH];
@@ -435,10 +532,11 @@ __global__ void __launch_bounds__(FXT, DM == 2 ? 2 : 3) k_zfx(const __grid_const
             issue_load(tile + (int)gridDim.x, b ^ 1);
             ++issued[b ^ 1];
         }
-        const int q = (tile & lmask) * S::COLS + c;   // the column
+        int q0;
+        const int item = locate(tile, q0), q = q0 + c;   // the column
         const int ky = q >> lnx2, kx = q & (nx2 - 1);
         const int kyr = ky <= a.ny ? ky : ny2 - ky, kxr = kx <= a.nx ? kx : nx2 - kx;
-        const double *hcol = ihhat[tile >> lgi] + ((size_t)kyr * (a.nx + 1) + kxr) * S::HS;
+        const double *hcol = ihhat[item] + ((size_t)kyr * (a.nx + 1) + kxr) * S::HS;
         auto slot_of = [&](int e) { return in + woff<double, L, S::RIN>(t + e * TPC, c); };
         // H-hat of row kz (pm_build_hhat's order): register e of the last
         // stage's order holds row kz, entry t * 16 + e of a thread-major table
@@ -487,7 +585,7 @@ __global__ void __launch_bounds__(FXT, DM == 2 ? 2 : 3) k_zfx(const __grid_const
                 const bool last = DM != 2 || j == 2;
                 if (tid == 0) {
                     // DM = 2: fx + i fy through smap, then fz + i Phi in place through lmap
-                    issue_store(tile, in, DM == 2 && last ? &B.lmap[tile >> lgi] : &B.smap[tile >> lgi]);
+                    issue_store(q0, in, DM == 2 && last ? &B.lmap[item] : &B.smap[item]);
                     bulk_commit();
                     if (!last) bulk_wait_read();   // read out before the second outputs overwrite the buffer
                 }

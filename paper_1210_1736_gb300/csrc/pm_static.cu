@@ -143,16 +143,20 @@ int run(const int64_t *rho, void *phi, int nx, int ny, int nz, double l_xy, doub
     a.nx = nx; a.ny = ny; a.nz = nz;
     a.scale = std::ldexp(1.0, -shift);
     a.err = err;
+    auto half = [&](PassBatch b) {   // one real set: half its spectrum
+        b.kend = pm_half_cols(nx, ny, nz, (int)sizeof(T));
+        return b;
+    };
     a.tw = twx;
-    SCK(pm_launch_xfwd<T>(pm_single_batch(a, nullptr, nullptr), st));
+    SCK(pm_launch_xfwd<T>(half(pm_single_batch(a, nullptr, nullptr)), st));
     a.tw = twy;
-    SCK(pm_launch_col<T>(pm_single_batch(a, &yfwd, &yinv), COL_YFWD, st));
+    SCK(pm_launch_col<T>(half(pm_single_batch(a, &yfwd, &yinv)), COL_YFWD, st));
     a.tw = twz;
-    SCK(pm_launch_col<T>(pm_single_batch(a, &zmap, nullptr), COL_ZCONV, st));
+    SCK(pm_launch_col<T>(half(pm_single_batch(a, &zmap, nullptr)), COL_ZCONV, st));
     a.tw = twy;
-    SCK(pm_launch_col<T>(pm_single_batch(a, &yinv, &yfwd), COL_YINV, st));
+    SCK(pm_launch_col<T>(half(pm_single_batch(a, &yinv, &yfwd)), COL_YINV, st));
     a.tw = twx;
-    SCK(pm_launch_xinv<T>(pm_single_batch(a, nullptr, nullptr), st));
+    SCK(pm_launch_xinv<T>(half(pm_single_batch(a, nullptr, nullptr)), st));
     SCK(launch_settle<T>(err, status, phi, (long long)nx * ny * nz, st));
 #undef SCK
     return PM_OK;
