@@ -6,9 +6,10 @@
 // transform of length L = 2n of the even extension of n + 1 values.  Two
 // columns travel as one complex transform (both results are real) in the fixed
 // point of pm_fx.cuh; the first axis evaluates H, the last writes the table.
-// For 128 x 128 x 32 in FP32 the three launches take 31, 15 and 17 us (the
-// first bound by H's FP64 operations) where H took 22 us, dense FP64 cosine
-// sums, bound by the FP64 pipe, 125 + 127 + 35 us and the table 9 us.  H-hat
+// For 128 x 128 x 32 in FP32 the three launches take 22, 15 and 17 us (the
+// first bound by H's FP64 operations: 31 us before the ones that integer or FP32
+// operations replace exactly were taken out) where H took 22 us, dense FP64
+// cosine sums, bound by the FP64 pipe, 125 + 127 + 35 us and the table 9 us.  H-hat
 // is also more exact: the FP64 potentials' error fell to a half or a third.
 #include <cuda_runtime.h>
 
@@ -29,11 +30,18 @@ struct HatArgs {
     double q, h000, scale;
 };
 
-// 1/sqrt(r2): an FP32 seed and one third-order step (relative error about
-// 2^-52, as the quotient by a rounded root; a third of the FP64 operations).
-__device__ __forceinline__ double inv_sqrt(double r2) {
-    if (!(r2 > 1e-30 && r2 < 1e30)) return 1.0 / sqrt(r2);
-    const double y = (double)rsqrtf((float)r2);
+// The FP64 value of a normal FP32 one by integer operations (the conversion
+// takes a slot of the FP64 pipe).
+__device__ __forceinline__ double widen(float f) {
+    const unsigned b = __float_as_uint(f);   // f > 0
+    return __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
+}
+// 1/sqrt(r2), r2 known to FP32 as rf: an FP32 seed and one third-order step
+// (relative error about 2^-52, as the quotient by a rounded root; a third of
+// the FP64 operations).
+__device__ __forceinline__ double inv_sqrt(double r2, float rf) {
+    if (!(rf > 1e-30f && rf < 1e30f)) return 1.0 / sqrt(r2);
+    const double y = widen(rsqrtf(rf));
     const double e = fma(-(r2 * y), y, 1.0);
     return fma(y * e, fma(0.375, e, 0.5), y);
 }
@@ -58,19 +66,30 @@ template <int L, int AX, typename T> __global__ void __launch_bounds__(pmk::FXT,
     // rows t + e TPC <= N of the two columns
     auto mine = [&](int e) { return sm + lay(t + e * TPC); };
     const int cnt = t == 0 ? E / 2 + 1 : E / 2;
+    // first axis: a column's squared distance from the axis in its two parts
+    int jj[2] = {0, 0};
+    double kk[2] = {0.0, 0.0};
+    if constexpr (AX == 0)
+#pragma unroll
+        for (int w = 0; w < 2; ++w) {
+            const int c = (int)col + w, k = c / a.ny1, j = c - k * a.ny1;
+            const double qk = a.q * (double)k;
+            jj[w] = j * j;
+            kk[w] = qk * qk;
+        }
+    const float kf[2] = {(float)kk[0], (float)kk[1]};
     unsigned m = 0;
 #pragma unroll 3
     for (int e = 0; e < cnt; ++e) {
         const int i = t + e * TPC;
         double2 d = make_double2(0.0, 0.0);
         if constexpr (AX == 0) {
-            auto green = [&](long long c) {
-                const int j = (int)(c % a.ny1), k = (int)(c / a.ny1);
-                const double qk = a.q * (double)k;
-                return c == 0 && i == 0 ? a.h000 : inv_sqrt((double)(i * i + j * j) + qk * qk);
+            auto green = [&](int w) {
+                const int n = i * i + jj[w];   // exact in FP32
+                return i == 0 && col + w == 0 ? a.h000 : inv_sqrt((double)n + kk[w], (float)n + kf[w]);
             };
-            if (va) d.x = green(col);
-            if (vb) d.y = green(col + 1);
+            if (va) d.x = green(0);
+            if (vb) d.y = green(1);
         } else {
             if (va) d.x = ha[i * stride];
             if (vb) d.y = hb[i * stride];
