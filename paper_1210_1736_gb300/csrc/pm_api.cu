@@ -755,17 +755,33 @@ template <typename T> int step_timed_impl(pm_ctx *c, const pm_particles *p, doub
 
 // ---- CIC variant (differentiable runs) -------------------------------------
 // The particles' spatial order at their current positions, for the CIC kernels
-// (unsorted, their atomics and gathers touch a cache line each).  The calls after a deposit run in the deposit's order: results
-// depend on no order, so for other particles of the same number it is only a
-// worse one.
+// (unsorted, their atomics and gathers touch a cache line each).  The calls
+// after a deposit run in the deposit's order: results depend on no order, so
+// for other particles of the same number it is only a worse one.  Captured
+// calls, which may neither allocate nor rely on a later state of the scratch,
+// and calls without memory for it run in the stored order.
 constexpr long long CIC_ORDER_MIN = 1LL << 16, CIC_ORDER_MAX = 1LL << 32;
+bool capturing(const pm_ctx *c) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->user, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
 template <typename T> int cic_order(pm_ctx *c, const pm_particles *p) {
+    if (capturing(c)) return PM_OK;
     c->ord_n = 0;
     if (p->n < CIC_ORDER_MIN || p->n >= CIC_ORDER_MAX) return PM_OK;
     if (p->n > c->ord_cap) {
-        PM_TRY(dev_alloc(c, (void **)&c->o_key, (size_t)p->n * 4));
-        PM_TRY(dev_alloc(c, (void **)&c->o_rank, (size_t)p->n * 4));
-        PM_TRY(dev_alloc(c, (void **)&c->o_ord, (size_t)p->n * 4));
+        void *a = nullptr;   // key, rank and order
+        if (cudaMalloc(&a, (size_t)p->n * 12) != cudaSuccess) {
+            cudaGetLastError();
+            return PM_OK;
+        }
+        c->allocs.push_back(a);
+        c->bytes += (size_t)p->n * 12;
+        c->o_key = (unsigned *)a;
+        c->o_rank = c->o_key + p->n;
+        c->o_ord = c->o_rank + p->n;
         c->ord_cap = p->n;
     }
     PM_CK(pm_launch_order<T>(part_k<T>(p), c->hs, c->d_cen, c->sortk, c->s_count, c->o_key, c->o_rank, c->s_bsum,
@@ -773,7 +789,9 @@ template <typename T> int cic_order(pm_ctx *c, const pm_particles *p) {
     c->ord_n = p->n;
     return PM_OK;
 }
-const unsigned *cic_ord(const pm_ctx *c, const pm_particles *p) { return c->ord_n == p->n ? c->o_ord : nullptr; }
+const unsigned *cic_ord(const pm_ctx *c, const pm_particles *p) {
+    return c->ord_n == p->n && c->ord_n > 0 && !capturing(c) ? c->o_ord : nullptr;
+}
 
 template <typename T> int cic_deposit_impl(pm_ctx *c, const pm_particles *p) {
     PM_TRY(cic_order<T>(c, p));

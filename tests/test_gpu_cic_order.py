@@ -93,3 +93,38 @@ def test_other_particles_of_the_same_number():
     sub = pm.Particles(cast(v, v["pos"])[:, :k], cast(v, v["vel"])[:, :k], m[:k], v["gal"][:k])
     b = torch.stack(ctx2.cic_force(sub))
     assert torch.equal(a[:, :k], b)
+
+
+def test_captured_calls_keep_the_stored_order():
+    """A captured deposit allocates nothing and its replay gives the ordered
+    deposit's densities; a call between capture and replay does not use an
+    order that no launch has written."""
+    import torch
+    n = 1 << 16
+    w = _case("fp32", n, False)
+    m = cast(w, w["m"])
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        ctx = pm.Context(w, W.mass_bound(m))
+        p = pm.Particles(cast(w, w["pos"]), cast(w, w["vel"]), m, w["gal"])
+        s.synchronize()
+        size = ctx.info()["bytes"]
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            ctx.cic_deposit(p)
+        assert ctx.info()["bytes"] == size
+        ctx.solve()
+        before = torch.stack(ctx.cic_force(p))   # of empty densities
+        g.replay()
+        captured = {k: ctx.density(*k) for k in ctx.shapes}
+        ctx.solve()
+        a = torch.stack(ctx.cic_force(p))
+        ctx.cic_deposit(p)
+        assert ctx.info()["bytes"] == size + 12 * n
+        assert all(np.array_equal(captured[k], ctx.density(*k)) for k in ctx.shapes)
+        ctx.solve()
+        b = torch.stack(ctx.cic_force(p))
+        s.synchronize()
+    assert not before.any()
+    assert a.any() and torch.equal(a, b)
+    ctx.close()
