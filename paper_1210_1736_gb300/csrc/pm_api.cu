@@ -1,7 +1,7 @@
 // C ABI of the nested-grid particle-mesh step (declared in include/pm.h).
 //
 // The context owns every grid buffer: per galaxy and mass set an int64
-// density, an FP32/FP64 spectrum work buffer ([z][y in 2ny][kx in nx+1]) and
+// density, an FP32/FP64 spectrum work buffer ([z][y in 2ny][kx in 2nx]) and
 // the potential; per distinct geometry the H-hat octant.  Particle arrays are
 // the caller's.  All work is ordered on the caller's stream; pm_step replays a
 // CUDA graph of one full step captured on a private stream.

@@ -6,10 +6,11 @@
 // (x and z passes) or a tile (y passes) shares one exponent, a value is
 // x 2^ex with a 64-bit integer x, additions are exact and a complex product
 // with a 60-bit twiddle takes 12 32x32+64-bit multiply-adds.  Before every
-// radix-16 stage the values are shifted so that the largest component fills
-// FX_K bits, the most for which the stage cannot overflow, so the rounding of
-// a stage is below 2^-55 of the largest component of the warp or tile, less
-// than the 2^-53 per operation of FP64 arithmetic.  Work arrays, H-hat and
+// radix-16 stage the values are shifted so that the largest sum of magnitudes
+// that one butterfly combines fills FX_TOP bits, the most for which the stage
+// cannot overflow, so the rounding of a stage is below 2^-55 of the largest
+// component of the warp or tile, less than the 2^-53 per operation of FP64
+// arithmetic.  Work arrays, H-hat and
 // potentials stay FP64 in memory.
 #pragma once
 

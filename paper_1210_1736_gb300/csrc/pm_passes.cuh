@@ -3,7 +3,9 @@
 // sets: two real densities of one geometry (grids 2 and 3, or 4 and 5) travel
 // as one complex field rho_a + i rho_b, so every transform is a plain complex
 // FFT of power-of-two length and, H being real, the result is
-// Phi_a + i Phi_b.  A set without partner uses rho_b = 0.
+// Phi_a + i Phi_b.  A set without partner is transformed by half its spectrum
+// (HALF: two rows as one complex row, columns kx < kend; see pm_half_cols),
+// or, as grid 1's difference fields need it, whole with rho_b = 0.
 //
 // Work array per pair: complex [z < nz][y < 2ny][kx < 2nx].
 //   x forward : rows (z, y < ny), inputs x < nx (zero padding implicit)
@@ -23,7 +25,7 @@
 // memory (y passes: one buffer, free once the inputs are in registers; z: two,
 // the next but one) while the block transforms the current one; every column
 // pass stages its outputs in shared memory and sends them by TMA store.  (A
-// second buffer cost the 512-point y forward 11 %: 463 us against 411 on the
+// second buffer cost the 512-point y forward 11 %: 463 us against 409 on the
 // 16.5M-particle step's grids; nothing at 256.)
 #pragma once
 

@@ -3,7 +3,8 @@
 // are the same; what differs is the arithmetic and the shape of the code.
 //
 // Bound by integer instructions (a 1M-particle galaxy's y forward: ALU pipe 64 %,
-// IMAD.WIDE pipe 50 %, issue 57 %, DRAM 20 %), after the instruction cache:
+// IMAD.WIDE pipe 50 %, issue 57 %, DRAM 20 %; its 256-point z pass: 53, 50, 52
+// and 9 %), after the instruction cache:
 // unrolled like the FP32 passes a z pass was 180 KB of code and its warps
 // waited for instructions.  So every transform runs the one forward plan (an
 // inverse swaps the components going in and coming out), equal stages share a
@@ -13,8 +14,8 @@
 // (128 registers) and two measured the same.
 //
 // One step of the 1M-particle galaxy (128^3, 128^3, 128x128x32 grids), FP64
-// arithmetic -> this: x forward 452 -> 112 us, y forward 826 -> 209, z 3381 ->
-// 950, y inverse 942 -> 239, x inverse 497 -> 139.  Error of the potential
+// arithmetic -> this: x forward 452 -> 120 us, y forward 826 -> 211, z 3381 ->
+// 921, y inverse 942 -> 240, x inverse 497 -> 143.  Error of the potential
 // against 80-bit arithmetic on grids of 16^3 to 64^3 and 256x16x64: 0.6-1.0
 // times that of the FP64 transforms.
 #pragma once
