@@ -137,6 +137,17 @@ template <int N> __device__ __forceinline__ void shift(fx2 *v, int s) {
     }
 }
 
+// shift for integers of all 64 bits (the rounding bit is added after the
+// shift: 2^(s-1) added before it would wrap within that of 2^63).
+template <int N> __device__ __forceinline__ void shift_full(fx2 *v, int s) {
+    if (s <= 0) return shift<N>(v, s);
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+        v[e].x = (v[e].x >> s) + ((v[e].x >> (s - 1)) & 1);
+        v[e].y = (v[e].y >> s) + ((v[e].y >> (s - 1)) & 1);
+    }
+}
+
 // FP64 <-> fixed point by integer operations (the conversions run on the FP64
 // pipe too).  hi word without sign: orders like |d|.
 __device__ __forceinline__ unsigned dmag(double d) { return (unsigned)__double2hiint(d) & 0x7fffffffu; }

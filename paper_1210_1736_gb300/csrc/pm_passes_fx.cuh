@@ -255,7 +255,7 @@ template <int L, bool INV, bool HALF> __global__ void __launch_bounds__(FXT, 3) 
             }
             // densities of any size to 59 bits (the sums below see only values beyond 2^32)
             const int sh = pmfx::warp_bits<E / 2>(v) - (pmfx::FX_TOP - 1);
-            pmfx::shift<E / 2>(v, sh);
+            pmfx::shift_full<E / 2>(v, sh);
             sc.ex += sh;
         }
         sc.template measure<16>(v, 0);

@@ -83,3 +83,33 @@ def test_mass_range(shape, heavy):
     # both sides round the stored passes and numpy's every operation: a few
     # units of 2^-53 of the largest value
     assert np.abs(p - ref).max() <= 16 * 2.0 ** -53 * np.abs(ref).max()
+
+
+def _static(rho, shape, shift=50, G=1.0, h000=1.0, precision=pm.PM_FP64):
+    """pm_potential_static of a host int64 density [z][y][x]."""
+    import torch
+    nx, ny, nz = shape
+    r = torch.tensor(rho, device="cuda")
+    phi = torch.empty(nz, ny, nx, device="cuda", dtype=torch.float64 if precision == pm.PM_FP64 else torch.float32)
+    st = torch.cuda.current_stream().cuda_stream
+    pm._check(pm.lib().pm_potential_static(r.data_ptr(), phi.data_ptr(), nx, ny, nz, 0.5, 0.25, G, h000, shift, precision, st))
+    pm._check(pm.lib().pm_potential_static_status(st))
+    return phi.cpu().numpy()
+
+
+@pytest.mark.parametrize("shape", [(16, 16, 16), (64, 32, 32)])   # whole and half spectra
+@pytest.mark.parametrize("near", [0, 3, 7, 8, 9, 40])
+@pytest.mark.parametrize("sign", [1, -1])
+def test_densities_up_to_the_integer_limits(shape, near, sign):
+    """Cells within a rounding unit of +-2^63, alone and beside small ones."""
+    nx, ny, nz = shape
+    rng = np.random.default_rng(4)
+    rho = rng.integers(-2 ** 40, 2 ** 40, size=(nz, ny, nx))
+    big = rho.copy()
+    for cell in ((0, 0, 0), (3, 5, 7), (nz - 1, ny - 1, nx - 1)):
+        big[cell] = 2 ** 63 - 1 - near if sign > 0 else -2 ** 63 + near
+    # the same to a relative 2^-59: heavy cells of 2^62, twice, as the potential is linear
+    heavy = np.where(big == rho, 0, sign * 2 ** 62)
+    a, b = _static(big, shape), 2.0 * _static(heavy, shape) + _static(np.where(big == rho, rho, 0), shape)
+    # three potentials, each within 16 units of 2^-53 of the largest value (see test_mass_range)
+    assert np.abs(a - b).max() <= 48 * 2.0 ** -53 * np.abs(b).max()
