@@ -20,6 +20,10 @@
  *     unless stated; only the pm_get_* and pm_diagnostics calls synchronise.
  *   - Every call returns PM_OK (0) or a negative PM_E_* status and never
  *     throws; pm_last_error() gives a message for the calling thread.
+ *   - Potentials of PM_FP64 contexts carry a full 53 bits where masses, H-hat
+ *     and results lie above about 2^-958; towards the least FP64 numbers the
+ *     unit of every intermediate stays at 2^-1018 and results below 2^-1022
+ *     are zero.
  *   - Particles flagged lost (PM_FLAG_LOST) contribute nothing and are not
  *     moved; the flag is set by pm_deposit and never cleared by the library.
  */

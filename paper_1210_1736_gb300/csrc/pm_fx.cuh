@@ -188,10 +188,17 @@ __device__ __forceinline__ unsigned warp_max(unsigned m) { return __reduce_max_s
 // Exponent of values that held an infinity or a NaN (they come out as NaN).
 constexpr int FX_NAN = 1 << 16;
 constexpr int FX_LOW = -(1 << 16);   // below every exponent
-// em and ex of a group whose largest dmag is m, converted with K bits.  A
-// group below 2^-958 vanishes (em beyond every shift).
-__device__ __forceinline__ int group_em(unsigned m) { return (int)(m >> 20) > 64 ? (int)(m >> 20) : 1 << 13; }
-__device__ __forceinline__ int group_ex(int em, int K) { return em == 0x7ff ? FX_NAN : em > 0x7ff ? -900 : em - 1022 - K; }
+constexpr int FX_ZERO = -900;        // the exponent given to zeros
+// em and ex of a group whose largest dmag is m, converted with K bits.  em is
+// at least 64, so that a zero, whose implicit bit from_double does not mask, is
+// shifted out: the unit of a group below 2^-958 stays at 2^(-958 - K), and what
+// is below it vanishes.  A group of zeros: em beyond every shift.
+__device__ __forceinline__ int group_em(unsigned m) {
+    const int e = (int)(m >> 20);
+    return e > 64 ? e : m ? 64 : 1 << 13;
+}
+__device__ __forceinline__ bool group_zero(int em) { return em > 0x7ff; }
+__device__ __forceinline__ int group_ex(int em, int K) { return em == 0x7ff ? FX_NAN : group_zero(em) ? FX_ZERO : em - 1022 - K; }
 
 }  // namespace pmfx
 

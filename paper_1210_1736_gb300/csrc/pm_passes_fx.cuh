@@ -402,9 +402,10 @@ template <int L, int MODE, bool HALF> __global__ void __launch_bounds__(FXT, 3) 
             v[e] = czero<fx2>();
             if (e < NIN) v[e] = INV ? swapped(*at(e)) : *at(e);
         }
+        // (a warp of zeros, e.g. beyond the grid's columns, has no say in it)
         FxScale<true> sc{pmfx::group_ex(em, pmfx::FX_TOP), sl, 0};
         sc.m = pmfx::warp_max(pmfx::group_sum<16>(v));
-        if ((tid & 31) == 0) atomicMax(sl, sc.ex + pmfx::sum_shift(sc.m, fx_top<L>(0)));
+        if ((tid & 31) == 0 && !pmfx::group_zero(em)) atomicMax(sl, sc.ex + pmfx::sum_shift(sc.m, fx_top<L>(0)));
         fence_async_smem();                // the buffer's conversions before the next load's writes
         if (tid == 0) bulk_wait_read();    // the previous tile's outputs have been read out of sm
         __syncthreads();
@@ -413,8 +414,9 @@ template <int L, int MODE, bool HALF> __global__ void __launch_bounds__(FXT, 3) 
             issue(tile + gridDim.x);
         }
         if (tid < 4) slot[(it & 1) ^ 1][tid] = tid ? 0 : pmfx::FX_LOW;   // last read before the barrier
-        pmfx::shift<E>(v, sl[0] - sc.ex);
-        sc.ex = sl[0];
+        const int tex = sl[0] == pmfx::FX_LOW ? pmfx::FX_ZERO : sl[0];
+        if (!pmfx::group_zero(em)) pmfx::shift<E>(v, tex - sc.ex);
+        sc.ex = tex;
         fx_fft<L, true>(v, sm, lay, t, tw, sc);
         // fx_fft leaves the exchange buffer free: the outputs, rows t + e TPC
         auto to = [&](int e) { return sm + (t + e * TPC) * COLS + c; };

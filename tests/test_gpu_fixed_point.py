@@ -113,3 +113,26 @@ def test_densities_up_to_the_integer_limits(shape, near, sign):
     a, b = _static(big, shape), 2.0 * _static(heavy, shape) + _static(np.where(big == rho, rho, 0), shape)
     # three potentials, each within 16 units of 2^-53 of the largest value (see test_mass_range)
     assert np.abs(a - b).max() <= 48 * 2.0 ** -53 * np.abs(b).max()
+
+
+# tiles wider than the grid (their warps beyond it hold zeros), whole and half spectra
+@pytest.mark.parametrize("shape", [(16, 16, 16), (8, 16, 8), (16, 8, 8), (64, 32, 32), (8, 64, 16)])
+@pytest.mark.parametrize("G,shift", [(-880, 50), (-925, 50), (-960, 50), (-975, 50), (900, 1000), (-960, -20)])
+def test_small_magnitudes(shape, G, shift):
+    """Green's functions and masses towards the least FP64 exponents: the
+    potential is that of G = 1 and shift = 50, scaled."""
+    nx, ny, nz = shape
+    rho = np.random.default_rng(6).integers(0, 2 ** 45, size=(nz, ny, nx))
+    a = _static(rho, shape)
+    k = G + 50 - shift   # the power of two between the two
+    b = _static(rho, shape, shift=shift, G=2.0 ** G)
+    assert b.any()
+    # Every conversion's unit is at most 2^-1018 where a group lies that low: of
+    # H-hat (times the sum of masses, for each of the 8N modes), of the masses'
+    # spectra (times the sum of H-hat, 8N H(0), H(0) below 4N G) and of the
+    # potential's (8N values summed twice)
+    N8, M, g = 8.0 * rho.size, float(rho.sum()) * 2.0 ** -shift, 2.0 ** G
+    unit = N8 * (M + 4 * g * N8 + 2) * 2.0 ** -1018
+    tol = unit + 64 * 2.0 ** -53 * np.ldexp(np.abs(a).max(), k)
+    print(f"tolerance {tol / np.ldexp(np.abs(a).max(), k):.1e} of the largest value")
+    assert np.abs(b - np.ldexp(a, k)).max() <= tol
