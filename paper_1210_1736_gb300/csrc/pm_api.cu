@@ -39,9 +39,11 @@ int fail(int code, const char *fmt, ...) {
 #define PM_CK(call)                                                                                  \
     do {                                                                                             \
         cudaError_t e_ = (call);                                                                     \
-        if (e_ != cudaSuccess)                                                                       \
+        if (e_ != cudaSuccess) {                                                                     \
+            cudaGetLastError(); /* reported here: not by the next launch */                          \
             return fail(PM_E_CUDA, "%s failed: %s (%s:%d)", #call, cudaGetErrorString(e_), __FILE__, \
                         __LINE__);                                                                   \
+        }                                                                                            \
     } while (0)
 
 #define PM_TRY(expr)               \
@@ -215,7 +217,10 @@ namespace {
 int dev_alloc(pm_ctx *c, void **p, size_t bytes) {
     if (bytes == 0) bytes = 16;
     cudaError_t e = cudaMalloc(p, bytes);
-    if (e != cudaSuccess) return fail(PM_E_CUDA, "cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(PM_E_CUDA, "cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
+    }
     c->allocs.push_back(*p);
     c->bytes += bytes;
     return PM_OK;
