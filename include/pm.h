@@ -231,6 +231,12 @@ int pm_set_launch_config(pm_ctx *ctx, int32_t batched, int32_t schedule);
  * call is the expected result, not a failure. */
 int pm_selftest_wait_expiry(pm_ctx *ctx);
 
+/* Test hook: scratch that calls keep only while memory allows (the particles'
+ * part of pm_disc_diagnostics) is refused from now on beyond `bytes` (negative:
+ * no limit, the default); results do not depend on it beyond the order of
+ * FP64 sums. */
+int pm_selftest_scratch_limit(pm_ctx *ctx, int64_t bytes);
+
 /* Spatial sort (no counterpart in the paper; a locality optimisation of the
  * NGP assignment of Eq. eqn:cell): permutes every particle array of p in
  * place so that particles are ordered by galaxy, region (core, shell,
@@ -316,8 +322,9 @@ int pm_cic_vjp(pm_ctx *ctx, const pm_particles *p, const void *ux, const void *u
  * out (host, 6 + 4 nbins + 2 nring mmax doubles): [n, E_heat, sigma_R,
  * sigma_phi, sigma_z, annulus mass, then per bin (mean R, count,
  * sqrt<z^2>, mean v_phi), then per ring and mode (Re A~_m, Im A~_m)].
- * Synchronises; allocates its scratch (0.5 MB and 48 bytes per particle) on
- * the first call and when n grows. */
+ * Synchronises; allocates its scratch (0.6 MB and 48 bytes per particle) on
+ * the first call and when n grows (the outgrown part is released).  Without
+ * memory for the particles' part it reads the particles in every pass. */
 typedef struct {
     int32_t gal;
     int32_t nbins;

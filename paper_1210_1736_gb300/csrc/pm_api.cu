@@ -151,6 +151,12 @@ struct ShapeGroup {
     std::vector<int> geos;
 };
 
+// A buffer that a call keeps for the next one while memory allows.
+struct Scratch {
+    void *p = nullptr;
+    size_t bytes = 0;
+};
+
 }  // namespace
 
 struct pm_ctx {
@@ -206,10 +212,10 @@ struct pm_ctx {
     size_t bytes = 0;
     std::vector<void *> allocs;
     bool any_recentre = false;
-    // disc diagnostics scratch (allocated on first use, the particles' part
-    // grown as needed)
+    // disc diagnostics: fixed part (allocated on first use), particles' part
     pmk::DiagBuf dg = {};
-    long long dg_cap = 0;
+    Scratch dg_part;
+    long long scratch_limit = -1;   // bytes a Scratch may hold (tests; < 0: no limit)
 };
 
 namespace {
@@ -224,6 +230,25 @@ int dev_alloc(pm_ctx *c, void **p, size_t bytes) {
     c->allocs.push_back(*p);
     c->bytes += bytes;
     return PM_OK;
+}
+
+// At least `bytes` of s, or null, without an error, where there is no memory
+// for them: the caller has a way without.  An outgrown buffer is released
+// first (cudaFree waits for the kernels that use it).
+void *keep_scratch(pm_ctx *c, Scratch &s, size_t bytes) {
+    if (bytes <= s.bytes) return s.p;
+    cudaFree(s.p);
+    c->bytes -= s.bytes;
+    s = Scratch();
+    if (c->scratch_limit >= 0 && bytes > (size_t)c->scratch_limit) return nullptr;
+    if (cudaMalloc(&s.p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        s.p = nullptr;
+        return nullptr;
+    }
+    s.bytes = bytes;
+    c->bytes += bytes;
+    return s.p;
 }
 
 int tw_index(int L) {
@@ -865,16 +890,18 @@ template <typename T> int disc_impl(pm_ctx *c, const pm_particles *p, const uint
                                     double *out) {
     cudaStream_t st = c->user;
     if (!c->dg.acc) {
-        PM_TRY(dev_alloc(c, (void **)&c->dg.state, sizeof(pmk::DiagState)));
-        PM_TRY(dev_alloc(c, (void **)&c->dg.hist, sizeof(unsigned) * 2048 * DG_MAXBINS));
-        PM_TRY(dev_alloc(c, (void **)&c->dg.acc, sizeof(double) * (4 * DG_MAXBINS + 8 + 2 * DG_MAXRM)));
+        constexpr size_t hist = sizeof(unsigned) * 2048 * DG_MAXBINS, state = (sizeof(pmk::DiagState) + 255) & ~(size_t)255;
+        unsigned char *m = nullptr;
+        PM_TRY(dev_alloc(c, (void **)&m, hist + state + sizeof(double) * (4 * DG_MAXBINS + 8 + 2 * DG_MAXRM)));
+        c->dg.hist = (unsigned *)m;
+        c->dg.state = (pmk::DiagState *)(m + hist);
+        c->dg.acc = (double *)(m + hist + state);
     }
-    if (p->n > c->dg_cap) {
-        PM_TRY(dev_alloc(c, (void **)&c->dg.key, sizeof(unsigned long long) * p->n));
-        PM_TRY(dev_alloc(c, (void **)&c->dg.idx, sizeof(long long) * p->n));
-        PM_TRY(dev_alloc(c, (void **)&c->dg.rest, sizeof(double4) * p->n));
-        c->dg_cap = p->n;
-    }
+    // per particle: rest (32 bytes), key and index; without memory for them
+    // every pass reads the particles instead
+    c->dg.rest = (double4 *)keep_scratch(c, c->dg_part, (size_t)p->n * 48);
+    c->dg.key = c->dg.rest ? (unsigned long long *)(c->dg.rest + p->n) : nullptr;
+    c->dg.idx = c->dg.rest ? (long long *)(c->dg.key + p->n) : nullptr;
     pmk::DiagP<T> d;
     d.x = (const T *)p->x; d.y = (const T *)p->y; d.z = (const T *)p->z;
     d.vx = (const T *)p->vx; d.vy = (const T *)p->vy; d.vz = (const T *)p->vz;
@@ -1283,6 +1310,7 @@ void pm_destroy(pm_ctx *c) {
     destroy_graph(c);
     for (cudaStream_t b : c->branch) cudaStreamSynchronize(b);
     for (void *p : c->allocs) cudaFree(p);
+    cudaFree(c->dg_part.p);
     if (c->cap) cudaStreamDestroy(c->cap);
     for (cudaStream_t b : c->branch) cudaStreamDestroy(b);
     for (cudaEvent_t e : c->ev_join) cudaEventDestroy(e);
@@ -1519,6 +1547,12 @@ int pm_selftest_wait_expiry(pm_ctx *c) {
     PM_CK(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->user));
     PM_CK(cudaStreamSynchronize(c->user));
     return rc;
+}
+
+int pm_selftest_scratch_limit(pm_ctx *c, int64_t bytes) {
+    if (!c) return fail(PM_E_ARG, "ctx is NULL");
+    c->scratch_limit = bytes;
+    return PM_OK;
 }
 
 int pm_info(pm_ctx *c, int64_t *out) {

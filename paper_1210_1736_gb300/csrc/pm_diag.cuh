@@ -28,8 +28,13 @@ __device__ __forceinline__ bool diag_take(const DiagP<T> &d, long long i) {
     return d.sel ? d.sel[i] != 0 : d.gal_id[i] == d.gal;
 }
 
-// Compacts the selected particles: key = bits of R^2 (the same operations as
-// the FP64 reference, no contraction) and index, in blocks of 1024 particles.
+// Bits of R^2 (the same operations as the FP64 reference, no contraction).
+__device__ __forceinline__ unsigned long long diag_key(double dx, double dy) {
+    return (unsigned long long)__double_as_longlong(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
+}
+
+// Counts the selected particles and compacts their key and index (key null:
+// counts only), in blocks of 1024 particles.
 template <typename T>
 __global__ void __launch_bounds__(256) k_diag_select(DiagP<T> d, const CenK *cen, DiagState *st,
                                                      unsigned long long *key, long long *idx) {
@@ -67,16 +72,32 @@ __global__ void __launch_bounds__(256) k_diag_select(DiagP<T> d, const CenK *cen
         const long long o = (long long)base + wtot[w];
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-            if (take[u]) {
+            if (take[u] && key) {
                 const long long i = b + u * 256 + threadIdx.x;
-                const double dx = __dsub_rn((double)d.x[i], cx), dy = __dsub_rn((double)d.y[i], cy);
-                key[o + before[u]] = (unsigned long long)__double_as_longlong(
-                    __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
+                key[o + before[u]] = diag_key(__dsub_rn((double)d.x[i], cx), __dsub_rn((double)d.y[i], cy));
                 idx[o + before[u]] = i;
             }
         __syncthreads();   // wtot and base are rewritten
     }
 }
+
+// The selected particles' keys: as k_diag_select left them, or from the
+// particles (no memory to keep them).
+struct DiagKept {
+    const unsigned long long *key;
+    __device__ __forceinline__ long long count(const DiagState *st) const { return (long long)st->nsel; }
+    __device__ __forceinline__ bool get(long long i, unsigned long long &k) const { k = key[i]; return true; }
+};
+template <typename T> struct DiagRead {
+    DiagP<T> d;
+    const CenK *cen;
+    __device__ __forceinline__ long long count(const DiagState *) const { return d.n; }
+    __device__ __forceinline__ bool get(long long i, unsigned long long &k) const {
+        if (!diag_take(d, i)) return false;
+        k = diag_key(__dsub_rn((double)d.x[i], cen->c[d.gal][0]), __dsub_rn((double)d.y[i], cen->c[d.gal][1]));
+        return true;
+    }
+};
 
 // Digits of the radix select: DG_BITS bits per pass from the top, the last
 // pass the remaining ones.
@@ -148,12 +169,12 @@ static __device__ void diag_resolve(int pass, int nbins, int np, long long n, Di
 // diag_high) count their next digit.  Lanes with one counter share an atomic
 // (the first digits, exponents, take few values).  The last block to finish
 // resolves the pass.
-static __global__ void __launch_bounds__(256) k_diag_hist(int pass, int nbins, DiagState *st,
-                                                          const unsigned long long *key, unsigned *hist) {
+template <class KEYS>
+__global__ void __launch_bounds__(256) k_diag_hist(int pass, int nbins, DiagState *st, KEYS keys, unsigned *hist) {
     __shared__ unsigned long long pref[DIAG_MAXBINS];
     __shared__ bool last;
     const int np = pass ? st->npref : 1;
-    const long long n = (long long)st->nsel;
+    const long long n = keys.count(st);
     if (threadIdx.x < np) pref[threadIdx.x] = pass ? st->pref[threadIdx.x] : 0;
     __syncthreads();
     const int low = diag_low(pass), high = diag_high(pass);
@@ -161,8 +182,8 @@ static __global__ void __launch_bounds__(256) k_diag_hist(int pass, int nbins, D
     for (long long b = (long long)blockIdx.x * 256; b < n; b += (long long)gridDim.x * 256) {
         const long long i = b + threadIdx.x;
         int bin = -1;
-        if (i < n) {
-            const unsigned long long k = key[i];
+        unsigned long long k;
+        if (i < n && keys.get(i, k)) {
             int j = 0;
             if (pass > 0) {
                 const unsigned long long pk = k >> high;
@@ -185,7 +206,7 @@ static __global__ void __launch_bounds__(256) k_diag_hist(int pass, int nbins, D
     __syncthreads();
     if (last) {
         __threadfence();
-        diag_resolve(pass, nbins, np, n, st, hist);
+        diag_resolve(pass, nbins, np, (long long)st->nsel, st, hist);
     }
 }
 
@@ -205,11 +226,26 @@ __device__ __forceinline__ void diag_root(double r2, double &R, double &inv) {
     R = fma(0.5 * inv, fma(-R, R, r2), R);
 }
 
-// R^2, R, 1/R and the cylindrical velocities of one selected particle; the
-// sums and, for the heat, R, v_phi, v_R^2 + v_z^2 and m per particle.
+// R, the direction and the cylindrical velocities of a particle.
+struct DiagPoint {
+    double R, c1, s1, vR, vphi;
+    __device__ __forceinline__ DiagPoint(unsigned long long key, double dx, double dy, double vx, double vy) {
+        double inv;
+        diag_root(__longlong_as_double((long long)key), R, inv);
+        c1 = dx * inv;
+        s1 = dy * inv;
+        vR = c1 * vx + s1 * vy;
+        vphi = c1 * vy - s1 * vx;
+    }
+    // what the heat needs
+    __device__ __forceinline__ double4 rest(double vz, double m) const { return make_double4(R, vphi, vR * vR + vz * vz, m); }
+};
+
+// The sums over the selected particles; KEPT: of k_diag_select's list, leaving
+// what the heat needs per particle, else of the particles themselves.
 // Accumulators in shared memory: with PRIVATE a column per thread (no
 // conflicts, no atomics), else one set per block.
-template <typename T, bool PRIVATE>
+template <typename T, bool PRIVATE, bool KEPT>
 __global__ void __launch_bounds__(256) k_diag_sums(DiagP<T> d, const CenK *cen, DiagQ q, const DiagState *st,
                                                    const unsigned long long *key, const long long *idx, double *acc,
                                                    double4 *rest) {
@@ -224,7 +260,7 @@ __global__ void __launch_bounds__(256) k_diag_sums(DiagP<T> d, const CenK *cen, 
         else atomicAdd(sh + k, v);
     };
     const double cx = cen->c[d.gal][0], cy = cen->c[d.gal][1], cz = cen->c[d.gal][2], iw = 1.0 / q.width;
-    const long long n = (long long)st->nsel, stride = (long long)gridDim.x * blockDim.x;
+    const long long n = KEPT ? (long long)st->nsel : d.n, stride = (long long)gridDim.x * blockDim.x;
     // few warps fit beside the columns: U particles' loads in flight each
     constexpr int U = 4;
     for (long long p0 = (long long)blockIdx.x * blockDim.x + threadIdx.x; p0 < n; p0 += U * stride) {
@@ -232,14 +268,18 @@ __global__ void __launch_bounds__(256) k_diag_sums(DiagP<T> d, const CenK *cen, 
         T xu[U], yu[U], zu[U], vxu[U], vyu[U], vzu[U], mu[U];
         long long iu[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (p0 + u * stride < n) {
-                ku[u] = key[p0 + u * stride];
-                iu[u] = idx[p0 + u * stride];
+        for (int u = 0; u < U; ++u) {
+            const long long p = p0 + u * stride;
+            iu[u] = -1;
+            if (KEPT) {
+                if (p < n) { ku[u] = key[p]; iu[u] = idx[p]; }
+            } else if (p < n && diag_take(d, p)) {
+                iu[u] = p;
             }
+        }
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (p0 + u * stride < n) {
+            if (iu[u] >= 0) {
                 const long long i = iu[u];
                 xu[u] = d.x[i]; yu[u] = d.y[i]; zu[u] = d.z[i];
                 vxu[u] = d.vx[i]; vyu[u] = d.vy[i]; vzu[u] = d.vz[i];
@@ -247,10 +287,9 @@ __global__ void __launch_bounds__(256) k_diag_sums(DiagP<T> d, const CenK *cen, 
             }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const long long p = p0 + u * stride;
-            if (p >= n) break;
-            const unsigned long long r2k = ku[u];
+            if (iu[u] < 0) continue;
             const double dx = __dsub_rn((double)xu[u], cx), dy = __dsub_rn((double)yu[u], cy);
+            const unsigned long long r2k = KEPT ? ku[u] : diag_key(dx, dy);
             const double dz = __dsub_rn((double)zu[u], cz);
             const double vx = vxu[u], vy = vyu[u], vz = vzu[u], m = mu[u];
             int b = 0;   // number of edges <= key
@@ -262,11 +301,9 @@ __global__ void __launch_bounds__(256) k_diag_sums(DiagP<T> d, const CenK *cen, 
                 }
                 b = lo;
             }
-            double R, inv;
-            diag_root(__longlong_as_double((long long)r2k), R, inv);
-            const double c1 = dx * inv, s1 = dy * inv;
-            const double vR = c1 * vx + s1 * vy, vphi = c1 * vy - s1 * vx;
-            rest[p] = make_double4(R, vphi, vR * vR + vz * vz, m);
+            const DiagPoint pt(r2k, dx, dy, vx, vy);
+            const double R = pt.R, c1 = pt.c1, s1 = pt.s1, vR = pt.vR, vphi = pt.vphi;
+            if (KEPT) rest[p0 + u * stride] = pt.rest(vz, m);
             add(4 * b + 0, R);
             add(4 * b + 1, 1.0);
             add(4 * b + 2, dz * dz);
@@ -323,8 +360,9 @@ __global__ void __launch_bounds__(256) k_diag_sums(DiagP<T> d, const CenK *cen, 
 
 // E_heat with vbar_c linear in R between the non-empty bins' (mean R, mean
 // v_phi), held constant outside.
-static __global__ void __launch_bounds__(256) k_diag_heat(int nbins, const DiagState *st, const double *acc,
-                                                          const double4 *rest, double *heat) {
+template <typename T, bool KEPT>
+__global__ void __launch_bounds__(256) k_diag_heat(DiagP<T> d, const CenK *cen, int nbins, const DiagState *st,
+                                                   const double *acc, const double4 *rest, double *heat) {
     __shared__ double xp[DIAG_MAXBINS], fp[DIAG_MAXBINS], sl[DIAG_MAXBINS], red[8];
     __shared__ int s_np;
     if (threadIdx.x < 32) {
@@ -346,10 +384,17 @@ static __global__ void __launch_bounds__(256) k_diag_heat(int nbins, const DiagS
     }
     __syncthreads();
     const int np = s_np;
-    const long long n = (long long)st->nsel, stride = (long long)gridDim.x * blockDim.x;
+    const long long n = KEPT ? (long long)st->nsel : d.n, stride = (long long)gridDim.x * blockDim.x;
     double e = 0.0;
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += stride) {
-        const double4 v = rest[p];
+        double4 v;
+        if (KEPT) {
+            v = rest[p];
+        } else {
+            if (!diag_take(d, p)) continue;
+            const double dx = __dsub_rn((double)d.x[p], cen->c[d.gal][0]), dy = __dsub_rn((double)d.y[p], cen->c[d.gal][1]);
+            v = DiagPoint(diag_key(dx, dy), dx, dy, d.vx[p], d.vy[p]).rest(d.vz[p], d.m[p]);
+        }
         const double R = v.x;
         double vb;
         if (R <= xp[0]) vb = fp[0];
@@ -377,6 +422,35 @@ static __global__ void __launch_bounds__(256) k_diag_heat(int nbins, const DiagS
 
 }  // namespace pmk
 
+template <typename T, bool KEPT>
+cudaError_t pm_launch_diag_k(const pmk::DiagP<T> &d, const CenK *cen, const pmk::DiagQ &q, const pmk::DiagBuf &b,
+                             cudaStream_t st) {
+    const int nacc = 4 * q.nbins + 7 + 2 * q.nring * q.mmax;
+    // a wave of blocks: the sums' epilogues cost FP64 operations per block
+    const unsigned wave = 152 * 8, by = (unsigned)std::min<long long>((d.n + 1023) / 1024, wave);
+    pmk::k_diag_select<T><<<by, 256, 0, st>>>(d, cen, b.state, b.key, b.idx);
+    if (q.nbins > 1)
+        for (int pass = 0; pass < pmk::DG_PASSES; ++pass) {
+            const unsigned g = std::min(by, 152u * 2);
+            if constexpr (KEPT) pmk::k_diag_hist<<<g, 256, 0, st>>>(pass, q.nbins, b.state, pmk::DiagKept{b.key}, b.hist);
+            else pmk::k_diag_hist<<<g, 256, 0, st>>>(pass, q.nbins, b.state, pmk::DiagRead<T>{d, cen}, b.hist);
+        }
+    // a column of accumulators per thread while 64 or 32 threads' fit two
+    // blocks on an SM
+    const size_t one = sizeof(double) * nacc;
+    const int threads = 64 * one <= 100u << 10 ? 64 : 32 * one <= 100u << 10 ? 32 : 0;
+    if (threads) {
+        const auto k = pmk::k_diag_sums<T, true, KEPT>;
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 << 10);
+        if (e != cudaSuccess) return e;
+        k<<<152 * 2, threads, threads * one, st>>>(d, cen, q, b.state, b.key, b.idx, b.acc, b.rest);
+    } else {
+        pmk::k_diag_sums<T, false, KEPT><<<std::min(by, 152u * 4), 256, one, st>>>(d, cen, q, b.state, b.key, b.idx, b.acc, b.rest);
+    }
+    pmk::k_diag_heat<T, KEPT><<<std::min(by, 152u * 4), 256, 0, st>>>(d, cen, q.nbins, b.state, b.acc, b.rest, b.acc + nacc);
+    return cudaGetLastError();
+}
+
 // Every step of pm_disc_diagnostics on the device (acc: nacc + 1 sums, the
 // last the heat; everything zeroed here).
 template <typename T>
@@ -388,25 +462,7 @@ cudaError_t pm_launch_diag(const pmk::DiagP<T> &d, const CenK *cen, const pmk::D
     if (e == cudaSuccess && q.nbins > 1)
         e = cudaMemsetAsync(b.hist, 0, sizeof(unsigned) * pmk::DG_ROW * (q.nbins - 1), st);
     if (e != cudaSuccess || d.n <= 0) return e;
-    // a wave of blocks: the sums' epilogues cost FP64 operations per block
-    const unsigned wave = 152 * 8, by = (unsigned)std::min<long long>((d.n + 1023) / 1024, wave);
-    pmk::k_diag_select<T><<<by, 256, 0, st>>>(d, cen, b.state, b.key, b.idx);
-    if (q.nbins > 1)
-        for (int pass = 0; pass < pmk::DG_PASSES; ++pass)
-            pmk::k_diag_hist<<<std::min(by, 152u * 2), 256, 0, st>>>(pass, q.nbins, b.state, b.key, b.hist);
-    // a column of accumulators per thread while 64 or 32 threads' fit two
-    // blocks on an SM
-    const size_t one = sizeof(double) * nacc;
-    const int threads = 64 * one <= 100u << 10 ? 64 : 32 * one <= 100u << 10 ? 32 : 0;
-    if (threads) {
-        e = cudaFuncSetAttribute(pmk::k_diag_sums<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 << 10);
-        if (e != cudaSuccess) return e;
-        pmk::k_diag_sums<T, true><<<152 * 2, threads, threads * one, st>>>(d, cen, q, b.state, b.key, b.idx, b.acc, b.rest);
-    } else {
-        pmk::k_diag_sums<T, false><<<std::min(by, 152u * 4), 256, one, st>>>(d, cen, q, b.state, b.key, b.idx, b.acc, b.rest);
-    }
-    pmk::k_diag_heat<<<std::min(by, 152u * 4), 256, 0, st>>>(q.nbins, b.state, b.acc, b.rest, b.acc + nacc);
-    return cudaGetLastError();
+    return b.key ? pm_launch_diag_k<T, true>(d, cen, q, b, st) : pm_launch_diag_k<T, false>(d, cen, q, b, st);
 }
 
 #define PM_DIAG_INSTANTIATE(T)                                                                                \

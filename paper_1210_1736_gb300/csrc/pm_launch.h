@@ -186,7 +186,8 @@ struct DiagState {
     int which[DIAG_MAXBINS];
 };
 // Scratch: state, counters (2048 per boundary), sums; per particle the key,
-// the index and what the heat needs (48 bytes).
+// the index and what the heat needs (48 bytes), or null: the passes then read
+// the particles themselves.
 struct DiagBuf {
     DiagState *state;
     unsigned *hist;

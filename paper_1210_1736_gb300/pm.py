@@ -89,6 +89,7 @@ _SIGS.update({
     "pm_cic_kick_drift": (C.c_int, [_vp, _P(pm_particles), C.c_double, C.c_double]),
     "pm_cic_vjp": (C.c_int, [_vp, _P(pm_particles), _vp, _vp, _vp, _vp, _vp, _vp, _vp]),
     "pm_selftest_wait_expiry": (C.c_int, [_vp]),
+    "pm_selftest_scratch_limit": (C.c_int, [_vp, C.c_int64]),
     "pm_recentre_sums": (C.c_int, [_vp, _P(pm_particles)]),
     "pm_recentre_apply": (C.c_int, [_vp]),
     "pm_exchange_buffers": (C.c_int, [_vp, _P(_vp), _P(C.c_int64), _P(_vp), _P(C.c_int64)]),
@@ -400,6 +401,10 @@ class Context:
         """Status of the bounded-wait self-test (PM_E_TIMEOUT is the expected
         result: the wait gave up and the host saw it); see include/pm.h."""
         return int(lib().pm_selftest_wait_expiry(self.h))
+
+    def selftest_scratch_limit(self, nbytes):
+        """Refuses optional scratch beyond nbytes (negative: no limit); see include/pm.h."""
+        _check(lib().pm_selftest_scratch_limit(self.h, int(nbytes)))
 
     def set_launch_config(self, batched, schedule):
         """The solve's launch grouping (batched 1/0) and branch schedule

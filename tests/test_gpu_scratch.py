@@ -25,3 +25,54 @@ def test_refused_allocation_is_reported_once():
     assert np.array_equal(rho, ctx.density(0, 5))
     ctx.sort(p)
     ctx.close()
+
+
+def _subset(p, n):
+    import torch
+    return pm.Particles.from_tensors(torch.stack([p.x, p.y, p.z])[:, :n].contiguous(),
+                                     torch.stack([p.vx, p.vy, p.vz])[:, :n].contiguous(), p.m[:n].contiguous(),
+                                     p.gal[:n].contiguous())
+
+
+def test_outgrown_disc_scratch_is_released():
+    """The context's bytes follow the largest particle number, not the sum."""
+    w = W.galaxy_small(n_total=4000)
+    ctx, p = gpu_setup(w)
+    base = ctx.info()["bytes"]
+    sizes = []
+    for n in (1000, 2000, 3000, 3500, 4000, 2500):
+        ctx.disc_diagnostics(_subset(p, n))
+        sizes.append(ctx.info()["bytes"] - base)
+    fixed = sizes[0] - 48 * 1000
+    assert 0 < fixed < 1 << 20
+    assert sizes == [fixed + 48 * n for n in (1000, 2000, 3000, 3500, 4000, 4000)]
+    ctx.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("nbins,nring,mmax,nsel", [(1, 1, 1, None), (20, 10, 4, None), (33, 3, 7, 100),
+                                                   (64, 16, 64, 5000), (64, 1, 1, 3), (5, 4, 2, 0)])
+def test_disc_diagnostics_without_scratch(precision, nbins, nring, mmax, nsel):
+    """Without memory for the particles' part the passes read the particles:
+    the same bins, the same terms in other sums."""
+    import torch
+    w = W.galaxy_small(precision=precision, n_total=20_000)
+    ctx, p = gpu_setup(w)
+    ctx.deposit(p)
+    disc = np.asarray(w["comp"]) == W.COMP_DISC
+    if nsel is not None:
+        disc &= np.cumsum(disc) <= nsel
+    sel = torch.tensor(disc, device="cuda")
+    out = []
+    for limit in (0, -1):
+        ctx.selftest_scratch_limit(limit)
+        before = ctx.info()["bytes"]
+        out.append(ctx.disc_diagnostics(p, sel, nbins=nbins, nring=nring, mmax=mmax)["raw"])
+        assert (ctx.info()["bytes"] - before >= 48 * p.n) == (limit < 0)
+    counts = slice(7, 6 + 4 * nbins, 4)
+    got, ref = out
+    assert np.array_equal(got[counts], ref[counts]) and got[0] == ref[0]
+    # FP64 sums of at most 20,000 terms in another order (as in test_gpu_diag_paths.py)
+    tol = 1e-9 * np.abs(ref) + 1e-12 * np.abs(ref[6 + 4 * nbins:]).max(initial=0.0)
+    assert np.all(np.abs(got - ref) <= tol)
+    ctx.close()
