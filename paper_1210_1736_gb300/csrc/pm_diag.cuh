@@ -445,7 +445,12 @@ cudaError_t pm_launch_diag_k(const pmk::DiagP<T> &d, const CenK *cen, const pmk:
         if (e != cudaSuccess) return e;
         k<<<152 * 2, threads, threads * one, st>>>(d, cen, q, b.state, b.key, b.idx, b.acc, b.rest);
     } else {
-        pmk::k_diag_sums<T, false, KEPT><<<std::min(by, 152u * 4), 256, one, st>>>(d, cen, q, b.state, b.key, b.idx, b.acc, b.rest);
+        // one set per block: small blocks, as few particles as there are for
+        // each, since a block's threads add to its set one after another (64
+        // bins, 16 x 64 modes, whole call with 20k / 100k / 1M particles: 482, 543
+        // and 1484 us; 256 threads, a block per 1024 particles 603, 628 and 1557)
+        const unsigned g = (unsigned)std::min<long long>((d.n + 127) / 128, 152 * 8);
+        pmk::k_diag_sums<T, false, KEPT><<<g, 128, one, st>>>(d, cen, q, b.state, b.key, b.idx, b.acc, b.rest);
     }
     pmk::k_diag_heat<T, KEPT><<<std::min(by, 152u * 4), 256, 0, st>>>(d, cen, q.nbins, b.state, b.acc, b.rest, b.acc + nacc);
     return cudaGetLastError();
