@@ -212,9 +212,9 @@ struct pm_ctx {
     size_t bytes = 0;
     std::vector<void *> allocs;
     bool any_recentre = false;
-    // disc diagnostics: fixed part (allocated on first use), particles' part
-    pmk::DiagBuf dg = {};
-    Scratch dg_part;
+    // disc diagnostics: everything, or the fixed part alone
+    Scratch dg_mem;
+    void *dg_fixed = nullptr;
     long long scratch_limit = -1;   // bytes a Scratch may hold (tests; < 0: no limit)
 };
 
@@ -889,19 +889,26 @@ constexpr int DG_MAXBINS = pmk::DIAG_MAXBINS, DG_MAXRM = 1024;
 template <typename T> int disc_impl(pm_ctx *c, const pm_particles *p, const uint8_t *sel, const pm_disc_query *q,
                                     double *out) {
     cudaStream_t st = c->user;
-    if (!c->dg.acc) {
-        constexpr size_t hist = sizeof(unsigned) * 2048 * DG_MAXBINS, state = (sizeof(pmk::DiagState) + 255) & ~(size_t)255;
-        unsigned char *m = nullptr;
-        PM_TRY(dev_alloc(c, (void **)&m, hist + state + sizeof(double) * (4 * DG_MAXBINS + 8 + 2 * DG_MAXRM)));
-        c->dg.hist = (unsigned *)m;
-        c->dg.state = (pmk::DiagState *)(m + hist);
-        c->dg.acc = (double *)(m + hist + state);
+    // fixed part, then per particle rest (32 bytes), key and index; without
+    // memory for those every pass reads the particles instead
+    constexpr size_t hist = sizeof(unsigned) * 2048 * DG_MAXBINS, state = (sizeof(pmk::DiagState) + 255) & ~(size_t)255;
+    constexpr size_t fixed = hist + state + sizeof(double) * (4 * DG_MAXBINS + 8 + 2 * DG_MAXRM);
+    static_assert(fixed % sizeof(double4) == 0, "alignment of the particles' part");
+    unsigned char *m = (unsigned char *)keep_scratch(c, c->dg_mem, fixed + (size_t)p->n * 48);
+    const bool kept = m != nullptr;
+    if (!kept) {
+        if (!c->dg_fixed) PM_TRY(dev_alloc(c, &c->dg_fixed, fixed));
+        m = (unsigned char *)c->dg_fixed;
     }
-    // per particle: rest (32 bytes), key and index; without memory for them
-    // every pass reads the particles instead
-    c->dg.rest = (double4 *)keep_scratch(c, c->dg_part, (size_t)p->n * 48);
-    c->dg.key = c->dg.rest ? (unsigned long long *)(c->dg.rest + p->n) : nullptr;
-    c->dg.idx = c->dg.rest ? (long long *)(c->dg.key + p->n) : nullptr;
+    pmk::DiagBuf dg = {};
+    dg.hist = (unsigned *)m;
+    dg.state = (pmk::DiagState *)(m + hist);
+    dg.acc = (double *)(m + hist + state);
+    if (kept) {
+        dg.rest = (double4 *)(m + fixed);
+        dg.key = (unsigned long long *)(dg.rest + p->n);
+        dg.idx = (long long *)(dg.key + p->n);
+    }
     pmk::DiagP<T> d;
     d.x = (const T *)p->x; d.y = (const T *)p->y; d.z = (const T *)p->z;
     d.vx = (const T *)p->vx; d.vy = (const T *)p->vy; d.vz = (const T *)p->vz;
@@ -921,11 +928,11 @@ template <typename T> int disc_impl(pm_ctx *c, const pm_particles *p, const uint
     dq.width = NR > 0 ? q->r_ring / NR : 1.0;
     dq.rlo = q->r0 - q->dr;
     dq.rhi = q->r0 + q->dr;
-    PM_CK(pm_launch_diag<T>(d, c->d_cen, dq, c->dg, st));
+    PM_CK(pm_launch_diag<T>(d, c->d_cen, dq, dg, st));
     std::vector<double> acc(nacc + 1);
     pmk::DiagState ds;
-    PM_CK(cudaMemcpyAsync(acc.data(), c->dg.acc, sizeof(double) * (nacc + 1), cudaMemcpyDeviceToHost, st));
-    PM_CK(cudaMemcpyAsync(&ds, c->dg.state, sizeof(ds), cudaMemcpyDeviceToHost, st));
+    PM_CK(cudaMemcpyAsync(acc.data(), dg.acc, sizeof(double) * (nacc + 1), cudaMemcpyDeviceToHost, st));
+    PM_CK(cudaMemcpyAsync(&ds, dg.state, sizeof(ds), cudaMemcpyDeviceToHost, st));
     PM_TRY(check_device_error(c));   // synchronises
     if (ds.err) return fail(PM_E_STATE, "radix select lost a rank (particles changed during the call?)");
     if (ds.nsel == 0) return PM_OK;
@@ -1310,7 +1317,7 @@ void pm_destroy(pm_ctx *c) {
     destroy_graph(c);
     for (cudaStream_t b : c->branch) cudaStreamSynchronize(b);
     for (void *p : c->allocs) cudaFree(p);
-    cudaFree(c->dg_part.p);
+    cudaFree(c->dg_mem.p);
     if (c->cap) cudaStreamDestroy(c->cap);
     for (cudaStream_t b : c->branch) cudaStreamDestroy(b);
     for (cudaEvent_t e : c->ev_join) cudaEventDestroy(e);
