@@ -276,10 +276,11 @@ int pm_step_timed(pm_ctx *ctx, const pm_particles *p, double dt, int32_t nsteps,
  *
  * pm_cic_deposit: lost test as pm_deposit, then int64 fixed-point CIC mass
  * (each of the 8 cell shares rounded separately) into the five sets.  Use
- * pm_solve afterwards.  From 65536 particles it also finds the particles'
- * spatial order, in which this and the following CIC calls work (no result
- * depends on it): 12 bytes per particle, allocated on the first call with
- * more particles than before.  Captured calls work in the stored order.
+ * pm_solve afterwards.  In nested systems, from 65536 particles and a
+ * sixteenth of the cells, it also finds the particles' spatial order, in which
+ * this and the following CIC calls work (no result depends on it): 12 bytes
+ * per particle, allocated on the first call with more particles than before.
+ * Captured calls work in the stored order.
  * pm_cic_force: ax, ay, az (device, context precision, n) = CIC acceleration
  * from the current potentials; lost particles get 0.
  * pm_cic_kick_drift: v += dt_kick a; x += dt_drift v (live particles).

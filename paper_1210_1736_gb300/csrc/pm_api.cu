@@ -790,7 +790,23 @@ template <typename T> int step_timed_impl(pm_ctx *c, const pm_particles *p, doub
 // for other particles of the same number it is only a worse one.  Captured
 // calls, which may neither allocate nor rely on a later state of the scratch,
 // and calls without memory for it run in the stored order.
-constexpr long long CIC_ORDER_MIN = 1LL << 16, CIC_ORDER_MAX = 1LL << 32;
+//
+// The order costs 26 us, more with the number of cells (its keys).  It pays
+// where cells are crowded: nested grids, whose coarse cells are as large as a
+// core.  Forward and backward of 4 steps, us, stored order -> ordered:
+//   one 64^3 grid, FP32        66k 2212 -> 2558, 1M 5376 -> 7124 (FP64 500k 7930 -> 8910)
+//   nested 32^3, 64^3, FP32    66k 3432 -> 3485, 3389 -> 3426; 100k 4311 -> 3992, 4086 -> 3789
+//   nested 64^3 and satellite  66k 4475 -> 4129, 100k 5384 -> 4542 (FP64 32k 8981 -> 8654)
+//   nested 128^3 (4.7M cells)  200k 8994 -> 9037, 300k 9845 -> 9380
+//   nested 32^3, FP64          32k 4304 -> 4367, 66k 5938 -> 5562
+// Most of the gain is the product's (its spread): a deposit without one gains
+// from about 1.2e5 particles in FP32 (66k 43 -> 56 us, 200k 101 -> 88).
+constexpr long long CIC_ORDER_MIN = 1LL << 16, CIC_ORDER_MAX = 1LL << 32, CIC_ORDER_CELLS = 16;
+bool cic_order_pays(const pm_ctx *c, long long n) {
+    bool nested = false;
+    for (int g = 0; g < c->sys.ngal; ++g) nested = nested || geom_present(c->gal[g].medium);
+    return nested && n >= CIC_ORDER_MIN && n >= c->sortk.nkeys / CIC_ORDER_CELLS && n < CIC_ORDER_MAX;
+}
 bool capturing(const pm_ctx *c) {
     cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(c->user, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
@@ -800,7 +816,7 @@ bool capturing(const pm_ctx *c) {
 template <typename T> int cic_order(pm_ctx *c, const pm_particles *p) {
     if (capturing(c)) return PM_OK;
     c->ord_n = 0;
-    if (p->n < CIC_ORDER_MIN || p->n >= CIC_ORDER_MAX) return PM_OK;
+    if (!cic_order_pays(c, p->n)) return PM_OK;
     if (p->n > c->ord_cap) {
         void *a = nullptr;   // key, rank and order
         if (cudaMalloc(&a, (size_t)p->n * 12) != cudaSuccess) {
@@ -832,8 +848,12 @@ template <typename T> int cic_deposit_impl(pm_ctx *c, const pm_particles *p) {
 
 template <typename T> int cic_field_impl(pm_ctx *c, int mode, const pm_particles *p, double dtk, double dtd,
                                          void *ox, void *oy, void *oz) {
+    // a kick-drift writes six arrays, scattered in an order: FP32 keeps the
+    // stored one (1M: 99 us, ordered 122), FP64, bound by arithmetic that
+    // neighbours share, does not (200k: 152, ordered 93)
+    const unsigned *ord = mode == 0 && sizeof(T) == 4 ? nullptr : cic_ord(c, p);
     PM_CK(pm_launch_cic_field<T>(mode, part_k<T>(p), c->hs, c->d_cen, dtk, dtd, (T *)ox, (T *)oy, (T *)oz, nullptr,
-                                 nullptr, nullptr, 0.0, cic_ord(c, p), c->user));
+                                 nullptr, nullptr, 0.0, ord, c->user));
     return PM_OK;
 }
 

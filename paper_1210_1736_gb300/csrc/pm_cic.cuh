@@ -27,12 +27,11 @@
 // lam_2 = a + b, lam_3 = b); coarse a = psi_4 - psi_5, b = psi_5.
 //
 // Bound by the atomics (32 per point and level in the adjoint spread, 80 G/s
-// for unsorted points).  So the particles run in spatial order (an index
-// computed per deposit, pm_launch_order, 55 us for 1M), runs of particles in
-// one cell share their atomics, and each point spreads once per level.  1M
-// points of two galaxies: deposit 333 -> 129 us, spread 1600 -> 558, direct term
-// 160 -> 104.  From 2^16 particles; below, the launches of the order cost more
-// than it saves.
+// for unsorted points).  So the particles of nested systems run in spatial order
+// (an index computed per deposit, pm_launch_order, 55 us for 1M; the rule and
+// both its sides: cic_order_pays in pm_api.cu), runs of particles in one cell
+// share their atomics, and each point spreads once per level.  1M points of two
+// galaxies: deposit 333 -> 129 us, spread 1600 -> 558, direct term 160 -> 104.
 #pragma once
 
 #include <algorithm>

@@ -128,3 +128,31 @@ def test_captured_calls_keep_the_stored_order():
     assert not before.any()
     assert a.any() and torch.equal(a, b)
     ctx.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_where_the_order_is_computed(precision):
+    """In nested systems from 2^16 particles and a sixteenth of the cells (32
+    and 128 cells a side here); not on a single grid."""
+    import torch
+
+    def grown(w, n):
+        ctx = pm.Context(w, W.mass_bound(cast(w, w["m"])))
+        p = pm.Particles(cast(w, w["pos"])[:, :n], cast(w, w["vel"])[:, :n], cast(w, w["m"])[:n], w["gal"][:n],
+                         precision=precision)
+        size = ctx.info()["bytes"]
+        ctx.cic_deposit(p)
+        ctx.solve()
+        a = torch.stack(ctx.cic_force(p))
+        assert torch.isfinite(a).all() and a.any()
+        size = ctx.info()["bytes"] - size
+        ctx.close()
+        return size
+
+    n = 1 << 16
+    w = _case(precision, n, False)
+    assert grown(w, n) == 12 * n and grown(w, n - 1) == 0
+    wide = dict(w, galaxies=[dict(w["galaxies"][0]), *w["galaxies"][1:]])
+    wide["galaxies"][0]["coarse"] = (128, 128, 128) + tuple(w["galaxies"][0]["coarse"][3:])
+    assert grown(wide, n) == 0
+    assert grown(W.big_box(n, 32, precision=precision), n) == 0
