@@ -232,9 +232,9 @@ int pm_set_launch_config(pm_ctx *ctx, int32_t batched, int32_t schedule);
 int pm_selftest_wait_expiry(pm_ctx *ctx);
 
 /* Test hook: scratch that calls keep only while memory allows (the particles'
- * part of pm_disc_diagnostics) is refused from now on beyond `bytes` (negative:
- * no limit, the default); results do not depend on it beyond the order of
- * FP64 sums. */
+ * part of pm_disc_diagnostics, the order of the CIC calls) is refused from now
+ * on beyond `bytes` (negative: no limit, the default); results do not depend on
+ * it beyond the order of FP64 sums. */
 int pm_selftest_scratch_limit(pm_ctx *ctx, int64_t bytes);
 
 /* Spatial sort (no counterpart in the paper; a locality optimisation of the
@@ -279,8 +279,9 @@ int pm_step_timed(pm_ctx *ctx, const pm_particles *p, double dt, int32_t nsteps,
  * pm_solve afterwards.  In nested systems, from 65536 particles and a
  * sixteenth of the cells, it also finds the particles' spatial order, in which
  * this and the following CIC calls work (no result depends on it): 12 bytes
- * per particle, allocated on the first call with more particles than before.
- * Captured calls work in the stored order.
+ * per particle, allocated on the first call with more particles than before
+ * (the outgrown buffer is released).  Captured calls, and calls without memory
+ * for it, work in the stored order.
  * pm_cic_force: ax, ay, az (device, context precision, n) = CIC acceleration
  * from the current potentials; lost particles get 0.
  * pm_cic_kick_drift: v += dt_kick a; x += dt_drift v (live particles).

@@ -207,8 +207,9 @@ struct pm_ctx {
     unsigned *s_count = nullptr, *s_key = nullptr, *s_rank = nullptr, *s_bsum = nullptr;
     void *s_arr[9] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     // processing order of the CIC kernels (a permutation of 0..ord_n - 1)
-    unsigned *o_key = nullptr, *o_rank = nullptr, *o_ord = nullptr;
-    long long ord_cap = 0, ord_n = 0;
+    Scratch o_mem;
+    unsigned *o_ord = nullptr;
+    long long ord_n = 0;
     size_t bytes = 0;
     std::vector<void *> allocs;
     bool any_recentre = false;
@@ -817,21 +818,12 @@ template <typename T> int cic_order(pm_ctx *c, const pm_particles *p) {
     if (capturing(c)) return PM_OK;
     c->ord_n = 0;
     if (!cic_order_pays(c, p->n)) return PM_OK;
-    if (p->n > c->ord_cap) {
-        void *a = nullptr;   // key, rank and order
-        if (cudaMalloc(&a, (size_t)p->n * 12) != cudaSuccess) {
-            cudaGetLastError();
-            return PM_OK;
-        }
-        c->allocs.push_back(a);
-        c->bytes += (size_t)p->n * 12;
-        c->o_key = (unsigned *)a;
-        c->o_rank = c->o_key + p->n;
-        c->o_ord = c->o_rank + p->n;
-        c->ord_cap = p->n;
-    }
-    PM_CK(pm_launch_order<T>(part_k<T>(p), c->hs, c->d_cen, c->sortk, c->s_count, c->o_key, c->o_rank, c->s_bsum,
-                             c->o_ord, c->user));
+    unsigned *key = (unsigned *)keep_scratch(c, c->o_mem, (size_t)p->n * 12);   // key, rank and order
+    if (!key) return PM_OK;
+    unsigned *rank = key + p->n;
+    c->o_ord = rank + p->n;
+    PM_CK(pm_launch_order<T>(part_k<T>(p), c->hs, c->d_cen, c->sortk, c->s_count, key, rank, c->s_bsum, c->o_ord,
+                             c->user));
     c->ord_n = p->n;
     return PM_OK;
 }
@@ -1338,6 +1330,7 @@ void pm_destroy(pm_ctx *c) {
     for (cudaStream_t b : c->branch) cudaStreamSynchronize(b);
     for (void *p : c->allocs) cudaFree(p);
     cudaFree(c->dg_mem.p);
+    cudaFree(c->o_mem.p);
     if (c->cap) cudaStreamDestroy(c->cap);
     for (cudaStream_t b : c->branch) cudaStreamDestroy(b);
     for (cudaEvent_t e : c->ev_join) cudaEventDestroy(e);

@@ -76,3 +76,32 @@ def test_disc_diagnostics_without_scratch(precision, nbins, nring, mmax, nsel):
     tol = 1e-9 * np.abs(ref) + 1e-12 * np.abs(ref[6 + 4 * nbins:]).max(initial=0.0)
     assert np.all(np.abs(got - ref) <= tol)
     ctx.close()
+
+
+def test_outgrown_order_is_released_and_refused():
+    """The CIC calls' order: 12 bytes for the largest particle number, and the
+    same densities and accelerations where it is refused."""
+    import torch
+    n = (1 << 16) + 3000
+    w = W.merger(n_gal=n - 3000, n_sat=3000, grids=((32,), (32,), (32, 32, 8), (16,)), seed_id=21, q_m=0.8, r_apo=3.0)
+    ctx, p = gpu_setup(w)
+    base = ctx.info()["bytes"]
+    for k, cap in ((n - 3000, n - 3000), (n - 2000, n - 2000), (n, n), (n - 1000, n)):
+        ctx.cic_deposit(_subset(p, k))
+        assert ctx.info()["bytes"] - base == 12 * cap
+    res = []
+    for limit in (-1, 0):
+        ctx, p = gpu_setup(w)
+        ctx.selftest_scratch_limit(limit)
+        base = ctx.info()["bytes"]
+        ctx.cic_deposit(p)
+        assert ctx.info()["bytes"] - base == (12 * n if limit < 0 else 0)
+        rho = {k: ctx.density(*k) for k in ctx.shapes}
+        ctx.solve()
+        a = torch.stack(ctx.cic_force(p))
+        g, gm = torch.zeros_like(a), torch.zeros_like(p.m)
+        ctx.cic_vjp(p, a, g, gm)
+        res.append((rho, a, g, gm))
+    (ra, *a), (rb, *b) = res
+    assert all(np.array_equal(ra[k], rb[k]) for k in ra)
+    assert all(torch.equal(s, t) for s, t in zip(a, b))
