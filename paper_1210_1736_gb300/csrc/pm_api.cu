@@ -235,14 +235,20 @@ int dev_alloc(pm_ctx *c, void **p, size_t bytes) {
 
 // At least `bytes` of s, or null, without an error, where there is no memory
 // for them: the caller has a way without.  An outgrown buffer is released
-// first (cudaFree waits for the kernels that use it).
+// first (cudaFree waits for the kernels that use it).  In relaxed capture mode:
+// another stream of the caller's may be capturing, which an allocation in the
+// default mode would end.
 void *keep_scratch(pm_ctx *c, Scratch &s, size_t bytes) {
     if (bytes <= s.bytes) return s.p;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
     cudaFree(s.p);
     c->bytes -= s.bytes;
     s = Scratch();
-    if (c->scratch_limit >= 0 && bytes > (size_t)c->scratch_limit) return nullptr;
-    if (cudaMalloc(&s.p, bytes) != cudaSuccess) {
+    cudaError_t e = cudaErrorMemoryAllocation;
+    if (c->scratch_limit < 0 || bytes <= (size_t)c->scratch_limit) e = cudaMalloc(&s.p, bytes);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
         cudaGetLastError();
         s.p = nullptr;
         return nullptr;

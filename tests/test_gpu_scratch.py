@@ -105,3 +105,32 @@ def test_outgrown_order_is_released_and_refused():
     (ra, *a), (rb, *b) = res
     assert all(np.array_equal(ra[k], rb[k]) for k in ra)
     assert all(torch.equal(s, t) for s, t in zip(a, b))
+
+
+def test_growth_beside_another_streams_capture():
+    """Scratch that grows while the caller captures on another stream neither
+    fails nor ends that capture."""
+    import torch
+    n = (1 << 16) + 2000
+    w = W.merger(n_gal=n - 3000, n_sat=3000, grids=((32,), (32,), (32, 32, 8), (16,)), seed_id=21, q_m=0.8, r_apo=3.0)
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        ctx, p = gpu_setup(w)
+        few = _subset(p, n - 1000)
+        ctx.cic_deposit(few)
+        s.synchronize()
+    t = torch.zeros(8, device="cuda")
+    torch.cuda.synchronize()
+    size = ctx.info()["bytes"]
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        t.add_(1)
+        ctx.cic_deposit(p)   # on s, which is not captured
+    assert ctx.info()["bytes"] == size + 12 * 1000
+    g.replay()
+    g.replay()
+    torch.cuda.synchronize()
+    assert (t == 2).all()
+    rho = {k: ctx.density(*k) for k in ctx.shapes}
+    ctx.cic_deposit(p)
+    assert all(np.array_equal(rho[k], ctx.density(*k)) for k in ctx.shapes)
