@@ -2,6 +2,7 @@
 // precision T (float or double).  Included once per precision.
 #pragma once
 
+#include <atomic>
 #include <utility>
 
 #include "pm_passes.cuh"
@@ -724,16 +725,6 @@ inline int particle_grid(long long n) {
     return (int)(b < cap ? (b > 0 ? b : 1) : cap);
 }
 
-inline int num_sms() {
-    static int n = 0;
-    if (!n) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
-    }
-    return n;
-}
-
 // Persistent passes: one wave of blocks (occupancy x SMs), each walking
 // tiles or groups of rows.
 template <typename K> int resident_blocks(K kernel, int threads, size_t smem) {
@@ -832,9 +823,9 @@ template <typename T, int L, bool INV, bool HALF> cudaError_t xpass_LH(PassBatch
     if (sizeof(T) == 8)
         while (threads > 32 && b.n * rows * TPC < (long long)threads * num_sms()) threads /= 2;
     b.lgi = ilog2(std::max(1LL, rows * TPC / threads));
-    static int cache[11];
-    int &nb = cache[ilog2(threads)];
-    if (!nb) nb = resident_blocks(P::kernel(), threads, P::smem(threads));
+    static std::atomic<int> cache[11];   // by block size; contexts of several threads fill it with equal values
+    int nb = cache[ilog2(threads)].load(std::memory_order_relaxed);
+    if (!nb) cache[ilog2(threads)].store(nb = resident_blocks(P::kernel(), threads, P::smem(threads)), std::memory_order_relaxed);
     const long long grid = std::min((long long)b.n << b.lgi, (long long)nb * num_sms());
     return launch_pdl(P::kernel(), (unsigned)grid, threads, P::smem(threads), st, b);
 }
@@ -954,10 +945,7 @@ cudaError_t pm_launch_recentre(const PartK<T> &p, const SysK &sk, CenK *cen, lon
         // one full wave of resident blocks (5 per SM in FP32, 48 registers
         // for four particles' loads in flight): each thread sums several
         // particles in registers before the one warp reduction
-        static int bps = 0;
-        if (!bps && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, pmk::k_recentre<T>, 256, 0) != cudaSuccess ||
-                     bps < 1))
-            bps = 1;
+        static const int bps = pmk_host::resident_blocks(pmk::k_recentre<T>, 256, 0);
         const int g = std::min(pmk_host::particle_grid(p.n), bps * pmk_host::num_sms());
         pmk::k_recentre<T><<<g, 256, 0, st>>>(p, sk, cen, part);
     }

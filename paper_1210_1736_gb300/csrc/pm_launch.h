@@ -6,6 +6,18 @@
 #include <cuda_runtime.h>
 #include "pm_internal.cuh"
 
+namespace pmk_host {
+// SMs of the device current at the first call.
+inline int num_sms() {
+    static const int sms = [] {
+        int dev = 0, n = 0;
+        cudaGetDevice(&dev);
+        return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0 ? n : 1;
+    }();
+    return sms;
+}
+}  // namespace pmk_host
+
 // One FFT pass over a pair of mass sets of one geometry packed as
 // rho_a + i rho_b (rho_b may be null).
 struct PairArgs {
