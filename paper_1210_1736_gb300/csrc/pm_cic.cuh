@@ -36,6 +36,7 @@
 
 #include <algorithm>
 
+#include "pm_launch.h"
 #include "pm_particle.cuh"
 
 namespace pmk {
@@ -533,7 +534,7 @@ cudaError_t pm_launch_cic_field(int mode, const PartK<T> &p, const SysK &sk, con
 }
 
 static cudaError_t cic_slots(long long *a, long long *b, long long n, cudaStream_t st) {
-    pmk::k_cic_slots<<<(unsigned)std::min<long long>((n / 2 + 255) / 256, 152 * 16), 256, 0, st>>>(a, b, n);
+    pmk::k_cic_slots<<<(unsigned)std::min<long long>((n / 2 + 255) / 256, 16LL * pmk_host::num_sms()), 256, 0, st>>>(a, b, n);
     return cudaGetLastError();
 }
 

@@ -427,11 +427,12 @@ cudaError_t pm_launch_diag_k(const pmk::DiagP<T> &d, const CenK *cen, const pmk:
                              cudaStream_t st) {
     const int nacc = 4 * q.nbins + 7 + 2 * q.nring * q.mmax;
     // a wave of blocks: the sums' epilogues cost FP64 operations per block
-    const unsigned wave = 152 * 8, by = (unsigned)std::min<long long>((d.n + 1023) / 1024, wave);
+    const unsigned sms = (unsigned)pmk_host::num_sms();
+    const unsigned by = (unsigned)std::min<long long>((d.n + 1023) / 1024, 8 * sms);
     pmk::k_diag_select<T><<<by, 256, 0, st>>>(d, cen, b.state, b.key, b.idx);
     if (q.nbins > 1)
         for (int pass = 0; pass < pmk::DG_PASSES; ++pass) {
-            const unsigned g = std::min(by, 152u * 2);
+            const unsigned g = std::min(by, 2 * sms);
             if constexpr (KEPT) pmk::k_diag_hist<<<g, 256, 0, st>>>(pass, q.nbins, b.state, pmk::DiagKept{b.key}, b.hist);
             else pmk::k_diag_hist<<<g, 256, 0, st>>>(pass, q.nbins, b.state, pmk::DiagRead<T>{d, cen}, b.hist);
         }
@@ -443,16 +444,16 @@ cudaError_t pm_launch_diag_k(const pmk::DiagP<T> &d, const CenK *cen, const pmk:
         const auto k = pmk::k_diag_sums<T, true, KEPT>;
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 << 10);
         if (e != cudaSuccess) return e;
-        k<<<152 * 2, threads, threads * one, st>>>(d, cen, q, b.state, b.key, b.idx, b.acc, b.rest);
+        k<<<2 * sms, threads, threads * one, st>>>(d, cen, q, b.state, b.key, b.idx, b.acc, b.rest);
     } else {
         // one set per block: small blocks, as few particles as there are for
         // each, since a block's threads add to its set one after another (64
         // bins, 16 x 64 modes, whole call with 20k / 100k / 1M particles: 482, 543
         // and 1484 us; 256 threads, a block per 1024 particles 603, 628 and 1557)
-        const unsigned g = (unsigned)std::min<long long>((d.n + 127) / 128, 152 * 8);
+        const unsigned g = (unsigned)std::min<long long>((d.n + 127) / 128, 8 * sms);
         pmk::k_diag_sums<T, false, KEPT><<<g, 128, one, st>>>(d, cen, q, b.state, b.key, b.idx, b.acc, b.rest);
     }
-    pmk::k_diag_heat<T, KEPT><<<std::min(by, 152u * 4), 256, 0, st>>>(d, cen, q.nbins, b.state, b.acc, b.rest, b.acc + nacc);
+    pmk::k_diag_heat<T, KEPT><<<std::min(by, 4 * sms), 256, 0, st>>>(d, cen, q.nbins, b.state, b.acc, b.rest, b.acc + nacc);
     return cudaGetLastError();
 }
 
