@@ -231,6 +231,11 @@ int pm_set_launch_config(pm_ctx *ctx, int32_t batched, int32_t schedule);
  * call is the expected result, not a failure. */
 int pm_selftest_wait_expiry(pm_ctx *ctx);
 
+/* Test hook: the FP64 roots that the H-hat build (inv_sqrt = 1/sqrt(r)) and
+ * the disc diagnostics (root = sqrt(r), inv = 1/root, 0 for 0) form, of n device
+ * arguments r >= 0 into device arrays.  Enqueued on `stream`. */
+int pm_selftest_roots(const double *r, int64_t n, double *inv_sqrt, double *root, double *inv, void *stream);
+
 /* Test hook: scratch that calls keep only while memory allows (the particles'
  * part of pm_disc_diagnostics, the order of the CIC calls) is refused from now
  * on beyond `bytes` (negative: no limit, the default); results do not depend on

@@ -1581,6 +1581,12 @@ int pm_selftest_scratch_limit(pm_ctx *c, int64_t bytes) {
     return PM_OK;
 }
 
+int pm_selftest_roots(const double *r, int64_t n, double *inv_sqrt, double *root, double *inv, void *stream) {
+    if (n < 0 || (n > 0 && (!r || !inv_sqrt || !root || !inv))) return fail(PM_E_ARG, "n < 0 or an array is NULL");
+    PM_CK(pm_launch_roots(r, n, inv_sqrt, root, inv, (cudaStream_t)stream));
+    return PM_OK;
+}
+
 int pm_info(pm_ctx *c, int64_t *out) {
     if (!c || !out) return fail(PM_E_ARG, "ctx or out is NULL");
     int nsets = 0;

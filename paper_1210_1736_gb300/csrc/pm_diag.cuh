@@ -19,6 +19,7 @@
 
 #include "pm_launch.h"
 #include "pm_particle.cuh"
+#include "pm_roots.cuh"
 
 namespace pmk {
 
@@ -210,28 +211,12 @@ __global__ void __launch_bounds__(256) k_diag_hist(int pass, int nbins, DiagStat
     }
 }
 
-// R = sqrt(r2) and 1/R (0 for 0): an FP32 seed, one third-order step for 1/R
-// and one residual correction for R, a third of the operations of the root and
-// the quotient.
-__device__ __forceinline__ void diag_root(double r2, double &R, double &inv) {
-    if (!(r2 > 1e-30 && r2 < 1e30)) {
-        R = __dsqrt_rn(r2);
-        inv = R > 0 ? 1.0 / R : 0.0;
-        return;
-    }
-    const double y = (double)rsqrtf((float)r2);
-    const double e = fma(-(r2 * y), y, 1.0);
-    inv = fma(y * e, fma(0.375, e, 0.5), y);
-    R = r2 * inv;
-    R = fma(0.5 * inv, fma(-R, R, r2), R);
-}
-
 // R, the direction and the cylindrical velocities of a particle.
 struct DiagPoint {
     double R, c1, s1, vR, vphi;
     __device__ __forceinline__ DiagPoint(unsigned long long key, double dx, double dy, double vx, double vy) {
         double inv;
-        diag_root(__longlong_as_double((long long)key), R, inv);
+        pmroot::root_inv(__longlong_as_double((long long)key), R, inv);
         c1 = dx * inv;
         s1 = dy * inv;
         vR = c1 * vx + s1 * vy;

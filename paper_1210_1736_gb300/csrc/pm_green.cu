@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include "pm_passes_fx.cuh"
+#include "pm_roots.cuh"
 
 namespace {
 
@@ -27,22 +28,6 @@ struct HatArgs {
     int ny1;                 // ny + 1 (first axis)
     double q, h000, scale;
 };
-
-// The FP64 value of a normal FP32 one by integer operations (the conversion
-// takes a slot of the FP64 pipe).
-__device__ __forceinline__ double widen(float f) {
-    const unsigned b = __float_as_uint(f);   // f > 0
-    return __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
-}
-// 1/sqrt(r2), r2 known to FP32 as rf: an FP32 seed and one third-order step
-// (relative error about 2^-52, as the quotient by a rounded root; a third of
-// the FP64 operations).
-__device__ __forceinline__ double inv_sqrt(double r2, float rf) {
-    if (!(rf > 1e-30f && rf < 1e30f)) return 1.0 / sqrt(r2);
-    const double y = widen(rsqrtf(rf));
-    const double e = fma(-(r2 * y), y, 1.0);
-    return fma(y * e, fma(0.375, e, 0.5), y);
-}
 
 // AX 0: evaluate H, transform along x; 1: along y; 2: along z, then scale into
 // T and store in the table's order (see pm_build_hhat).
@@ -84,7 +69,7 @@ template <int L, int AX, typename T> __global__ void __launch_bounds__(pmk::FXT,
         if constexpr (AX == 0) {
             auto green = [&](int w) {
                 const int n = i * i + jj[w];   // exact in FP32
-                return i == 0 && col + w == 0 ? a.h000 : inv_sqrt((double)n + kk[w], (float)n + kf[w]);
+                return i == 0 && col + w == 0 ? a.h000 : pmroot::inv_sqrt((double)n + kk[w], (float)n + kf[w]);
             };
             if (va) d.x = green(0);
             if (vb) d.y = green(1);

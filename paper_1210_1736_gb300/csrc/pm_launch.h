@@ -238,6 +238,9 @@ template <typename T>
 cudaError_t pm_build_hhat(double *h, T *out, const fxw *tw, int nx, int ny, int nz, double q, double h000, double scale,
                           cudaStream_t st);
 
+// The FP64 roots of pm_roots.cuh of n arguments.
+cudaError_t pm_launch_roots(const double *r, long long n, double *inv_sqrt, double *root, double *inv, cudaStream_t st);
+
 // Self-test of the bounded waits: one block waits on an mbarrier nothing
 // arrives at, gives up after the time limit and sets *err to 1.
 cudaError_t pm_launch_wait_expiry(int *err, cudaStream_t st);

@@ -89,6 +89,7 @@ _SIGS.update({
     "pm_cic_kick_drift": (C.c_int, [_vp, _P(pm_particles), C.c_double, C.c_double]),
     "pm_cic_vjp": (C.c_int, [_vp, _P(pm_particles), _vp, _vp, _vp, _vp, _vp, _vp, _vp]),
     "pm_selftest_wait_expiry": (C.c_int, [_vp]),
+    "pm_selftest_roots": (C.c_int, [_vp, C.c_int64, _vp, _vp, _vp, _vp]),
     "pm_selftest_scratch_limit": (C.c_int, [_vp, C.c_int64]),
     "pm_recentre_sums": (C.c_int, [_vp, _P(pm_particles)]),
     "pm_recentre_apply": (C.c_int, [_vp]),
