@@ -1,6 +1,6 @@
-"""The CIC kernels' processing order: from 2^16 particles they run in spatial
-order, share atomics within runs of one cell and take each point once per
-level.  Densities, gradients and trajectories must not depend on it."""
+"""The CIC kernels' processing order: in nested systems from 2^16 particles they
+run in spatial order, share atomics within runs of one cell and take each point
+once per level.  Densities, gradients and trajectories must not depend on it."""
 import numpy as np
 import pytest
 
@@ -19,15 +19,16 @@ def _case(precision, n, crowd):
     return w
 
 
-def _all(w, perm, order):
-    """Densities, accelerations and vector-Jacobian product with the particles
-    stored in the order perm, given back in w's; order: whether the library
-    may order them (with one particle fewer than it asks for, it may not)."""
+def _cotangent(w):
+    return cast(w, np.random.default_rng(5).normal(size=w["pos"].shape))
+
+
+def _all(w, perm, u):
+    """Densities, accelerations and vector-Jacobian product for the cotangent
+    u with the particles stored in the order perm, given back in w's."""
     import torch
     m = cast(w, w["m"])
     ctx = pm.Context(w, W.mass_bound(m))
-    rng = np.random.default_rng(5)
-    u = cast(w, rng.normal(size=w["pos"].shape))
     p = pm.Particles(cast(w, w["pos"])[:, perm], cast(w, w["vel"])[:, perm], m[perm], w["gal"][perm],
                      precision=w["precision"])
     ctx.cic_deposit(p)
@@ -46,8 +47,9 @@ def _all(w, perm, order):
 @pytest.mark.parametrize("n,crowd", [(1 << 16, False), ((1 << 16) + 1, True), (70_003, False)])
 def test_order_changes_nothing(precision, n, crowd):
     w = _case(precision, n, crowd)
-    a_rho, a = _all(w, np.arange(n), True)
-    b_rho, b = _all(w, np.random.default_rng(3).permutation(n), True)
+    u = _cotangent(w)
+    a_rho, a = _all(w, np.arange(n), u)
+    b_rho, b = _all(w, np.random.default_rng(3).permutation(n), u)
     for k in a_rho:
         assert np.array_equal(a_rho[k], b_rho[k]), k
     for s, t in zip(a, b):
@@ -57,7 +59,8 @@ def test_order_changes_nothing(precision, n, crowd):
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
 def test_ordered_equals_unordered(precision):
     """The same system just below the limit, and above it with massless
-    particles added: the sums are the same integers."""
+    particles without cotangent added: the sums are the same integers, also of
+    the adjoint densities where both numbers give one fixed-point scale."""
     n = (1 << 16) - 1
     w = _case(precision, n, True)
     big = dict(w)
@@ -65,11 +68,18 @@ def test_ordered_equals_unordered(precision):
         big[k] = np.concatenate([w[k], w[k][:, :500]], axis=1)
     big["m"] = np.concatenate([w["m"], np.zeros(500)])
     big["gal"] = np.concatenate([w["gal"], w["gal"][:500]])
-    a_rho, a = _all(w, np.arange(n), False)
-    b_rho, b = _all(big, np.arange(n + 500), True)
+    u = _cotangent(w)
+    ub = np.concatenate([u, np.zeros_like(u[:, :500])], axis=1)
+    # the scale is 2^(61 - ceil(log2(1.01 n max|u| max(1/l_xy + 1/(2 l_z)))))
+    ls = [g for q in w["galaxies"] for g in map(pm.geometry, (q["coarse"], q["medium"], q["fine"]))]
+    bound = 1.01 * float(np.abs(u).astype(np.float32).max()) * max(1 / g.l_xy + 1 / (2 * g.l_z) for g in ls)
+    assert np.ceil(np.log2(n * bound)) == np.ceil(np.log2((n + 500) * bound))
+    a_rho, a = _all(w, np.arange(n), u)
+    b_rho, b = _all(big, np.arange(n + 500), ub)
     for k in a_rho:
         assert np.array_equal(a_rho[k], b_rho[k]), k
-    assert np.array_equal(a[0], b[0][:, :n])
+    for s, t in zip(a, b):   # accelerations, position and mass gradients
+        assert s.any() and np.array_equal(s, t[..., :n])
 
 
 def test_other_particles_of_the_same_number():
