@@ -248,8 +248,8 @@ int pm_selftest_scratch_limit(pm_ctx *ctx, int64_t bytes);
  * outer) and cell of that region's grid (cells binned so a grid has at most
  * 2^21 bins); lost particles go last.  Order within a cell is unspecified.
  * If perm is not NULL (device int64[n]) it receives perm[new] = old.
- * Results of the step do not depend on the order.  Allocates its scratch
- * (about 48 bytes per particle) on first use. */
+ * Results of the step do not depend on the order.  Allocates its scratch (44
+ * bytes per particle in FP32, 72 in FP64) on first use and when n grows. */
 int pm_sort(pm_ctx *ctx, const pm_particles *p, int64_t *perm);
 /* pm_step re-sorts the particles before every k-th step (k = 0: never, the
  * default); resets the step counter so the next step sorts. */

@@ -8,10 +8,13 @@
 // with a 60-bit twiddle takes 12 32x32+64-bit multiply-adds.  Before every
 // radix-16 stage the values are shifted so that the largest sum of magnitudes
 // that one butterfly combines fills FX_TOP bits, the most for which the stage
-// cannot overflow, so the rounding of a stage is below 2^-55 of the largest
-// component of the warp or tile, less than the 2^-53 per operation of FP64
-// arithmetic.  Work arrays, H-hat and
-// potentials stay FP64 in memory.
+// cannot overflow: the largest of its 32 components is then at least about 2^54
+// units.  A value enters the butterfly with an error of up to two units (half a
+// unit from the shift, up to 1.5 from a twiddle product, which drops the low
+// parts' products).  These errors are relative to the largest component of the
+// warp or tile, FP64's to each value; measured against 80-bit arithmetic the
+// potentials' error is 0.6-1.0 of that of FP64 transforms (grids of 16^3 to 64^3
+// and 256 x 16 x 64).  Work arrays, H-hat and potentials stay FP64 in memory.
 #pragma once
 
 #include "pm_internal.cuh"

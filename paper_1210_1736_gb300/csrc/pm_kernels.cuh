@@ -91,9 +91,12 @@ struct DepCache {
 // collectives.  DEP_CACHED, unsorted particles of a system with nested grids,
 // whose coarse cells are as large as a core: the coarse and medium grids' hot
 // cells are cached (with the cold densities of a first launch 48k particles
-// 16 -> 10 us, 200k 49 -> 28, 1M 134 -> 65).  DEP_PLAIN: a single grid resolves
-// its core and has no hot cells (65k particles on 32^3: the cache cost 1.5 us
-// a step).
+// 16 -> 10 us, 200k 49 -> 28, 1M 134 -> 65).  DEP_PLAIN, single grids: a body
+// that fills its grid has few hot cells, and the cache costs as much as it saves
+// or more (Plummer sphere on 32^3, 65k particles FP32 12.9 -> 12.9 us, FP64 12 ->
+// 15; 64^3, 1M 21 -> 24, FP64 8M 210 -> 228).  The rule does not see a body much
+// smaller than its single grid, which would gain (a tenth of the size on 32^3:
+// 65k 40 -> 11 us, 1M 455 -> 22).
 enum { DEP_SORTED = 0, DEP_CACHED = 1, DEP_PLAIN = 2 };
 template <typename T, int HOW>
 __global__ void __launch_bounds__(256, 6) k_deposit(PartK<T> p, const __grid_constant__ SysK s, const CenK *cen) {
