@@ -808,7 +808,8 @@ template <typename T> int step_timed_impl(pm_ctx *c, const pm_particles *p, doub
 //   nested 32^3, FP64          32k 4304 -> 4367, 66k 5938 -> 5562
 // Most of the gain is the product's (its spread): a deposit without one gains
 // from about 1.2e5 particles in FP32 (66k 43 -> 56 us, 200k 101 -> 88).
-constexpr long long CIC_ORDER_MIN = 1LL << 16, CIC_ORDER_MAX = 1LL << 32, CIC_ORDER_CELLS = 16;
+constexpr long long CIC_ORDER_MIN = 1LL << 16, CIC_ORDER_MAX = 1LL << 32, CIC_ORDER_CELLS = 16,
+                    CIC_KICK_ORDER_MIN = 1LL << 18;
 bool cic_order_pays(const pm_ctx *c, long long n) {
     bool nested = false;
     for (int g = 0; g < c->sys.ngal; ++g) nested = nested || geom_present(c->gal[g].medium);
@@ -846,10 +847,14 @@ template <typename T> int cic_deposit_impl(pm_ctx *c, const pm_particles *p) {
 
 template <typename T> int cic_field_impl(pm_ctx *c, int mode, const pm_particles *p, double dtk, double dtd,
                                          void *ox, void *oy, void *oz) {
-    // a kick-drift writes six arrays, scattered in an order: FP32 keeps the
-    // stored one (1M: 99 us, ordered 122), FP64, bound by arithmetic that
-    // neighbours share, does not (200k: 152, ordered 93)
-    const unsigned *ord = mode == 0 && sizeof(T) == 4 ? nullptr : cic_ord(c, p);
+    // A kick-drift writes six arrays, scattered in an order.  FP32, one galaxy:
+    // the stored order at every size (1M: 99 us, ordered 122).  Several galaxies'
+    // gathers per particle outweigh that from 2^18 particles (64^3 grids and a
+    // satellite, 4-step gradients, stored / ordered: 160k 5168 / 5412 us, 300k
+    // 6742 / 6699, 2M 28253 / 27892).  FP64, bound by arithmetic that neighbours
+    // share: ordered (200k: 93 us, stored 152).
+    const bool stored = mode == 0 && sizeof(T) == 4 && (c->sys.ngal == 1 || p->n < CIC_KICK_ORDER_MIN);
+    const unsigned *ord = stored ? nullptr : cic_ord(c, p);
     PM_CK(pm_launch_cic_field<T>(mode, part_k<T>(p), c->hs, c->d_cen, dtk, dtd, (T *)ox, (T *)oy, (T *)oz, nullptr,
                                  nullptr, nullptr, 0.0, ord, c->user));
     return PM_OK;

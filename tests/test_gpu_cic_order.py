@@ -82,6 +82,28 @@ def test_ordered_equals_unordered(precision):
         assert s.any() and np.array_equal(s, t[..., :n])
 
 
+@pytest.mark.parametrize("precision,n", [("fp32", 1 << 16), ("fp32", (1 << 18) - 1), ("fp32", 1 << 18), ("fp64", 1 << 16)])
+def test_kick_drift_in_either_order(precision, n):
+    """Positions and velocities after a kick-drift, which runs in the stored
+    order or in the computed one, do not depend on how particles are stored."""
+    w = _case(precision, n, False)
+    m, out = cast(w, w["m"]), []
+    for perm in (np.arange(n), np.random.default_rng(3).permutation(n)):
+        ctx = pm.Context(w, W.mass_bound(m))
+        p = pm.Particles(cast(w, w["pos"])[:, perm], cast(w, w["vel"])[:, perm], m[perm], w["gal"][perm],
+                         precision=precision)
+        ctx.cic_deposit(p)
+        ctx.solve()
+        ctx.cic_kick_drift(p, 0.01, 0.02)
+        pos, vel, _ = p.host()
+        back = np.argsort(perm)
+        out.append((pos[:, back], vel[:, back]))
+        ctx.close()
+    assert not np.array_equal(out[0][0], cast(w, w["pos"]))
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
 def test_other_particles_of_the_same_number():
     """A call after another set's deposit runs in that set's order: results
     are those of its own particles."""
