@@ -155,7 +155,7 @@ template <int N> __device__ __forceinline__ void shift_full(fx2 *v, int s) {
 // pipe too).  hi word without sign: orders like |d|.
 __device__ __forceinline__ unsigned dmag(double d) { return (unsigned)__double2hiint(d) & 0x7fffffffu; }
 // d as q 2^(em - 1022 - K) with |q| < 2^K, K in 53..63 (truncated; negative
-// values one unit low).  em: group_em.
+// values one unit low, a zero's too).  em: group_em.
 template <int K> __device__ __forceinline__ long long from_double(double d, int em) {
     const int hi = __double2hiint(d);
     const int e = (hi >> 20) & 0x7ff;
@@ -165,9 +165,10 @@ template <int K> __device__ __forceinline__ long long from_double(double d, int 
 }
 // x 2^ex for |x| < 2^61, rounded to nearest (a negative x one unit high).
 // CHECK: ex may put the result out of range (then 0, infinity or, for
-// FX_NAN, NaN); without, -1000 < ex < 900.
+// FX_NAN, NaN); without, -1000 < ex < 900.  Never -0.0, of which from_double
+// would make a unit.
 template <bool CHECK> __device__ __forceinline__ double to_double(long long x, int ex) {
-    const int s = (int)(x >> 63);
+    int s = (int)(x >> 63);
     unsigned h = (unsigned)(x >> 32) ^ (unsigned)s, l = (unsigned)x ^ (unsigned)s;
     int E = 1023 + 62 - 1 + ex;   // biased exponent - 1 of a leading bit 62 (which adds it)
     if (h == 0) { h = l; l = 0; E -= 32; }
@@ -179,7 +180,7 @@ template <bool CHECK> __device__ __forceinline__ double to_double(long long x, i
     if (h == 0) m = 0;
     if (CHECK) {
         if (ex > (1 << 15)) m = 0x7ff8000000000000ull;
-        else if (E < 0) m = 0;
+        else if (E < 0) { m = 0; s = 0; }
         else if (E >= 2046) m = 0x7ff0000000000000ull;
     }
     return __hiloint2double((int)((unsigned)(m >> 32) | ((unsigned)s & 0x80000000u)), (int)(unsigned)m);
@@ -202,6 +203,9 @@ __device__ __forceinline__ int group_em(unsigned m) {
 }
 __device__ __forceinline__ bool group_zero(int em) { return em > 0x7ff; }
 __device__ __forceinline__ int group_ex(int em, int K) { return em == 0x7ff ? FX_NAN : group_zero(em) ? FX_ZERO : em - 1022 - K; }
+// What a factor converted with FX_Q bits adds to a product's exponent; a factor
+// of zero takes every value below the FP64 range (and leaves FX_NAN beyond it).
+__device__ __forceinline__ int factor_ex(int em) { return group_zero(em) ? -(1 << 14) : group_ex(em, FX_Q) + FX_Q; }
 
 }  // namespace pmfx
 

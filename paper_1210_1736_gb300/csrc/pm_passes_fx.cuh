@@ -403,9 +403,9 @@ template <int L, int MODE, bool HALF> __global__ void __launch_bounds__(FXT, 3) 
             if (e < NIN) v[e] = INV ? swapped(*at(e)) : *at(e);
         }
         // (a warp of zeros, e.g. beyond the grid's columns, has no say in it)
-        FxScale<true> sc{pmfx::group_ex(em, pmfx::FX_TOP), sl, 0};
+        FxScale<true> sc{pmfx::group_zero(em) ? pmfx::FX_LOW : pmfx::group_ex(em, pmfx::FX_TOP), sl, 0};
         sc.m = pmfx::warp_max(pmfx::group_sum<16>(v));
-        if ((tid & 31) == 0 && !pmfx::group_zero(em)) atomicMax(sl, sc.ex + pmfx::sum_shift(sc.m, fx_top<L>(0)));
+        if ((tid & 31) == 0) atomicMax(sl, sc.ex + pmfx::sum_shift(sc.m, fx_top<L>(0)));
         fence_async_smem();                // the buffer's conversions before the next load's writes
         if (tid == 0) bulk_wait_read();    // the previous tile's outputs have been read out of sm
         __syncthreads();
@@ -414,8 +414,8 @@ template <int L, int MODE, bool HALF> __global__ void __launch_bounds__(FXT, 3) 
             issue(tile + gridDim.x);
         }
         if (tid < 4) slot[(it & 1) ^ 1][tid] = tid ? 0 : pmfx::FX_LOW;   // last read before the barrier
-        const int tex = sl[0] == pmfx::FX_LOW ? pmfx::FX_ZERO : sl[0];
-        if (!pmfx::group_zero(em)) pmfx::shift<E>(v, tex - sc.ex);
+        const int tex = sl[0] == pmfx::FX_LOW ? pmfx::FX_ZERO : sl[0];   // a tile of zeros
+        pmfx::shift<E>(v, tex - sc.ex);
         sc.ex = tex;
         fx_fft<L, true>(v, sm, lay, t, tw, sc);
         // fx_fft leaves the exchange buffer free: the outputs, rows t + e TPC
@@ -609,7 +609,7 @@ __global__ void __launch_bounds__(FXT, DM == 2 ? 2 : 3) k_zfx(const __grid_const
                     *kept(e) = w;
                     m = max(m, (unsigned)max(abs((int)(w.x >> 32)), abs((int)(w.y >> 32))));
                 }
-                kex = sc.ex + pmfx::group_ex(hem, pmfx::FX_Q) + pmfx::FX_Q;
+                kex = sc.ex + pmfx::factor_ex(hem);
                 if constexpr (DM != 0) {   // components below 2^59: the difference factors' moduli reach sqrt(2)
                     const int sh = 64 - __clz((int)pmfx::warp_max(m + 1)) - (pmfx::FX_TOP - 1);
 #pragma unroll 2
@@ -633,7 +633,7 @@ __global__ void __launch_bounds__(FXT, DM == 2 ? 2 : 3) k_zfx(const __grid_const
                     pmfx::wsplit(pmfx::from_double<pmfx::FX_Q>(fi, em), f.ih, f.il);
 #pragma unroll 2
                     for (int e = 0; e < E; ++e) *mine(e) = cmul(*kept(e), f);
-                    sc.ex += pmfx::group_ex(em, pmfx::FX_Q) + pmfx::FX_Q;
+                    sc.ex += pmfx::factor_ex(em);
                 } else {
                     // D_z + i in units of 2^-59, the second half of D's table
                     const longlong2 *dz = static_cast<const longlong2 *>(a.dtz) + L;

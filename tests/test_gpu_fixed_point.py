@@ -136,3 +136,18 @@ def test_small_magnitudes(shape, G, shift):
     tol = unit + 64 * 2.0 ** -53 * np.ldexp(np.abs(a).max(), k)
     print(f"tolerance {tol / np.ldexp(np.abs(a).max(), k):.1e} of the largest value")
     assert np.abs(b - np.ldexp(a, k)).max() <= tol
+
+
+@pytest.mark.parametrize("shape", [(16, 16, 16), (64, 32, 32), (8, 64, 16)])
+@pytest.mark.parametrize("G", [0.0, -0.0, 2.0 ** -1060, -2.0 ** -1060])
+def test_vanishing_strength(shape, G):
+    """No Green's function, and one whose potential is below every FP64 number:
+    groups of zeros of either sign stay zero."""
+    nx, ny, nz = shape
+    rho = np.random.default_rng(6).integers(-2 ** 45, 2 ** 45, size=(nz, ny, nx))
+    b = _static(rho, shape, G=G)
+    if G == 0:
+        assert not b.any()
+    # the unit of the conversions (see test_small_magnitudes)
+    N8, M = 8.0 * rho.size, float(np.abs(rho).sum()) * 2.0 ** -50
+    assert np.abs(b).max() <= N8 * (M + 2) * 2.0 ** -1018
