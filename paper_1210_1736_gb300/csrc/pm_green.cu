@@ -13,6 +13,8 @@
 // is also more exact: the FP64 potentials' error fell to a half or a third.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "pm_passes_fx.cuh"
 #include "pm_roots.cuh"
 
@@ -134,14 +136,12 @@ template <int L, int AX, typename T> __global__ void __launch_bounds__(pmk::FXT,
 }
 
 template <int L, int AX, typename T> cudaError_t launch_axis(const HatArgs &a, cudaStream_t st) {
-    constexpr int TPC = L / E, LDR = L + L / 16, per = pmk::FXT / TPC;
-    constexpr size_t smem = ((size_t)pmfft::tw_dir_size(L, false) + (size_t)per * LDR) * sizeof(fx2);
-    static_assert(smem <= 48 << 10, "no opt-in");
-    // (blocks of one warp, which spread few columns over more SMs, measured the
-    // same or slower: 32^3 13.8, 11.3, 13.5 us against 13.7, 10.0, 12.8, 16^3
-    // 12.4, 9.2, 12.0 against 13.2, 9.1, 12.0)
-    const long long lines = (a.ncol + 1) / 2;
-    k_hat_axis<L, AX, T><<<(unsigned)((lines + per - 1) / per), pmk::FXT, smem, st>>>(a);
+    constexpr int TPC = L / E, LDR = L + L / 16;
+    const int threads = std::max(32, a.ncol / 2 * TPC < 32LL * 608 ? 32 : pmk::FXT);   // few columns: a warp per block
+    const size_t smem = ((size_t)pmfft::tw_dir_size(L, false) + (size_t)threads / TPC * LDR) * sizeof(fx2);
+    static_assert(((size_t)pmfft::tw_dir_size(L, false) + (size_t)pmk::FXT / TPC * LDR) * sizeof(fx2) <= 48 << 10, "no opt-in");
+    const long long lines = (a.ncol + 1) / 2, per = threads / TPC;
+    k_hat_axis<L, AX, T><<<(unsigned)((lines + per - 1) / per), threads, smem, st>>>(a);
     return cudaGetLastError();
 }
 template <int AX, typename T> cudaError_t axis(int n, const HatArgs &a, cudaStream_t st) {
