@@ -13,8 +13,6 @@
 // is also more exact: the FP64 potentials' error fell to a half or a third.
 #include <cuda_runtime.h>
 
-#include <algorithm>
-
 #include "pm_passes_fx.cuh"
 #include "pm_roots.cuh"
 
@@ -137,7 +135,12 @@ template <int L, int AX, typename T> __global__ void __launch_bounds__(pmk::FXT,
 
 template <int L, int AX, typename T> cudaError_t launch_axis(const HatArgs &a, cudaStream_t st) {
     constexpr int TPC = L / E, LDR = L + L / 16;
-    const int threads = std::max(32, a.ncol / 2 * TPC < 32LL * 608 ? 32 : pmk::FXT);   // few columns: a warp per block
+    // Fewer warps than the SMs have schedulers: blocks of one warp, which spread
+    // over more SMs (whole calls of pm_potential_static, one after another, 32 /
+    // 128 threads: FP32 8 x 8 x 128 55.6 / 59.5 us, 8 x 256 x 8 61.9 / 66.1, 64 x
+    // 64 x 32 68.9 / 71.1, 16 x 16 x 256 70.7 / 68.1).  From there on both
+    // measure the same (128 x 64 x 32 77.9 us).
+    const int threads = a.ncol / 2 * TPC < 32LL * 4 * pmk_host::num_sms() ? 32 : pmk::FXT;
     const size_t smem = ((size_t)pmfft::tw_dir_size(L, false) + (size_t)threads / TPC * LDR) * sizeof(fx2);
     static_assert(((size_t)pmfft::tw_dir_size(L, false) + (size_t)pmk::FXT / TPC * LDR) * sizeof(fx2) <= 48 << 10, "no opt-in");
     const long long lines = (a.ncol + 1) / 2, per = threads / TPC;
