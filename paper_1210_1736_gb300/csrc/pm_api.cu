@@ -804,16 +804,18 @@ template <typename T> int step_timed_impl(pm_ctx *c, const pm_particles *p, doub
 //   one 64^3 grid, FP32        66k 2212 -> 2558, 1M 5376 -> 7124 (FP64 500k 7930 -> 8910)
 //   nested 32^3, 64^3, FP32    66k 3432 -> 3485, 3389 -> 3426; 100k 4311 -> 3992, 4086 -> 3789
 //   nested 64^3 and satellite  66k 4475 -> 4129, 100k 5384 -> 4542 (FP64 32k 8981 -> 8654)
-//   nested 128^3 (4.7M cells)  200k 8994 -> 9037, 300k 9845 -> 9380
+//   nested 128^3, FP32         190k 8097 -> 8176, 260k 8675 -> 8580 (4.3M cells)
 //   nested 32^3, FP64          32k 4304 -> 4367, 66k 5938 -> 5562
+//   nested 128^3, FP64         66k 33166 -> 33212, 100k 34477 -> 33761 (4.3M cells)
 // Most of the gain is the product's (its spread): a deposit without one gains
 // from about 1.2e5 particles in FP32 (66k 43 -> 56 us, 200k 101 -> 88).
-constexpr long long CIC_ORDER_MIN = 1LL << 16, CIC_ORDER_MAX = 1LL << 32, CIC_ORDER_CELLS = 16,
+constexpr long long CIC_ORDER_MIN = 1LL << 16, CIC_ORDER_MAX = 1LL << 32,
                     CIC_KICK_ORDER_MIN = 1LL << 18;
 bool cic_order_pays(const pm_ctx *c, long long n) {
     bool nested = false;
     for (int g = 0; g < c->sys.ngal; ++g) nested = nested || geom_present(c->gal[g].medium);
-    return nested && n >= CIC_ORDER_MIN && n >= c->sortk.nkeys / CIC_ORDER_CELLS && n < CIC_ORDER_MAX;
+    const long long cells = c->prec == PM_FP32 ? c->sortk.nkeys / 20 : c->sortk.nkeys / 64;
+    return nested && n >= CIC_ORDER_MIN && n >= cells && n < CIC_ORDER_MAX;
 }
 bool capturing(const pm_ctx *c) {
     cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
