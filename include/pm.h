@@ -281,8 +281,9 @@ int pm_step_timed(pm_ctx *ctx, const pm_particles *p, double dt, int32_t nsteps,
  *
  * pm_cic_deposit: lost test as pm_deposit, then int64 fixed-point CIC mass
  * (each of the 8 cell shares rounded separately) into the five sets.  Use
- * pm_solve afterwards.  In nested systems, from 65536 particles and a
- * twentieth (FP64: a 64th) of the cells, it also finds the particles' spatial order, in which
+ * pm_solve afterwards.  In nested systems, from 65536 particles (FP32 and one
+ * galaxy: and a tenth of its coarse cells), it also finds the particles'
+ * spatial order, in which
  * this and the following CIC calls work (no result depends on it): 12 bytes
  * per particle, allocated on the first call with more particles than before
  * (the outgrown buffer is released).  Captured calls, and calls without memory

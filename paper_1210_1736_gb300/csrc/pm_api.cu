@@ -800,22 +800,28 @@ template <typename T> int step_timed_impl(pm_ctx *c, const pm_particles *p, doub
 //
 // The order costs 26 us, more with the number of cells (its keys).  It pays
 // where cells are crowded: nested grids, whose coarse cells are as large as a
-// core.  Forward and backward of 4 steps, us, stored order -> ordered:
-//   one 64^3 grid, FP32        66k 2212 -> 2558, 1M 5376 -> 7124 (FP64 500k 7930 -> 8910)
-//   nested 32^3, 64^3, FP32    66k 3432 -> 3485, 3389 -> 3426; 100k 4311 -> 3992, 4086 -> 3789
-//   nested 64^3 and satellite  66k 4475 -> 4129, 100k 5384 -> 4542 (FP64 32k 8981 -> 8654)
-//   nested 128^3, FP32         190k 8097 -> 8176, 260k 8675 -> 8580 (4.3M cells)
-//   nested 32^3, FP64          32k 4304 -> 4367, 66k 5938 -> 5562
-//   nested 128^3, FP64         66k 33166 -> 33212, 100k 34477 -> 33761 (4.3M cells)
-// Most of the gain is the product's (its spread): a deposit without one gains
-// from about 1.2e5 particles in FP32 (66k 43 -> 56 us, 200k 101 -> 88).
-constexpr long long CIC_ORDER_MIN = 1LL << 16, CIC_ORDER_MAX = 1LL << 32,
-                    CIC_KICK_ORDER_MIN = 1LL << 18;
+// core, the more the fewer coarse cells there are, the more galaxies each
+// particle spreads to, and in FP64, whose kernels are dearer.  Forward and
+// backward of 3 steps (one grid: 4), us, stored order -> ordered; coarse and
+// medium grid:
+//   FP32  one 64^3 grid    66k 2212 -> 2558, 1M 5376 -> 7124 (FP64 500k 7930 -> 8910)
+//         32^3, 32^3       66k 3359 -> 3306, 90k 3680 -> 3467, 190k 5251 -> 4677
+//         64^3, 128^3      66k 4339 -> 4481, 90k 4754 -> 4828, 130k 5467 -> 5242
+//         128^3, 32^3      130k 5003 -> 5043, 190k 5667 -> 5549
+//         128^3, 128^3     130k 6984 -> 7131, 190k 7455 -> 7404, 280k 8109 -> 7729
+//         with a satellite: 32^3, 32^3 66k 3806 -> 3523; 128^3, 128^3 66k 7225 -> 7299,
+//                          90k 7668 -> 7446
+//   FP64  32^3, 32^3       66k 4808 -> 4502; 128^3, 128^3 66k 26660 -> 26796, 90k 27429 ->
+//                          27092
+// So from 2^16 particles, and a single galaxy in FP32 from a tenth of its coarse
+// cells.  Most of the gain is the product's (its spread): a deposit without one
+// gains from about 1.2e5 particles in FP32 (66k 43 -> 56 us, 200k 101 -> 88).
+constexpr long long CIC_ORDER_MIN = 1LL << 16, CIC_ORDER_MAX = 1LL << 32, CIC_KICK_ORDER_MIN = 1LL << 18;
 bool cic_order_pays(const pm_ctx *c, long long n) {
     bool nested = false;
     for (int g = 0; g < c->sys.ngal; ++g) nested = nested || geom_present(c->gal[g].medium);
-    const long long cells = c->prec == PM_FP32 ? c->sortk.nkeys / 20 : c->sortk.nkeys / 64;
-    return nested && n >= CIC_ORDER_MIN && n >= cells && n < CIC_ORDER_MAX;
+    if (!nested || n < CIC_ORDER_MIN || n >= CIC_ORDER_MAX) return false;
+    return c->prec == PM_FP64 || c->sys.ngal > 1 || n >= c->geos[c->set_geo[0][4]].A / 10;
 }
 bool capturing(const pm_ctx *c) {
     cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;

@@ -164,8 +164,8 @@ def test_captured_calls_keep_the_stored_order():
 
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
 def test_where_the_order_is_computed(precision):
-    """In nested systems from 2^16 particles and a twentieth (FP64: a 64th) of
-    the cells (32 and 128 cells a side here); not on a single grid."""
+    """In nested systems from 2^16 particles, and a tenth of the coarse cells
+    for a single galaxy in FP32; not on a single grid."""
     import torch
 
     def grown(w, n):
@@ -184,7 +184,8 @@ def test_where_the_order_is_computed(precision):
     n = 1 << 16
     w = _case(precision, n, False)
     assert grown(w, n) == 12 * n and grown(w, n - 1) == 0
-    wide = dict(w, galaxies=[dict(w["galaxies"][0]), *w["galaxies"][1:]])
-    wide["galaxies"][0]["coarse"] = (128, 128, 128) + tuple(w["galaxies"][0]["coarse"][3:])
-    assert grown(wide, n) == (12 * n if precision == "fp64" else 0)
+    g = W.galaxy_small(precision=precision, n_total=n)
+    assert grown(g, n) == 12 * n
+    g["galaxies"][0]["coarse"] = (128, 128, 128) + tuple(g["galaxies"][0]["coarse"][3:])
+    assert grown(g, n) == (12 * n if precision == "fp64" else 0)
     assert grown(W.big_box(n, 32, precision=precision), n) == 0
