@@ -923,8 +923,7 @@ template <typename T> int disc_impl(pm_ctx *c, const pm_particles *p, const uint
     // fixed part, then per particle rest (32 bytes), key and index; without
     // memory for those every pass reads the particles instead
     constexpr size_t hist = sizeof(unsigned) * 2048 * DG_MAXBINS, state = (sizeof(pmk::DiagState) + 255) & ~(size_t)255;
-    constexpr size_t fixed = hist + state + sizeof(double) * (4 * DG_MAXBINS + 8 + 2 * DG_MAXRM);
-    static_assert(fixed % sizeof(double4) == 0, "alignment of the particles' part");
+    constexpr size_t fixed = (hist + state + sizeof(double) * (4 * DG_MAXBINS + 8 + 2 * DG_MAXRM) + 255) & ~(size_t)255;
     unsigned char *m = (unsigned char *)keep_scratch(c, c->dg_mem, fixed + (size_t)p->n * 48);
     const bool kept = m != nullptr;
     if (!kept) {
