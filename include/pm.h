@@ -283,11 +283,10 @@ int pm_step_timed(pm_ctx *ctx, const pm_particles *p, double dt, int32_t nsteps,
  * (each of the 8 cell shares rounded separately) into the five sets.  Use
  * pm_solve afterwards.  In nested systems, from 65536 particles (FP32 and one
  * galaxy: and a tenth of its coarse cells), it also finds the particles'
- * spatial order, in which
- * this and the following CIC calls work (no result depends on it): 12 bytes
- * per particle, allocated on the first call with more particles than before
- * (the outgrown buffer is released).  Captured calls, and calls without memory
- * for it, work in the stored order.
+ * spatial order, in which this and the following CIC calls work (no result
+ * depends on it): 12 bytes per particle, allocated on the first call with more
+ * particles than before (the outgrown buffer is released).  Captured calls, and
+ * calls without memory for it, work in the stored order.
  * pm_cic_force: ax, ay, az (device, context precision, n) = CIC acceleration
  * from the current potentials; lost particles get 0.
  * pm_cic_kick_drift: v += dt_kick a; x += dt_drift v (live particles).

@@ -11,8 +11,10 @@
 // device; one pass forms every sum and leaves what the heat needs.  1M
 // particles, 400k selected, launches under ncu: radix passes over all particles
 // 353 us (and a host step each), sums by FP64 shared atomics 318, heat 130;
-// now select and radix passes 155, sums 113 (FP64 operations and read-modify-
-// writes of 4 warps per SM, as many as the columns leave room for), heat 18.
+// now select and radix passes 163, sums 105 (FP64 operations and read-modify-
+// writes of 4 warps per SM, as many as the columns leave room for), heat 17.
+// Without memory for the list every pass reads the particles (the whole call
+// 389 -> 690 us).
 #pragma once
 
 #include <algorithm>
